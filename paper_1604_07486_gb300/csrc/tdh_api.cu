@@ -283,15 +283,29 @@ int run(tdh_plan_t plan, const void* in, void* out, int64_t batch, void* stream,
     // A = A_m ... A_1: the first step reads `in`, later steps work in place on `out` (each
     // cluster reads its whole vector before writing it; sparse factors save their tiles'
     // halos first); A^T runs the steps in reverse.
-    for (size_t i = 0; i < nsteps; ++i) {
-        const Step& st = plan->steps[adjoint ? nsteps - 1 - i : i];
-        const void* src = i == 0 ? in : out;
-        if (st.sp_M > 0)
-            TDH_TRY(sparse_launch(st, plan->params.prec, src, out, batch, adjoint, s));
-        else
-            TDH_TRY(exec_launch(st, plan->params.prec, src, out, batch, adjoint, s));
+    // Between consecutive inverse sparse steps of a float32 chain the values are pairs of floats,
+    // in a scratch buffer of their own.
+    auto step = [&](size_t i) -> const Step& { return plan->steps[adjoint ? nsteps - 1 - i : i]; };
+    auto wide_after = [&](size_t i) {
+        return i + 1 < nsteps && step(i).sp_sums == 2 && step(i + 1).sp_sums == 2;
+    };
+    bool need_wide = false;
+    for (size_t i = 0; i < nsteps; ++i) need_wide = need_wide || wide_after(i);
+    void* wide = nullptr;
+    if (need_wide) TDH_TRY(scratch_alloc(&wide, 2 * bytes, s));
+    const void* src = in;
+    int rc = TDH_OK;
+    for (size_t i = 0; rc == TDH_OK && i < nsteps; ++i) {
+        const Step& st = step(i);
+        const bool win = i > 0 && wide_after(i - 1), wout = wide_after(i);
+        void* dst = wout ? wide : out;
+        rc = st.sp_M > 0 ? sparse_launch(st, plan->params.prec, src, dst, batch, adjoint, win,
+                                         wout, s)
+                         : exec_launch(st, plan->params.prec, src, dst, batch, adjoint, s);
+        src = dst;
     }
-    return TDH_OK;
+    if (wide) scratch_free(wide, s);
+    return rc;
 }
 
 // Host buffers: the batch goes through the device in chunks, two device slots each way, so
@@ -684,6 +698,7 @@ int tdh_plan_create(int kind, int64_t n_max, const tdh_params* params, double to
     for (auto& st : plan->steps) {
         if (rc != TDH_OK) break;
         st.status = plan->status;
+        st.sp_alone = plan->steps.size() == 1 && st.sp_M == 1;
         rc = build_step(st, tol, (params->flags & TDH_FLAG_TARGET) ? 1 : 0, kmax, params->prec, s);
         if (rc != TDH_OK) break;
     }

@@ -152,6 +152,9 @@ struct Step {
     int sp_family = 0;     // SP_ULTRA (offset 2), SP_JACOBI (offset 1), SP_IDENTITY
     int sp_off = 0;        // band offset of the factors
     int sp_inverse = 0;    // apply the factors' inverses (step to a smaller parameter)
+    int sp_alone = 0;      // the plan's only step, one factor
+    int sp_sums = 0;       // inverses: 0 affine scans, 1 weighted prefix sums, 2 the same in pairs
+                           // of floats (float32 chains)
     int sp_flip = 0;       // Jacobi: factors conjugated by diag((-1)^k) (reflected frame)
     double sp_par0 = 0;    // parameter of the first factor (l, or a of S_(a,b))
     double sp_dir = 1;     // parameter change from one factor to the next (+1 or -1)
@@ -211,8 +214,11 @@ namespace tdh {
 // the factors (or of their inverses) applied to in, or its transpose; in == out allowed.
 enum { SP_ULTRA = 0, SP_JACOBI = 1, SP_IDENTITY = 2 };
 int sparse_prepare(Step& st, int prec, cudaStream_t s);
+// wide_in / wide_out (steps with sp_sums == 2 only): in / out hold pairs of floats.
 int sparse_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
-                  cudaStream_t s);
+                  bool wide_in, bool wide_out, cudaStream_t s);
+// out[j] = Gamma(j + a) / Gamma(j + b), j < count, float64 device array.
+int gamma_ratio_launch(double a, double b, int64_t count, double* out, cudaStream_t s);
 // P_k^(-1/2,-1/2)(1) = Gamma(k+1/2)/(Gamma(1/2) Gamma(k+1)), k < n (its reciprocal if
 // `inverse`), float64 device array: T_k = P_k^(-1/2,-1/2) / P_k^(-1/2,-1/2)(1).
 int chebyshev_scale_launch(int64_t n, int inverse, double* out, cudaStream_t s);

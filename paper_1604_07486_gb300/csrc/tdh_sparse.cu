@@ -24,6 +24,7 @@
 // forms rounded once to the execute precision, so the kernels do no division.  All of this
 // is ~3 flops per 8 bytes moved: bound by HBM.
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <type_traits>
 
@@ -518,6 +519,335 @@ __global__ void __launch_bounds__(kThreads) k_scan_solve(const T* in, T* out, in
     }
 }
 
+// ------------------------------------------------- back-substitution as a weighted prefix sum
+//
+// With W the solution of the homogeneous recurrence, W_j = mu_j W_{j+off}, the inverse factor is
+//   x_j = W_j sum_{i >= j, i = j mod off} U_i c_i,   U = rho / W,
+// (and its transpose x_i = U_i sum_{j <= i} W_j g_j): a plain sum per chain between two
+// products, where the affine scan above carries a multiplier.  W and U are closed forms:
+//   ultraspherical  W_j = l + j,                                    U_j = 1 / (p_j W_j);
+//   Jacobi          W_j = (2j+s+1) Gamma(j+s+1) / Gamma(j+b+1),     U_j = 1 / (p_j W_j),  s = a+b
+// (W_0 = mu_0 W_1), scaled so that both stay near 1 in the middle of their range; signs of a
+// flipped factor and the diagonal scalings fold into them.  Taken where ln W spans at most
+// kSumRange, so that products with ordinary inputs neither overflow nor vanish in float32; the
+// affine scan stays for larger parameters.
+//
+// Precision.  A single factor sums in its own precision (log2 n roundings per sum instead of n).
+// Float32 chains of several factors or steps amplify what one inverse leaves behind (a factor
+// sums its predecessor's errors over the whole tail), so there the tables, the sums and the
+// values between consecutive inverse factors are pairs of floats (FF, about 44 bits), rounded
+// once at the end; float64 chains keep the affine scan.
+//
+// Bound by HBM: k_sum_tiles reads the vectors once (tile sums), k_sum_solve reads them again,
+// from L2 when the batch fits, and writes the result; it also forms the tile sums the next
+// factor needs.  16 x 2^20 float32, C^(1.25) -> C^(0.25): 46 us against 140 us for the three
+// kernels of the affine scan (a plain copy of the batch: 20 us); two factors in pairs of
+// floats, C^(2.25) -> C^(0.25): 216 against 277 us.
+constexpr double kSumRange = 40.0;
+constexpr int kSumChunks = 4;  // pieces per thread
+
+// A pair of floats h + l, |l| <= ulp(h) / 2 (Dekker 1971; Knuth's two-sum).
+struct __align__(8) FF {
+    float h, l;
+};
+__device__ __forceinline__ FF ff_fast(float a, float b) {
+    const float s = __fadd_rn(a, b);
+    return FF{s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ FF add(FF a, FF b) {
+    const float s = __fadd_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
+    return ff_fast(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF mul(FF a, float b) {
+    const float p = __fmul_rn(a.h, b);
+    return ff_fast(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+__device__ __forceinline__ FF mul(FF a, FF b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return ff_fast(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ float add(float a, float b) { return a + b; }
+__device__ __forceinline__ float mul(float a, float b) { return a * b; }
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+__device__ __forceinline__ double mul(double a, double b) { return a * b; }
+__device__ __forceinline__ void put(float& o, float v) { o = v; }
+__device__ __forceinline__ void put(double& o, double v) { o = v; }
+__device__ __forceinline__ void put(float& o, FF v) { o = v.h; }
+__device__ __forceinline__ void put(FF& o, FF v) { o = v; }
+__device__ __forceinline__ void from_double(float& o, double v) { o = (float)v; }
+__device__ __forceinline__ void from_double(double& o, double v) { o = v; }
+__device__ __forceinline__ void from_double(FF& o, double v) {
+    o.h = (float)v;
+    o.l = isfinite(o.h) ? (float)(v - (double)o.h) : 0.0f;
+}
+template <bool DOWN, typename A>
+__device__ __forceinline__ A shfl_by(A v, int d) {
+    if constexpr (std::is_same<A, FF>::value)
+        return FF{shfl_by<DOWN>(v.h, d), shfl_by<DOWN>(v.l, d)};
+    else
+        return DOWN ? __shfl_down_sync(0xffffffffu, v, d) : __shfl_up_sync(0xffffffffu, v, d);
+}
+template <typename A>
+__device__ __forceinline__ A shfl_at(A v, int lane) {
+    if constexpr (std::is_same<A, FF>::value)
+        return FF{shfl_at(v.h, lane), shfl_at(v.l, lane)};
+    else
+        return __shfl_sync(0xffffffffu, v, lane);
+}
+
+// A: type of the sums and tables; V coefficients per piece.
+template <typename A>
+struct SumTile {
+    static constexpr int V = std::is_same<A, double>::value ? 2 : 4;
+    static constexpr int chunk = kThreads * V;
+    static constexpr int tile = kSumChunks * chunk;
+};
+
+// V consecutive values at j (ALIGNED: n a multiple of V, 16-byte accesses), 0 past n
+template <int V, bool ALIGNED, typename X>
+__device__ __forceinline__ void load_piece(const X* p, int64_t j, int64_t n, X (&v)[V]) {
+    if constexpr (ALIGNED) {
+        constexpr int W = (int)(V * sizeof(X) / 4);
+        float* f = reinterpret_cast<float*>(v);
+        if (j < n) {
+            const float* q = reinterpret_cast<const float*>(p + j);
+#pragma unroll
+            for (int i = 0; i < W; i += 4) {
+                const float4 t = *reinterpret_cast<const float4*>(q + i);
+                f[i] = t.x, f[i + 1] = t.y, f[i + 2] = t.z, f[i + 3] = t.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < W; ++i) f[i] = 0.0f;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) v[i] = j + i < n ? p[j + i] : X{};
+    }
+}
+template <int V, bool ALIGNED, typename X>
+__device__ __forceinline__ void store_piece(X* p, int64_t j, int64_t n, const X (&v)[V]) {
+    if constexpr (ALIGNED) {
+        constexpr int W = (int)(V * sizeof(X) / 4);
+        const float* f = reinterpret_cast<const float*>(v);
+        if (j < n) {
+            float* q = reinterpret_cast<float*>(p + j);
+#pragma unroll
+            for (int i = 0; i < W; i += 4)
+                *reinterpret_cast<float4*>(q + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            if (j + i < n) p[j + i] = v[i];
+    }
+}
+
+template <typename A, int OFF>
+struct ChainSum {
+    A v[OFF];
+};
+
+// Sum over the block, the same in every thread (fixed order); red: [kThreads / 32] slots.
+template <typename A, int OFF>
+__device__ __forceinline__ ChainSum<A, OFF> block_sum(ChainSum<A, OFF> x, ChainSum<A, OFF>* red) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1)
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) x.v[c] = add(x.v[c], shfl_at(x.v[c], lane ^ k));
+    if (lane == 0) red[threadIdx.x >> 5] = x;
+    __syncthreads();
+    ChainSum<A, OFF> t = red[0];
+#pragma unroll
+    for (int w = 1; w < kThreads / 32; ++w)
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) t.v[c] = add(t.v[c], red[w].v[c]);
+    return t;
+}
+
+// sum[v ntiles + t]: per chain (j mod OFF), the sum of weight_j in_j over tile t.
+template <typename A, typename TI, int OFF, bool ALIGNED>
+__global__ void __launch_bounds__(kThreads) k_sum_tiles(const TI* __restrict__ in, int64_t n,
+                                                        int64_t ntiles,
+                                                        const A* __restrict__ weight,
+                                                        ChainSum<A, OFF>* __restrict__ sum) {
+    constexpr int V = SumTile<A>::V;
+    __shared__ ChainSum<A, OFF> red[kThreads / 32];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int64_t vec = blockIdx.x / ntiles, tile = blockIdx.x % ntiles;
+    const TI* x = in + vec * n;
+    ChainSum<A, OFF> s{};
+    TI xv[kSumChunks][V];
+    A wv[kSumChunks][V];
+#pragma unroll
+    for (int k = 0; k < kSumChunks; ++k) {
+        const int64_t j = tile * SumTile<A>::tile + k * SumTile<A>::chunk + threadIdx.x * V;
+        load_piece<V, ALIGNED>(x, j, n, xv[k]);
+        load_piece<V, ALIGNED>(weight, j, n, wv[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kSumChunks; ++k)
+#pragma unroll
+        for (int i = 0; i < V; ++i) s.v[i % OFF] = add(s.v[i % OFF], mul(wv[k][i], xv[k][i]));
+    s = block_sum<A, OFF>(s, red);
+    if (threadIdx.x == 0) sum[blockIdx.x] = s;
+}
+
+// out_j = wout_j (sum over the chain of win_i in_i, i >= j (REV) or i <= j); then, where `next` is
+// given, the tile sums of next_j out_j.  The block's carry is the sum of the tiles after (before)
+// its own, added in a fixed order.  In place allowed: a block reads its tile before writing it.
+// `first`: the input is older than the previous kernel, so it may be read before waiting for it.
+template <typename A, typename TI, typename TO, int OFF, bool REV, bool ALIGNED>
+__global__ void __launch_bounds__(kThreads) k_sum_solve(const TI* in, TO* out, int64_t n,
+                                                        int64_t ntiles, const A* __restrict__ win,
+                                                        const A* __restrict__ wout,
+                                                        const ChainSum<A, OFF>* sum,
+                                                        const A* __restrict__ next,
+                                                        ChainSum<A, OFF>* next_sum, int first) {
+    constexpr int V = SumTile<A>::V;
+    constexpr int NW = kThreads / 32;
+    __shared__ ChainSum<A, OFF> red[NW], part[kSumChunks * NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int64_t vec = blockIdx.x / ntiles, tile = blockIdx.x % ntiles;
+    const TI* x = in + vec * n;
+    if (!first) asm volatile("griddepcontrol.wait;" ::: "memory");
+    A v[kSumChunks][V];
+    {
+        TI xv[kSumChunks][V];
+        A w[kSumChunks][V];
+#pragma unroll
+        for (int k = 0; k < kSumChunks; ++k) {
+            const int64_t j = tile * SumTile<A>::tile + k * SumTile<A>::chunk + tid * V;
+            load_piece<V, ALIGNED>(x, j, n, xv[k]);
+            load_piece<V, ALIGNED>(win, j, n, w[k]);
+        }
+        // within a thread, in the direction of the sums
+#pragma unroll
+        for (int k = 0; k < kSumChunks; ++k) {
+#pragma unroll
+            for (int i = 0; i < V; ++i) v[k][i] = mul(w[k][i], xv[k][i]);
+            if constexpr (REV) {
+#pragma unroll
+                for (int i = V - 1 - OFF; i >= 0; --i) v[k][i] = add(v[k][i], v[k][i + OFF]);
+            } else {
+#pragma unroll
+                for (int i = OFF; i < V; ++i) v[k][i] = add(v[k][i], v[k][i - OFF]);
+            }
+        }
+    }
+    // exclusive scan of the threads' totals over the warp, per piece
+    ChainSum<A, OFF> before[kSumChunks];
+#pragma unroll
+    for (int k = 0; k < kSumChunks; ++k) {
+        ChainSum<A, OFF> s;
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) s.v[c] = REV ? v[k][c] : v[k][V - OFF + c];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+            for (int c = 0; c < OFF; ++c) {
+                const A o = shfl_by<REV>(s.v[c], d);
+                if (REV ? lane + d < 32 : lane >= d) s.v[c] = add(s.v[c], o);
+            }
+        if (lane == (REV ? 0 : 31)) part[k * NW + warp] = s;
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) {
+            const A o = shfl_by<REV>(s.v[c], 1);
+            before[k].v[c] = lane == (REV ? 31 : 0) ? A{} : o;
+        }
+    }
+    if (first) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the other tiles' sums
+    ChainSum<A, OFF> carry{};
+    for (int64_t t = (REV ? tile + 1 : 0) + tid; t < (REV ? ntiles : tile); t += kThreads)
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) carry.v[c] = add(carry.v[c], sum[vec * ntiles + t].v[c]);
+    carry = block_sum<A, OFF>(carry, red);  // its barrier also publishes `part`
+    // the block's (piece, warp) totals that come first: one scan of 32 values per warp
+    static_assert(kSumChunks * NW == 32, "one warp scans the block's totals");
+    {
+        ChainSum<A, OFF> s = part[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+            for (int c = 0; c < OFF; ++c) {
+                const A o = shfl_by<REV>(s.v[c], d);
+                if (REV ? lane + d < 32 : lane >= d) s.v[c] = add(s.v[c], o);
+            }
+#pragma unroll
+        for (int k = 0; k < kSumChunks; ++k) {
+            const int at = k * NW + warp + (REV ? 1 : -1);  // inclusive total just before
+#pragma unroll
+            for (int c = 0; c < OFF; ++c) {
+                const A o = shfl_at(s.v[c], at & 31);
+                before[k].v[c] = add(before[k].v[c], carry.v[c]);
+                if (at >= 0 && at < 32) before[k].v[c] = add(before[k].v[c], o);
+            }
+        }
+    }
+    TO* y = out + vec * n;
+    ChainSum<A, OFF> ns{};
+#pragma unroll
+    for (int k = 0; k < kSumChunks; ++k) {
+        const int64_t j = tile * SumTile<A>::tile + k * SumTile<A>::chunk + tid * V;
+        A o[V];
+        load_piece<V, ALIGNED>(wout, j, n, o);
+#pragma unroll
+        for (int i = 0; i < V; ++i) o[i] = mul(o[i], add(v[k][i], before[k].v[i % OFF]));
+        if (next) {
+            A nw[V];
+            load_piece<V, ALIGNED>(next, j, n, nw);
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                ns.v[i % OFF] = add(ns.v[i % OFF], mul(nw[i], o[i]));
+        }
+        TO t[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) put(t[i], o[i]);
+        store_piece<V, ALIGNED>(y, j, n, t);
+    }
+    if (next) {
+        __syncthreads();  // every thread has read `red`
+        ns = block_sum<A, OFF>(ns, red);
+        if (tid == 0) next_sum[blockIdx.x] = ns;
+    }
+}
+
+// tab[f][0][j] = s_j W_j, tab[f][1][j] = U_j sigma_j of factor f (signs of a flipped factor
+// included); g: Gamma(j+s+1) / Gamma(j+b+1) (Jacobi), scale: W's normalisation.
+template <typename A>
+__global__ void k_sum_tables(FactorSpec F, int f, const double* __restrict__ g, double scale,
+                             const double* __restrict__ sout, const double* __restrict__ sin,
+                             A* __restrict__ tab) {
+    const int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (j >= F.ld) return;
+    A* t = tab + (int64_t)f * 2 * F.ld;
+    if (j >= F.n) {
+        t[j] = t[F.ld + j] = A{};
+        return;
+    }
+    const double par = F.par0 + F.dir * (double)f, x = (double)j, s = par + F.b;
+    FactorSpec U = F;
+    U.flip = 0;
+    double p, q, W;
+    factor_pq(U, par, j, &p, &q);
+    if (F.family == SP_ULTRA) {
+        W = (par + x) * scale;
+    } else if (j == 0) {
+        W = -q / p * (s + 3.0) * g[1] * scale;  // mu_0 W_1
+    } else {
+        W = (2.0 * x + s + 1.0) * g[j] * scale;
+    }
+    const double sign = (F.flip && (j & 1)) ? -1.0 : 1.0;
+    const double so = f == F.M - 1 && sout ? sout[j] : 1.0;
+    const double si = f == 0 && sin ? sin[j] : 1.0;
+    from_double(t[j], so * W * sign);
+    from_double(t[F.ld + j], sign * si / (p * W));
+}
+
 unsigned blocks_for(int64_t count) { return (unsigned)((count + kThreads - 1) / kThreads); }
 
 template <typename T, int OFF>
@@ -620,14 +950,169 @@ int inverse_typed(const Step& st, const void* in, void* out, int64_t batch, int 
     return TDH_OK;
 }
 
+// in: TI, out: TO, the values between the step's own factors: M (all may share one buffer when
+// they are of one type; `mid` otherwise).
+template <typename A, typename TI, typename TO, typename M, int OFF, bool REV, bool ALIGNED>
+int sums_typed(const Step& st, const void* in, void* out, int64_t batch, cudaStream_t s) {
+    using S = ChainSum<A, OFF>;
+    const int64_t n = st.n, ntiles = (n + SumTile<A>::tile - 1) / SumTile<A>::tile;
+    if (batch * ntiles > INT32_MAX) {
+        set_error("back-substitution: batch * tiles above 2^31");
+        return TDH_ERR_UNSUPPORTED;
+    }
+    const unsigned grid = (unsigned)(batch * ntiles);
+    // two sets of tile sums: a factor reads one while it writes the next factor's
+    const size_t sum_bytes = (sizeof(S) * 2 * (size_t)grid + 255) / 256 * 256;
+    const bool own_mid = st.sp_M > 1 && !std::is_same<M, TO>::value;
+    char* scr = nullptr;
+    TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&scr),
+                          sum_bytes + (own_mid ? sizeof(M) * (size_t)(batch * n) : 0), s));
+    S* sum = reinterpret_cast<S*>(scr);
+    M* mid = own_mid ? reinterpret_cast<M*>(scr + sum_bytes) : static_cast<M*>(out);
+    // A^{-1} applies the factors' inverses in order; its transpose (REV = false) in reverse
+    auto row = [&](int f, int second) {
+        const int ff = REV ? f : st.sp_M - 1 - f;
+        return static_cast<const A*>(st.sp_tab) + ((int64_t)ff * 2 + second) * st.sp_ld;
+    };
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_sum_tiles<A, TI, OFF, ALIGNED>,
+                                       static_cast<const TI*>(in), n, ntiles, row(0, REV), sum);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    for (int f = 0; f < st.sp_M && e == cudaSuccess; ++f) {
+        const bool first = f == 0, last = f + 1 == st.sp_M;
+        const A* next = last ? nullptr : row(f + 1, REV);
+        const S* from = sum + (f & 1) * (size_t)grid;
+        S* to = sum + ((f + 1) & 1) * (size_t)grid;
+        if (first && last)
+            e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, TI, TO, OFF, REV, ALIGNED>,
+                                   static_cast<const TI*>(in), static_cast<TO*>(out), n, ntiles,
+                                   row(f, REV), row(f, !REV), from, next, to, 1);
+        else if (first)
+            e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, TI, M, OFF, REV, ALIGNED>,
+                                   static_cast<const TI*>(in), mid, n, ntiles, row(f, REV),
+                                   row(f, !REV), from, next, to, 1);
+        else if (last)
+            e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, M, TO, OFF, REV, ALIGNED>,
+                                   (const M*)mid, static_cast<TO*>(out), n, ntiles, row(f, REV),
+                                   row(f, !REV), from, next, to, 0);
+        else
+            e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, M, M, OFF, REV, ALIGNED>, (const M*)mid,
+                                   mid, n, ntiles, row(f, REV), row(f, !REV), from, next, to, 0);
+    }
+    scratch_free(scr, s);
+    if (e != cudaSuccess) {
+        set_error("back-substitution: %s", cudaGetErrorString(e));
+        return TDH_ERR_CUDA;
+    }
+    note_launches(1 + st.sp_M);
+    return TDH_OK;
+}
+
+template <typename A, typename TI, typename TO, typename M, int OFF>
+int sums_launch(const Step& st, const void* in, void* out, int64_t batch, int adjoint,
+                cudaStream_t s) {
+    // 16-byte accesses: rows of the vectors and of the tables (ld a multiple of four) aligned
+    const bool al = st.n % SumTile<A>::V == 0 && (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
+    if (adjoint)
+        return al ? sums_typed<A, TI, TO, M, OFF, false, true>(st, in, out, batch, s)
+                  : sums_typed<A, TI, TO, M, OFF, false, false>(st, in, out, batch, s);
+    return al ? sums_typed<A, TI, TO, M, OFF, true, true>(st, in, out, batch, s)
+              : sums_typed<A, TI, TO, M, OFF, true, false>(st, in, out, batch, s);
+}
+
+// The step's sums: wide_in / wide_out say that in / out hold pairs of floats (between consecutive
+// inverse steps of a float32 chain).
+template <typename T, int OFF>
+int sums_dispatch(const Step& st, const void* in, void* out, int64_t batch, int adjoint,
+                  bool wide_in, bool wide_out, cudaStream_t s) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (st.sp_sums == 2) {
+            if (wide_in && wide_out)
+                return sums_launch<FF, FF, FF, FF, OFF>(st, in, out, batch, adjoint, s);
+            if (wide_in)
+                return sums_launch<FF, FF, float, FF, OFF>(st, in, out, batch, adjoint, s);
+            if (wide_out)
+                return sums_launch<FF, float, FF, FF, OFF>(st, in, out, batch, adjoint, s);
+            return sums_launch<FF, float, float, FF, OFF>(st, in, out, batch, adjoint, s);
+        }
+    }
+    return sums_launch<T, T, T, T, OFF>(st, in, out, batch, adjoint, s);
+}
+
 template <typename T>
 int launch_typed(const Step& st, const void* in, void* out, int64_t batch, int adjoint,
-                 cudaStream_t s) {
+                 bool wide_in, bool wide_out, cudaStream_t s) {
+    if (st.sp_inverse && st.sp_sums)
+        return st.sp_off == 2
+                   ? sums_dispatch<T, 2>(st, in, out, batch, adjoint, wide_in, wide_out, s)
+                   : sums_dispatch<T, 1>(st, in, out, batch, adjoint, wide_in, wide_out, s);
     if (st.sp_inverse)
         return st.sp_off == 2 ? inverse_typed<T, 2>(st, in, out, batch, adjoint, s)
                               : inverse_typed<T, 1>(st, in, out, batch, adjoint, s);
     return st.sp_off == 2 ? forward_typed<T, 2>(st, in, out, batch, adjoint, s)
                           : forward_typed<T, 1>(st, in, out, batch, adjoint, s);
+}
+
+}  // namespace
+
+namespace {
+
+// ln W at the ends of [0, n) for factor f of F (see k_sum_tables), before normalisation.
+void weight_range(const FactorSpec& F, int f, double* lo, double* hi) {
+    const double par = F.par0 + F.dir * (double)f, s = par + F.b, last = (double)(F.n - 1);
+    if (F.family == SP_ULTRA) {
+        *lo = std::log(par);
+        *hi = std::log(par + last);
+        return;
+    }
+    auto lnw = [&](double j) {
+        return std::log(2.0 * j + s + 1.0) + std::lgamma(j + s + 1.0) - std::lgamma(j + F.b + 1.0);
+    };
+    *lo = std::log((F.b + 1.0) / (s + 3.0)) + lnw(1.0);
+    *hi = F.n > 1 ? lnw(last) : *lo;
+}
+
+bool sums_serve(const FactorSpec& F) {
+    for (int f = 0; f < F.M; ++f) {
+        double lo, hi;
+        weight_range(F, f, &lo, &hi);
+        if (!(std::fabs(hi - lo) <= kSumRange)) return false;
+    }
+    return true;
+}
+
+template <typename A>
+int sum_tables(const Step& st, const FactorSpec& F, cudaStream_t s) {
+    double* g = nullptr;  // Gamma ratios of one factor (Jacobi; entry 1 is read even for n = 1)
+    const int64_t count = std::max<int64_t>(F.n, 2);
+    if (F.family == SP_JACOBI) TDH_TRY(dev_alloc_t(&g, (size_t)count));
+    int rc = TDH_OK;
+    for (int f = 0; rc == TDH_OK && f < F.M; ++f) {
+        double lo, hi;
+        weight_range(F, f, &lo, &hi);
+        const double par = F.par0 + F.dir * (double)f;
+        if (g) rc = gamma_ratio_launch(par + F.b + 1.0, F.b + 1.0, count, g, s);
+        if (rc != TDH_OK) break;
+        k_sum_tables<A><<<blocks_for(F.ld), kThreads, 0, s>>>(F, f, g, std::exp(-0.5 * (lo + hi)),
+                                                              st.scale_out, st.scale_in,
+                                                              static_cast<A*>(st.sp_tab));
+        if (cudaGetLastError() != cudaSuccess) {
+            set_error("back-substitution tables: launch failed");
+            rc = TDH_ERR_CUDA;
+        }
+    }
+    if (g) {
+        cudaStreamSynchronize(s);
+        dev_free(g);
+    }
+    return rc;
 }
 
 }  // namespace
@@ -653,9 +1138,18 @@ int sparse_prepare(Step& st, int prec, cudaStream_t s) {
     F.n = st.n;
     F.ld = (st.n + 2 + 3) / 4 * 4;  // float4 rows stay 16-byte aligned
     st.sp_ld = F.ld;
-    const int rows = st.sp_inverse ? kInvRows : 2;
-    const size_t esz = prec != TDH_FP64 ? 4 : 8;
+    if (!st.sp_inverse || !sums_serve(F))
+        st.sp_sums = 0;
+    else if (st.sp_alone)
+        st.sp_sums = 1;
+    else
+        st.sp_sums = prec != TDH_FP64 ? 2 : 0;
+    const int rows = st.sp_inverse && !st.sp_sums ? kInvRows : 2;
+    const size_t esz = prec != TDH_FP64 && st.sp_sums != 2 ? 4 : 8;
     TDH_TRY(dev_alloc(&st.sp_tab, esz * (size_t)F.ld * rows * st.sp_M));
+    if (st.sp_sums == 2) return sum_tables<FF>(st, F, s);
+    if (st.sp_sums)
+        return prec != TDH_FP64 ? sum_tables<float>(st, F, s) : sum_tables<double>(st, F, s);
     const unsigned blocks = blocks_for(F.ld * F.M);
     if (prec != TDH_FP64)
         k_sparse_tables<float><<<blocks, kThreads, 0, s>>>(F, st.scale_out, st.scale_in,
@@ -668,9 +1162,10 @@ int sparse_prepare(Step& st, int prec, cudaStream_t s) {
 }
 
 int sparse_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
-                  cudaStream_t s) {
-    if (prec != TDH_FP64) return launch_typed<float>(st, in, out, batch, adjoint, s);
-    return launch_typed<double>(st, in, out, batch, adjoint, s);
+                  bool wide_in, bool wide_out, cudaStream_t s) {
+    if (prec != TDH_FP64)
+        return launch_typed<float>(st, in, out, batch, adjoint, wide_in, wide_out, s);
+    return launch_typed<double>(st, in, out, batch, adjoint, wide_in, wide_out, s);
 }
 
 }  // namespace tdh

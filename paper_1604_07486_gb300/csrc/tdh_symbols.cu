@@ -151,6 +151,10 @@ bool is_nonpos_integer(double x) { return x <= 0.0 && std::floor(x) == x; }
 
 }  // namespace
 
+int gamma_ratio_launch(double a, double b, int64_t count, double* out, cudaStream_t st) {
+    return launch_table(ratio_spec(a, b, 0.0, 1.0, 1.0), count, out, st);
+}
+
 int chebyshev_scale_launch(int64_t n, int inverse, double* out, cudaStream_t st) {
     // Gamma(k + 1/2) / (Gamma(1/2) Gamma(k + 1)), or its reciprocal
     const double sqrtpi = 1.7724538509055160273;
