@@ -7,6 +7,11 @@
  * H ~ sum_r l_r l_r^T / a_r (Sec. 2.1, Fig. 2); and beta = A alpha is computed as
  * D1 sum_r D_{u_r} T D_{u_r} D2 alpha with u_r = l_r / sqrt(a_r) (Eq. (5)),
  * each Toeplitz product by zero-padded FFTs of length about 2N (Sec. 1).
+ * T o H itself is also smooth away from the diagonal, and the float32 and float64 executes use
+ * that instead where it holds (every conversion but Laguerre changes of one or more): its far
+ * blocks by interpolation in a tree of boxes, its near ones entry by entry, in O(N) operations
+ * and without a truncation (the hierarchical product).  The FFT form runs TDH_BF16X3 plans, and
+ * any plan whose FFT schedule is asked for (tdh_plan_set_schedule).
  *
  * Conventions for every entry point
  *   - Pointers named d_* or documented as "device" are CUDA device pointers on the current
@@ -157,11 +162,12 @@ int tdh_plan_execute(tdh_plan_t plan, const void* in, void* out, int64_t batch, 
  * The plan must have been created with TDH_FLAG_RAGGED (else TDH_ERR_INVALID_ARG) and have a
  * single T o H conversion step (Legendre/Chebyshev/ultraspherical Case 2; plan creation with
  * the flag returns UNSUPPORTED for other chains) with FFT lengths within
- * one thread-block cluster.  Vectors are grouped by FFT length on the device; each length
- * class is converted by one persistent launch that takes vectors from a work counter, and the
- * classes run concurrently on plan-owned streams forked from `stream` (capturable in a CUDA
- * graph).  Calls from several host threads are serialised while they enqueue (the fork and
- * join events are the plan's).  Asynchronous; scratch is stream-ordered (see Scratch above).
+ * one thread-block cluster.  The hierarchical product sorts the vectors by length on the device
+ * and converts vectors of similar length together, on `stream`.  On FFT schedules, vectors are
+ * grouped by FFT length; each length class is converted by one persistent launch that takes
+ * vectors from a work counter, and the classes run concurrently on plan-owned streams forked
+ * from `stream`.  Both are capturable in a CUDA graph.  Calls from several host threads are
+ * serialised while they enqueue (the fork and join events are the plan's).  Asynchronous; scratch is stream-ordered (see Scratch above).
  */
 int tdh_plan_execute_ragged(tdh_plan_t plan, const void* in, void* out, const int64_t* offsets,
                             int64_t batch, void* stream);
@@ -224,18 +230,21 @@ int tdh_plan_query(tdh_plan_t plan, int64_t* K, int64_t* n_max);
  * plan's "configurations" are, in order: the dense configuration of each T o H step of its
  * chain, then (TDH_FLAG_RAGGED plans) one per FFT length class 2^8, 2^9, ... .  At creation
  * every configuration takes its default schedule (schedule 0).  Schedules differ only in
- * the order of floating-point operations.
+ * the order of floating-point operations.  A plan that runs the hierarchical product leaves
+ * its schedules unused, and their tables unbuilt, until one is asked for.
  *
  * tdh_plan_schedule_count -- *count (host) receives the number of configurations.
  * tdh_plan_schedule_info -- info (host, 8 ints) receives, for configuration `config`:
  *   {log2 L, log2 LC, C, R, NT, MINB, index of the schedule in use, number of schedules}.
  *   Errors: INVALID_ARG (NULL plan/info, config out of range).
  * tdh_plan_set_schedule -- every configuration takes its schedule min(index, count - 1) (the
- *   execute tables are rebuilt where the schedule changes).  Synchronises `stream`.
+ *   execute tables are built where the schedule changes) and runs it from then on, in place of
+ *   the hierarchical product.  Synchronises `stream`.
  * tdh_plan_autotune -- times every schedule of every configuration on synthetic input (the
  *   dense configurations on `batch` vectors of n_max coefficients, each ragged length class on
  *   max(1, batch / classes) vectors of the class's longest length), shortest of three
- *   launches after one untimed, and keeps the fastest.  Uses about 2 * batch * n_max values of
+ *   launches after one untimed, and keeps the fastest; the hierarchical product is timed the
+ *   same way and runs where it is the faster.  Uses about 2 * batch * n_max values of
  *   device memory while it runs; synchronises `stream`.  Errors: INVALID_ARG (batch < 1),
  *   NOMEM, CUDA.
  * Both calls that change schedules are synchronous, must not run while executes of the plan

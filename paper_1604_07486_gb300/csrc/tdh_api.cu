@@ -165,6 +165,7 @@ void release_step(Step& st) {
     dev_free(st.pair_s);
     dev_free(st.pair_c);
     exec_release(st.ex);
+    hier_release(st.hier);
     st = Step{};
 }
 
@@ -172,6 +173,15 @@ void release_step(Step& st) {
 // Relative stop threshold of the Cholesky of an accuracy-targeted plan: run to the rounding
 // floor, then keep the prefix the truncation bound asks for.
 constexpr double kTargetRelTol = 1e-18;
+
+// Steps whose T and H are smooth away from the diagonal, as the hierarchical product needs: every
+// T o H step of a parameter change below one (Cases 2 and 3), and Legendre / Chebyshev.  A
+// Laguerre change beyond that has a Toeplitz part that alternates or ends.
+bool hier_serves(const Step& st) {
+    if (st.kind != TDH_LAG2LAG) return true;
+    const double d = st.p[0] - st.p[1];
+    return std::fabs(d) < 1.0;
+}
 
 int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStream_t s) {
     const int64_t n = st.n;
@@ -230,7 +240,10 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
         TDH_TRY(rc);
         st.K = K;
     }
-    return exec_prepare(st, prec, s);
+    TDH_TRY(exec_prepare(st, prec, s));
+    // split-bfloat16 steps run their tensor-core FFT passes
+    if (hier_serves(st) && !st.ex.g.tc) return hier_prepare(st, prec, s);
+    return exec_build(st, prec, s);
 }
 
 void destroy_plan_streams(tdh_plan_s* plan) {
@@ -280,31 +293,42 @@ int run(tdh_plan_t plan, const void* in, void* out, int64_t batch, void* stream,
         TDH_CUDA(cudaMemcpyAsync(out, in, bytes, cudaMemcpyDeviceToDevice, s));
         return TDH_OK;
     }
-    // A = A_m ... A_1: the first step reads `in`, later steps work in place on `out` (each
-    // cluster reads its whole vector before writing it; sparse factors save their tiles'
-    // halos first); A^T runs the steps in reverse.
+    // A = A_m ... A_1: the first step reads `in`; A^T runs the steps in reverse.  Later steps work
+    // in place where they can (the FFT kernels read a whole vector before writing it, sparse
+    // factors save their tiles' halos first); a hierarchical step reads other rows' inputs while
+    // it writes, so the steps around it alternate between `out` and a scratch buffer.
     // Between consecutive inverse sparse steps of a float32 chain the values are pairs of floats,
     // in a scratch buffer of their own.
     auto step = [&](size_t i) -> const Step& { return plan->steps[adjoint ? nsteps - 1 - i : i]; };
+    auto distinct = [&](size_t i) { return step(i).sp_M == 0 && step(i).hier.use; };
     auto wide_after = [&](size_t i) {
         return i + 1 < nsteps && step(i).sp_sums == 2 && step(i + 1).sp_sums == 2;
     };
-    bool need_wide = false;
-    for (size_t i = 0; i < nsteps; ++i) need_wide = need_wide || wide_after(i);
-    void* wide = nullptr;
-    if (need_wide) TDH_TRY(scratch_alloc(&wide, 2 * bytes, s));
+    bool need_tmp = false, need_wide = false;
+    int flips = 0;  // buffer changes still ahead: step i writes `out` when they are even
+    for (size_t i = 0; i < nsteps; ++i) {
+        if (i > 0 && distinct(i)) ++flips;
+        need_wide = need_wide || wide_after(i);
+    }
+    need_tmp = flips > 0;
+    char* scratch = nullptr;
+    const size_t tmp_bytes = need_tmp ? (bytes + 255) / 256 * 256 : 0;
+    if (need_tmp || need_wide)
+        TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&scratch),
+                              tmp_bytes + (need_wide ? 2 * bytes : 0), s));
     const void* src = in;
     int rc = TDH_OK;
     for (size_t i = 0; rc == TDH_OK && i < nsteps; ++i) {
+        if (i > 0 && distinct(i)) --flips;
         const Step& st = step(i);
         const bool win = i > 0 && wide_after(i - 1), wout = wide_after(i);
-        void* dst = wout ? wide : out;
+        void* dst = wout ? scratch + tmp_bytes : flips % 2 ? scratch : out;
         rc = st.sp_M > 0 ? sparse_launch(st, plan->params.prec, src, dst, batch, adjoint, win,
                                          wout, s)
                          : exec_launch(st, plan->params.prec, src, dst, batch, adjoint, s);
         src = dst;
     }
-    if (wide) scratch_free(wide, s);
+    if (scratch) scratch_free(scratch, s);
     return rc;
 }
 
@@ -707,7 +731,9 @@ int tdh_plan_create(int kind, int64_t n_max, const tdh_params* params, double to
             set_error("ragged batches need a single-step conversion");
             rc = TDH_ERR_UNSUPPORTED;
         } else {
-            rc = exec_prepare_ragged(plan->steps[0], params->prec, s);
+            rc = exec_prepare_ragged(plan->steps[0], params->prec);
+            if (rc == TDH_OK && !plan->steps[0].hier.use_ragged)
+                rc = exec_build(plan->steps[0], params->prec, s);
         }
         const size_t ncls = plan->steps.empty() ? 0 : plan->steps[0].rcls.size();
         for (size_t i = 0; rc == TDH_OK && i < ncls; ++i) {

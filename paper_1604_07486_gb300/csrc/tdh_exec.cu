@@ -421,6 +421,10 @@ int prepare_pairs(Step& st, cudaStream_t s) {
         sc[p] = f;
         cc[p] = (T)(1.0 / (f * f));
     }
+    dev_free(st.pair_idx);  // left by an attempt that ran out of memory
+    dev_free(st.pair_s);
+    st.pair_idx = nullptr;
+    st.pair_s = nullptr;
     TDH_TRY(dev_alloc_t(&st.pair_idx, (size_t)K));
     TDH_TRY(dev_alloc_t(&st.pair_s, (size_t)KP));
     TDH_TRY(dev_alloc(&st.pair_c, sizeof(T) * (size_t)KP));
@@ -510,26 +514,14 @@ int exec_prepare(Step& st, int prec, cudaStream_t s) {
                   (long long)st.n, logL);
         return TDH_ERR_UNSUPPORTED;
     }
-    if (prec != TDH_FP64) {
-        TDH_TRY(prepare_diagonals<float>(st, s));
-        if (st.full && st.K > 0) TDH_TRY(prepare_pairs<float>(st, s));
-        return prepare_typed<float>(st, ex, ex.g, nullptr, 0, s);
-    }
-    TDH_TRY(prepare_diagonals<double>(st, s));
-    if (st.full && st.K > 0) TDH_TRY(prepare_pairs<double>(st, s));
-    return prepare_typed<double>(st, ex, ex.g, nullptr, 0, s);
+    return prec != TDH_FP64 ? prepare_diagonals<float>(st, s) : prepare_diagonals<double>(st, s);
 }
 
-namespace {
-template <typename T>
-int prepare_ragged_typed(Step& st, int prec, cudaStream_t s) {
-    using V = typename cx<T>::t;
-    const int64_t half = (st.n + 1) / 2;
-    TDH_TRY(dev_alloc(&st.u_nat, sizeof(V) * (size_t)std::max<int64_t>(st.K, 1) * half));
-    if (st.K > 0)
-        k_u_gather<T><<<blocks_for(st.K * half), kThreads, 0, s>>>(st.u64, st.n, st.K, 1,
-                                                                   (int)half, (V*)st.u_nat);
-    TDH_CUDA(cudaGetLastError());
+int exec_prepare_ragged(Step& st, int prec) {
+    if (st.full || st.sp_M > 0) {
+        set_error("ragged batches are built for the parity-packed kinds");
+        return TDH_ERR_UNSUPPORTED;
+    }
     for (int logL = 8; logL <= st.ex.g.logL; ++logL) {
         st.rcls.emplace_back();
         ExecData& ex = st.rcls.back();
@@ -538,20 +530,51 @@ int prepare_ragged_typed(Step& st, int prec, cudaStream_t s) {
             set_error("ragged batches are built for FFT lengths within one cluster");
             return TDH_ERR_UNSUPPORTED;
         }
-        const bool nat = ex.g.C == 1;
-        TDH_TRY(prepare_typed<T>(st, ex, ex.g, nat ? st.u_nat : nullptr, nat ? half : 0, s));
     }
     return TDH_OK;
 }
+
+namespace {
+
+// The factors in natural order that the ragged single-CTA classes share, once per step: rows
+// of u_nat_ld packed pairs, as long as the largest such class reads (zero past n).
+template <typename T>
+int prepare_u_nat(Step& st, cudaStream_t s) {
+    using V = typename cx<T>::t;
+    if (st.u_nat) return TDH_OK;
+    const int cap = sizeof(T) == 4 ? 14 : 13;
+    st.u_nat_ld = std::max<int64_t>((st.n + 1) / 2, (int64_t)1 << (std::min(st.ex.g.logL, cap) - 1));
+    TDH_TRY(dev_alloc(&st.u_nat, sizeof(V) * (size_t)(std::max<int64_t>(st.K, 1) * st.u_nat_ld)));
+    if (st.K > 0)
+        k_u_gather<T><<<blocks_for(st.K * st.u_nat_ld), kThreads, 0, s>>>(
+            st.u64, st.n, st.K, 1, (int)st.u_nat_ld, (V*)st.u_nat);
+    TDH_CUDA(cudaGetLastError());
+    return TDH_OK;
+}
+
+// Tables of one FFT configuration (ex.g set) of step st: a ragged length class or the dense one.
+template <typename T>
+int build_tables_typed(Step& st, ExecData& ex, bool ragged, cudaStream_t s) {
+    const bool nat = ragged && ex.g.C == 1;  // ragged single-CTA classes share u_nat
+    if (nat) TDH_TRY(prepare_u_nat<T>(st, s));
+    if (st.full && st.K > 0 && !st.pair_c) TDH_TRY(prepare_pairs<T>(st, s));
+    TDH_TRY(prepare_typed<T>(st, ex, ex.g, nat ? st.u_nat : nullptr, nat ? st.u_nat_ld : 0, s));
+    ex.built = 1;
+    return TDH_OK;
+}
+
+int build_tables(Step& st, ExecData& ex, bool ragged, int prec, cudaStream_t s) {
+    return prec != TDH_FP64 ? build_tables_typed<float>(st, ex, ragged, s)
+                            : build_tables_typed<double>(st, ex, ragged, s);
+}
+
 }  // namespace
 
-int exec_prepare_ragged(Step& st, int prec, cudaStream_t s) {
-    if (st.full || st.sp_M > 0) {
-        set_error("ragged batches are built for the parity-packed kinds");
-        return TDH_ERR_UNSUPPORTED;
-    }
-    if (prec != TDH_FP64) return prepare_ragged_typed<float>(st, prec, s);
-    return prepare_ragged_typed<double>(st, prec, s);
+int exec_build(Step& st, int prec, cudaStream_t s) {
+    if (!st.ex.built) TDH_TRY(build_tables(st, st.ex, false, prec, s));
+    for (ExecData& ex : st.rcls)
+        if (!ex.built) TDH_TRY(build_tables(st, ex, true, prec, s));
+    return TDH_OK;
 }
 
 void exec_release(ExecData& ex) {
@@ -681,12 +704,19 @@ int launch_ragged_typed(const Step& st, const void* in, void* out, const int64_t
 int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s, const std::vector<cudaStream_t>& side,
                        const std::vector<cudaEvent_t>& ev) {
+    if (st.hier.use_ragged) return hier_launch_ragged(st, prec, in, out, offs, batch, s);
     if (prec != TDH_FP64) return launch_ragged_typed<float>(st, in, out, offs, batch, s, side, ev);
     return launch_ragged_typed<double>(st, in, out, offs, batch, s, side, ev);
 }
 
 int exec_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
                 cudaStream_t s) {
+    if (st.hier.use) return hier_launch(st, prec, in, out, batch, adjoint, s);
+    return fft_launch(st, prec, in, out, batch, adjoint, s);
+}
+
+int fft_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
+               cudaStream_t s) {
     if (st.ex.multipass) return mp_launch(st, prec, in, out, batch, adjoint, s);
     if (prec != TDH_FP64) return launch_typed<float>(st, in, out, batch, adjoint, s);
     return launch_typed<double>(st, in, out, batch, adjoint, s);
@@ -716,15 +746,11 @@ ExecData& config_data(const ConfigRef& r) { return r.cls < 0 ? r.st->ex : r.st->
 // Rebuild configuration r's tables for schedule g (nothing to do if it already runs g).
 int rebuild_config(const ConfigRef& r, int prec, const Geometry& g, cudaStream_t s) {
     ExecData& cur = config_data(r);
-    if (same_schedule(cur.g, g)) return TDH_OK;
+    if (cur.built && same_schedule(cur.g, g)) return TDH_OK;
     ExecData nx;
     nx.m = cur.m;
     nx.g = g;
-    const bool nat = r.cls >= 0 && g.C == 1;  // ragged single-CTA classes share u_nat
-    const void* su = nat ? r.st->u_nat : nullptr;
-    const int64_t ss = nat ? (r.st->n + 1) / 2 : 0;
-    const int rc = prec != TDH_FP64 ? prepare_typed<float>(*r.st, nx, g, su, ss, s)
-                                    : prepare_typed<double>(*r.st, nx, g, su, ss, s);
+    const int rc = build_tables(*r.st, nx, r.cls >= 0, prec, s);
     if (rc != TDH_OK) {
         exec_release(nx);
         return rc;
@@ -778,10 +804,11 @@ void tune_shape(const ConfigRef& r, int64_t batch, int64_t* b, int64_t* len) {
     *len = std::min<int64_t>(r.st->n, (int64_t)1 << r.st->rcls[r.cls].g.logL);
 }
 
-// Shortest of three timed launches of configuration r (after one untimed).
+// Shortest of three timed launches of configuration r (after one untimed), on its FFT schedule
+// or (hier) by the step's hierarchical product.
 template <typename T>
-int time_config(const ConfigRef& r, int64_t batch, const TuneBuffers& tb, cudaStream_t s,
-                float* ms) {
+int time_config(const ConfigRef& r, int64_t batch, const TuneBuffers& tb, bool hier,
+                cudaStream_t s, float* ms) {
     int64_t b, len;
     tune_shape(r, batch, &b, &len);
     const Step& st = *r.st;
@@ -790,8 +817,11 @@ int time_config(const ConfigRef& r, int64_t batch, const TuneBuffers& tb, cudaSt
         TDH_CUDA(cudaGetLastError());
     }
     auto launch = [&]() -> int {
-        if (r.cls < 0) return exec_launch(st, std::is_same<T, float>::value ? TDH_FP32 : TDH_FP64,
-                                          tb.in, tb.out, b, 0, s);
+        const int prec = std::is_same<T, float>::value ? TDH_FP32 : TDH_FP64;
+        if (hier)
+            return r.cls < 0 ? hier_launch(st, prec, tb.in, tb.out, b, 0, s)
+                             : hier_launch_ragged(st, prec, tb.in, tb.out, tb.offs, b, s);
+        if (r.cls < 0) return fft_launch(st, prec, tb.in, tb.out, b, 0, s);
         TDH_CUDA(cudaMemsetAsync(tb.ctr + 1, 0, sizeof(int), s));
         const ExecData& ex = st.rcls[r.cls];
         ExecParams<T> P = ragged_params<T>(st, ex, tb.in, tb.out, tb.offs, tb.list, tb.ctr,
@@ -860,22 +890,33 @@ int autotune_typed(tdh_plan_s& plan, int64_t batch, cudaStream_t s) {
         cleanup();
         return TDH_ERR_CUDA;
     }
+    float ragged_fft = 0, ragged_hier = 0;  // length classes together: they run in one call
     for (const ConfigRef& r : cfgs) {
         const std::vector<Geometry> cands =
             schedule_candidates(prec, config_data(r).g.logL, r.cls >= 0);
-        if (cands.size() < 2) continue;
         int best = -1;
         float best_ms = 0;
         for (size_t i = 0; rc == TDH_OK && i < cands.size(); ++i) {
             float ms = 0;
             rc = rebuild_config(r, prec, cands[i], s);
-            if (rc == TDH_OK) rc = time_config<T>(r, batch, tb, s, &ms);
+            if (rc == TDH_OK) rc = time_config<T>(r, batch, tb, false, s, &ms);
             if (rc == TDH_OK && (best < 0 || ms < best_ms)) {
                 best = (int)i;
                 best_ms = ms;
             }
         }
         if (rc == TDH_OK) rc = rebuild_config(r, prec, cands[best], s);
+        if (rc == TDH_OK && r.st->hier.on) {
+            float ms = 0;
+            rc = time_config<T>(r, batch, tb, true, s, &ms);
+            if (r.cls < 0) {
+                r.st->hier.use = ms <= best_ms;
+            } else {
+                ragged_fft += best_ms;
+                ragged_hier += ms;
+                r.st->hier.use_ragged = ragged_hier <= ragged_fft;
+            }
+        }
         if (rc != TDH_OK) break;
     }
     cleanup();
@@ -928,6 +969,8 @@ int exec_set_schedule(tdh_plan_s& plan, int index, cudaStream_t s) {
         TDH_TRY(rebuild_config(r, plan.params.prec, cands[std::min<size_t>(index, cands.size() - 1)],
                                s));
     }
+    // every table is there: from now on the FFT schedules asked for
+    for (Step& st : plan.steps) st.hier.use = st.hier.use_ragged = 0;
     return TDH_OK;
 }
 

@@ -119,6 +119,7 @@ struct Geometry {
 // Device data of one execute configuration.
 struct ExecData {
     Geometry g{};
+    int built = 0;        // the tables below are there
     int64_t m = 0;        // complex length of the packed vector (ceil(n/2))
     void* spec = nullptr; // [LC][C] complex: conj(DFT(symbol)) / L in the kernel's order
     void* twx = nullptr;  // [LC] complex: omega_L^{f1(pos)} (C > 1)
@@ -134,6 +135,19 @@ struct ExecData {
     void* twl_hi = nullptr;  // omega_L^{i << twl_shift}
     void* twl_lo = nullptr;  // omega_L^{i}, i < 2^twl_shift
     int twl_shift = 0;
+};
+
+// Hierarchical product of a step (tdh_hier.cuh): tables in execute precision.
+struct HierData {
+    int on = 0;           // the tables are built
+    int use = 0;          // dense executes take this path (else the FFT schedules)
+    int use_ragged = 0;   // ragged executes take it
+    int64_t mpad = 0;     // packed indices per channel, padded to whole 2048-boxes
+    void* tab = nullptr;  // one allocation: s, the two Hankel tables, leaf and transfer weights
+    void* s = nullptr;    // s[-32 .. mpad]
+    void* hf = nullptr;   // Hankel table, forward
+    void* hr = nullptr;   // Hankel table, reversed (transpose)
+    void* w = nullptr;    // Lagrange weights: leaf [P][32], then transfers [3][4][P][P]
 };
 
 // One T o H conversion step of a plan.
@@ -175,6 +189,7 @@ struct Step {
     void* d2x = nullptr;
     void* row0 = nullptr;  // CHEB2LEG: row 0 of A in execute precision, else null
     ExecData ex;
+    HierData hier;
     // rank-pair packing (full): the terms of pair p are pair_idx[2p] and pair_idx[2p+1] (sorted
     // by max_k |u_r[k] D2_k|), the second scaled by pair_s[p] on the way in and its output by
     // pair_c[p] = 1 / pair_s[p]^2 (execute precision), so both halves of the packed complex FFT
@@ -184,7 +199,8 @@ struct Step {
     void* pair_c = nullptr;
     // ragged batches: one execute configuration per FFT length 2^(8+i), sharing u_nat
     std::vector<ExecData> rcls;
-    void* u_nat = nullptr;  // [K][ceil(n/2)] packed factor pairs in execute precision
+    void* u_nat = nullptr;  // [K][u_nat_ld] packed factor pairs in execute precision
+    int64_t u_nat_ld = 0;
 };
 
 }  // namespace tdh
@@ -222,15 +238,26 @@ int gamma_ratio_launch(double a, double b, int64_t count, double* out, cudaStrea
 // P_k^(-1/2,-1/2)(1) = Gamma(k+1/2)/(Gamma(1/2) Gamma(k+1)), k < n (its reciprocal if
 // `inverse`), float64 device array: T_k = P_k^(-1/2,-1/2) / P_k^(-1/2,-1/2)(1).
 int chebyshev_scale_launch(int64_t n, int inverse, double* out, cudaStream_t s);
-// Build the execute configuration of `st` for precision `prec` (spectrum, twiddles, factors).
+// Choose the FFT geometry of `st` for precision `prec` and build its diagonals.
 int exec_prepare(Step& st, int prec, cudaStream_t s);
+// The tables of its FFT configurations (spectrum, twiddles, factors) that are not there yet:
+// at creation for steps that run their FFTs, else when a schedule is asked for.
+int exec_build(Step& st, int prec, cudaStream_t s);
 void exec_release(ExecData& ex);
 // Configurations for every FFT length a ragged batch of vectors up to st.n can need.
-int exec_prepare_ragged(Step& st, int prec, cudaStream_t s);
+int exec_prepare_ragged(Step& st, int prec);
 // Ragged batch: vector v = in[offs[v] .. offs[v+1]), length <= st.n.
 int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s, const std::vector<cudaStream_t>& side,
                        const std::vector<cudaEvent_t>& ev);
+// Hierarchical product: tables of a step it serves (hier.on says whether it does), dense and
+// ragged executes.  in and out must not overlap.
+int hier_prepare(Step& st, int prec, cudaStream_t s);
+void hier_release(HierData& h);
+int hier_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
+                cudaStream_t s);
+int hier_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
+                       int64_t batch, cudaStream_t s);
 // Execute schedules (FFT geometries with a compiled kernel) of the plan's T o H steps.
 // Configurations in order: each T o H step's dense configuration, then (ragged plans) one per
 // FFT length class.  info = {log2 L, log2 LC, C, R, NT, MINB, index, count}.
@@ -244,7 +271,10 @@ int exec_autotune(tdh_plan_s& plan, int64_t batch, cudaStream_t s);
 // Multi-pass execute of one step (FFT longer than one cluster's shared memory).
 int mp_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
               cudaStream_t s);
-// beta = A alpha (adjoint = 0) or A^T g (adjoint = 1) for one step.
+// beta = A alpha (adjoint = 0) or A^T g (adjoint = 1) for one step: its hierarchical product
+// (in and out distinct) or its FFT schedule (fft_launch; in == out allowed).
+int fft_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
+               cudaStream_t s);
 int exec_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
                 cudaStream_t s);
 }  // namespace tdh
