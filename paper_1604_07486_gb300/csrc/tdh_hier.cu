@@ -14,11 +14,11 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int kTopKernel = 32;  // 2048-boxes from which their exchange is a kernel of its own
 constexpr int kTopSplit = 8;  // ways the 2048-boxes' exchange is split over a CTA's threads
 
 template <typename T>
 struct HierParams {
-    static constexpr int P = HierP<T>::P;
     const T* in;
     T* out;
     int64_t n;       // coefficients per vector (dense)
@@ -35,8 +35,13 @@ struct HierParams {
     T* mom[kHierLevels];
     int leaf0, leaves;  // leaves [leaf0, leaves) hold coefficients (dense)
     int rev, sign_in, sign_out;
-    int nseg, seg_leaves, nvt, unvt;  // down-kernel segments; vectors per CTA (down, up)
-    short x[kHierLevels][P];
+    int aligned;        // dense: every vector starts on a 16-byte boundary
+    T* loc;             // leaf expansions [leaf][bpad][P][NC] (null: no far field)
+    int nseg, seg_leaves, nvt, unvt;  // far segments; vectors per CTA (far, moments)
+    T* top;             // 2048-boxes' exchange, [group][ntop][NC][nvt][P] (null: by k_hier_far)
+    int ntop;           // 2048-boxes of a vector
+    int run;            // leaves a warp of the near kernel walks
+    int64_t runs;       // such walks per vector group
     const int64_t* offs;  // ragged: vector i of the launch is list[i]
     const int* list;
     const int* count;     // vectors to convert, all launches of the call together
@@ -59,6 +64,9 @@ struct Vec16<float> {
         const float4 q = *reinterpret_cast<const float4*>(p);
         v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
     }
+    __device__ __forceinline__ void store(float* p) const {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    }
 };
 template <>
 struct Vec16<double> {
@@ -67,6 +75,9 @@ struct Vec16<double> {
     __device__ __forceinline__ void load(const double* p) {
         const double2 q = *reinterpret_cast<const double2*>(p);
         v[0] = q.x, v[1] = q.y;
+    }
+    __device__ __forceinline__ void store(double* p) const {
+        *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
     }
 };
 
@@ -112,18 +123,132 @@ __device__ __forceinline__ T scaled_input(const HierParams<T>& P, const T* x, in
     return (P.sign_in && (k & 1)) ? -v : v;
 }
 
+// Two values of T that go through the same operation: one 64-bit register operand in float32
+// (fma.rn.f32x2: as many multiply-adds per cycle as scalar ones in half the instructions, which
+// leaves issue slots to the loads), two scalar operations in float64.
+using F2 = float2;
+struct __align__(16) D2 {
+    double x, y;
+};
+template <typename T>
+struct PairOf;
+template <>
+struct PairOf<float> {
+    using t = F2;
+};
+template <>
+struct PairOf<double> {
+    using t = D2;
+};
+__device__ __forceinline__ F2 pair_zero(float) { return make_float2(0.0f, 0.0f); }
+__device__ __forceinline__ D2 pair_zero(double) { return D2{0.0, 0.0}; }
+__device__ __forceinline__ void pair_fma(F2& c, F2 a, F2 b) {  // c += a b
+    c = __ffma2_rn(a, b, c);
+}
+__device__ __forceinline__ void pair_fma(D2& c, D2 a, D2 b) {
+    c.x = fma(a.x, b.x, c.x);
+    c.y = fma(a.y, b.y, c.y);
+}
+__device__ __forceinline__ F2 pair_mul(F2 a, F2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ D2 pair_mul(D2 a, D2 b) { return D2{a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ F2 pair_make(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ D2 pair_make(double x, double y) { return D2{x, y}; }
+__device__ __forceinline__ float pair_x(F2 a) { return a.x; }
+__device__ __forceinline__ float pair_y(F2 a) { return a.y; }
+__device__ __forceinline__ double pair_x(D2 a) { return a.x; }
+__device__ __forceinline__ double pair_y(D2 a) { return a.y; }
+// two consecutive pairs at p (16-byte aligned)
+__device__ __forceinline__ void pair_load2(const F2* p, F2& a, F2& b) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    a = make_float2(q.x, q.y);
+    b = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void pair_load2(const D2* p, D2& a, D2& b) {
+    const double2 q0 = *reinterpret_cast<const double2*>(p);
+    const double2 q1 = *reinterpret_cast<const double2*>(p + 1);
+    a = D2{q0.x, q0.y};
+    b = D2{q1.x, q1.y};
+}
+
+__device__ __forceinline__ void load_pair(const float* p, float& a, float& b) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    a = q.x, b = q.y;
+}
+__device__ __forceinline__ void load_pair(const double* p, double& a, double& b) {
+    const double2 q = *reinterpret_cast<const double2*>(p);
+    a = q.x, b = q.y;
+}
+
+// Coefficients k, k + 1 of a vector of len coefficients (0 outside it).
+template <typename T>
+__device__ __forceinline__ void load_two(const T* x, int64_t k, int64_t len, T& a, T& b) {
+    if (k >= 0 && k + 1 < len && ((reinterpret_cast<uintptr_t>(x + k) & (2 * sizeof(T) - 1)) == 0)) {
+        if constexpr (sizeof(T) == 4) {
+            const float2 q = *reinterpret_cast<const float2*>(x + k);
+            a = q.x, b = q.y;
+        } else {
+            const double2 q = *reinterpret_cast<const double2*>(x + k);
+            a = q.x, b = q.y;
+        }
+    } else {
+        a = (k >= 0 && k < len) ? x[k] : T(0);
+        b = (k + 1 >= 0 && k + 1 < len) ? x[k + 1] : T(0);
+    }
+}
+template <typename T>
+__device__ __forceinline__ void store_two(T* y, int64_t k, int64_t len, T a, T b) {
+    if (k >= 0 && k + 1 < len && ((reinterpret_cast<uintptr_t>(y + k) & (2 * sizeof(T) - 1)) == 0)) {
+        if constexpr (sizeof(T) == 4)
+            *reinterpret_cast<float2*>(y + k) = make_float2(a, b);
+        else
+            *reinterpret_cast<double2*>(y + k) = make_double2(a, b);
+    } else {
+        if (k >= 0 && k < len) y[k] = a;
+        if (k + 1 >= 0 && k + 1 < len) y[k + 1] = b;
+    }
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+// one value (4 or 8 bytes), or zero
+template <int BYTES>
+__device__ __forceinline__ void cp_async_small(void* dst, const void* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "n"(BYTES), "r"(valid ? BYTES : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // ------------------------------------------------------------------------------- moments
 //
 // A CTA forms the moments of one 2048-box (64 leaves, their parents, ...) for unvt vectors.  A
 // warp takes one leaf of VW vectors at a time: lane (p, v) holds the 32 weights L_p in
-// registers, so each 16-byte shared load of inputs feeds 16 bytes' worth of multiply-adds.
+// registers, so each 16-byte shared load of inputs feeds 16 bytes' worth of multiply-adds; the
+// next leaf's inputs are loaded meanwhile.
 template <typename T, int NC, bool RAGGED>
-__global__ void __launch_bounds__(kThreads) k_hier_up(const __grid_constant__ HierParams<T> P) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_hier_up(const __grid_constant__ HierParams<T> P) {
     constexpr int NP = HierP<T>::P;
     constexpr int VW = 32 / NP;
     constexpr int XW = NC * kHierLeaf;                 // inputs of a leaf
     constexpr int XS = XW + 16 / (int)sizeof(T);       // padded row
     constexpr int QV = Vec16<T>::N;
+    constexpr int LPR = XW / 2;                        // lanes of a row (two inputs each)
+    constexpr int RPI = 32 / LPR;                      // rows per load instruction
+    constexpr int NL = VW / RPI > 0 ? VW / RPI : 1;    // load instructions per leaf
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_trigger();
@@ -140,31 +265,69 @@ __global__ void __launch_bounds__(kThreads) k_hier_up(const __grid_constant__ Hi
     const int row = NC * P.unvt * NP;                  // one box's moments
     T* ms1 = ms0 + (size_t)kHierTopLeaves * row;
     T* ms2 = ms1 + (size_t)(kHierTopLeaves / 4) * row;
+    T* tw = ms2 + (size_t)(kHierTopLeaves / 16) * row;  // transfer weights
+    for (int i = tid; i < 12 * NP * NP; i += kThreads) tw[i] = P.tr[i];
     const int p = lane % NP, vq = lane / NP;
     T lw[kHierLeaf];
 #pragma unroll
     for (int a = 0; a < kHierLeaf; ++a) lw[a] = P.lw[p * kHierLeaf + a];
-    const int gu = P.unvt / VW;  // vector groups per leaf
     const int64_t boxrow = (int64_t)NC * P.bpad * NP;
-    for (int item = warp; item < nl4 * gu; item += kWarps) {
-        const int li = item / gu, gv = item % gu;
+    // row rv of load i is vector i RPI + lane / LPR; a lane loads two neighbouring inputs (in
+    // reversed order they change places)
+    const int rl = lane / LPR, col = 2 * (lane % LPR);
+    const T* vx[NL];
+    int64_t vlen[NL];
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+        const int v = i * RPI + rl;
+        int64_t base = 0, len = 0;
+        if (v < VW) vector_at<T, RAGGED>(P, g0 + v, &base, &len);
+        vx[i] = P.in + base;
+        vlen[i] = len;
+    }
+    T xa[NL], xb[NL], da = T(0), db = T(0);
+    auto load = [&](int leaf) {
+        const int64_t kp = (int64_t)leaf * XW + col;
+        const int64_t k = P.rev ? P.npk - 2 - kp : kp;
+        load_two(P.din, k, P.n, da, db);
+        if (P.sign_in) {
+            if (k & 1)
+                da = -da;
+            else
+                db = -db;
+        }
+        // whole leaf inside and two-value aligned: plain loads
+        if (!RAGGED && P.aligned && k + 1 < P.n && k >= 0) {
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                xa[i] = xb[i] = T(0);
+                if (vlen[i] > 0) load_pair(vx[i] + k, xa[i], xb[i]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < NL; ++i) load_two(vx[i], k, vlen[i], xa[i], xb[i]);
+        }
+    };
+    const int first = l0 + warp;
+    if (first < l0 + nl) load(first);
+    for (int li = warp; li < nl4; li += kWarps) {
         const int leaf = l0 + li;
         T acc[NC];
 #pragma unroll
         for (int c = 0; c < NC; ++c) acc[c] = T(0);
-        if (leaf >= P.leaf0 && li < nl) {
+        if (li < nl) {
             __syncwarp();
 #pragma unroll
-            for (int v = 0; v < VW; ++v) {
-                int64_t base, len;
-                vector_at<T, RAGGED>(P, g0 + gv * VW + v, &base, &len);
-                const T* x = P.in + base;
-#pragma unroll
-                for (int i = 0; i < NC; ++i)
-                    xw[v * XS + lane + 32 * i] =
-                        scaled_input(P, x, len, (int64_t)leaf * XW + lane + 32 * i);
+            for (int i = 0; i < NL; ++i) {
+                const int v = i * RPI + rl;
+                const T a = xa[i] * da, b = xb[i] * db;
+                if (v < VW) {
+                    xw[v * XS + col] = P.rev ? b : a;
+                    xw[v * XS + col + 1] = P.rev ? a : b;
+                }
             }
             __syncwarp();
+            if (li + kWarps < nl) load(leaf + kWarps);
             const T* xv = xw + vq * XS;
 #pragma unroll
             for (int i = 0; i < XW; i += QV) {
@@ -176,42 +339,56 @@ __global__ void __launch_bounds__(kThreads) k_hier_up(const __grid_constant__ Hi
         }
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            ms0[(size_t)li * row + (c * P.unvt + gv * VW + vq) * NP + p] = acc[c];
+            ms0[(size_t)li * row + (c * P.unvt + vq) * NP + p] = acc[c];
             if (li < nl)
-                P.mom[0][leaf * boxrow + ((int64_t)c * P.bpad + g0 + gv * VW + vq) * NP + p] =
-                    acc[c];
+                P.mom[0][leaf * boxrow + ((int64_t)c * P.bpad + g0 + vq) * NP + p] = acc[c];
         }
     }
-    // parents from children, level by level
+    // parents from children, level by level: a thread takes HPT of one box's points for one
+    // vector, their weights the same for all vectors and channels
     int nb = nl4 / 4;
     const T* src = ms0;
     T* dst = ms1;
+    constexpr int HPT = sizeof(T) == 4 ? NP / 2 : 2, SPL = NP / HPT;
     for (int l = 1; l < kHierLevels; ++l) {
         __syncthreads();
         const int nbp = l < kHierLevels - 1 ? (nb + 3) & ~3 : nb;
-        for (int i = tid; i < nbp * row; i += kThreads) {
-            const int box = i / row, e = i % row;
-            const int pp = e % NP, cv = e / NP;
-            T acc = T(0);
-            if (box < nb) {
+        const int cvs = NC * P.unvt;
+        for (int i = tid; i < nbp * SPL * cvs; i += kThreads) {
+            const int cv = i % cvs, hb = i / cvs;
+            const int box = hb / SPL, p0 = hb % SPL * HPT;
+            T acc[HPT];
 #pragma unroll
+            for (int pp = 0; pp < HPT; ++pp) acc[pp] = T(0);
+            if (box < nb) {
+#pragma unroll 1
                 for (int c = 0; c < 4; ++c) {
                     const T* m = src + (size_t)(4 * box + c) * row + cv * NP;
-                    const T* w = P.tr + (((l - 1) * 4 + c) * NP + pp) * NP;
+                    const T* w = tw + (((l - 1) * 4 + c) * NP + p0) * NP;
 #pragma unroll
                     for (int q = 0; q < NP; q += QV) {
-                        Vec16<T> mv, wv;
+                        Vec16<T> mv;
                         mv.load(m + q);
-                        wv.load(w + q);
 #pragma unroll
-                        for (int j = 0; j < QV; ++j) acc += wv.v[j] * mv.v[j];
+                        for (int pp = 0; pp < HPT; ++pp) {
+                            Vec16<T> wv;
+                            wv.load(w + pp * NP + q);
+#pragma unroll
+                            for (int j = 0; j < QV; ++j) acc[pp] += wv.v[j] * mv.v[j];
+                        }
                     }
                 }
                 const int64_t gb = (l0 >> (2 * l)) + box;
                 const int c = cv / P.unvt, v = cv % P.unvt;
-                P.mom[l][gb * boxrow + ((int64_t)c * P.bpad + g0 + v) * NP + pp] = acc;
+                T* o = P.mom[l] + gb * boxrow + ((int64_t)c * P.bpad + g0 + v) * NP + p0;
+#pragma unroll
+                for (int pp = 0; pp < HPT; ++pp) o[pp] = acc[pp];
             }
-            if (l < kHierLevels - 1) dst[(size_t)box * row + e] = acc;
+            if (l < kHierLevels - 1) {
+                T* o = dst + (size_t)box * row + cv * NP + p0;
+#pragma unroll
+                for (int pp = 0; pp < HPT; ++pp) o[pp] = acc[pp];
+            }
         }
         src = dst;
         dst = ms2;
@@ -219,25 +396,113 @@ __global__ void __launch_bounds__(kThreads) k_hier_up(const __grid_constant__ Hi
     }
 }
 
-// ------------------------------------------------------------------- exchange, near field
+// ------------------------------------------------------------------------------ far field
 //
-// A CTA computes the rows of one segment (seg_leaves leaves: 64, 16, 4 or 1) of nvt vectors:
-// the exchange of the segment's boxes (and of the boxes above it, on its path), the local
-// expansions down to its leaves, the near field, and the scaled output.
+// A CTA forms the local expansions of one segment's leaves (seg_leaves leaves: 16 or 4) for NVT
+// vectors: the exchange of the segment's boxes of every level (and of the boxes above it, on
+// its path), then parents into children; the leaves' expansions go to P.loc
+// ([leaf][vector][P][NC], channels in their natural order).
 //
-// Near field: a warp takes one leaf of NV vectors; the two half-warps take half of the
-// vectors each, a lane rows r and r + 16, so each 16-byte broadcast of inputs feeds eight
-// multiply-adds, and the entries s h (formed per lane) serve all of the half-warp's vectors.
-template <typename T, int NC, int NV, bool RAGGED>
-__global__ void __launch_bounds__(kThreads, 2) k_hier_down(const __grid_constant__ HierParams<T> P) {
+// Exchange: a warp takes one box, its lanes the box's points, channels and VTL groups of VPT
+// vectors, so a coefficient s h that a lane forms (table offsets of the points are constants of
+// the level) serves VPT vectors.  Children: a thread takes one box of one vector whole, its
+// weights broadcast from shared memory.
+template <typename T, int NC, int NVT>
+struct FarShape {
+    static constexpr int NP = HierP<T>::P;
+    static constexpr int VTL = 32 / (NP * NC) < NVT ? 32 / (NP * NC) : NVT;  // vector groups
+    static constexpr int VPT = NVT / VTL;
+    static constexpr int erow = NC * NVT * NP;  // one box's expansions
+    static constexpr int trw = 3 * 4 * NP * NP;
+    static constexpr int MG = VPT * NP + 16 / (int)sizeof(T);  // staged moments of a lane group
+};
+
+// One box of level L (index i): the far boxes' moments at this lane's point.
+template <typename T, int NC, int VPT, int L>
+__device__ __forceinline__ void far_box(const T* sp, const T* hp, const T* m0, int64_t boxrow,
+                                        int d0, int d1, int step, T (&acc)[VPT]) {
     constexpr int NP = HierP<T>::P;
     constexpr int QV = Vec16<T>::N;
-    constexpr int KV = NV / 2;                 // vectors per half-warp
-    constexpr int VPT = NV < 4 ? NV : 4;       // vectors per thread of the exchange
+    constexpr int size = hier_size(L);
+    const T* m = m0 + d0 * boxrow;
+    sp += d0 * size;
+    hp += d0 * size;
+#pragma unroll 1
+    for (int d = d0; d < d1; d += step) {
+#pragma unroll
+        for (int q0 = 0; q0 < NP; q0 += QV) {
+            T cf[QV];
+#pragma unroll
+            for (int j = 0; j < QV; ++j)
+                cf[j] = sp[hier_point<NP>(L, q0 + j)] * hp[hier_point<NP>(L, q0 + j)];
+#pragma unroll
+            for (int u = 0; u < VPT; ++u) {
+                Vec16<T> mv;
+                mv.load(m + u * NP + q0);
+#pragma unroll
+                for (int j = 0; j < QV; ++j) acc[u] += cf[j] * mv.v[j];
+            }
+        }
+        m += step * boxrow;
+        sp += step * size;
+        hp += step * size;
+    }
+}
+
+// Long vectors: the exchange of the 2048-boxes, one CTA per box and NVT vectors, the far boxes
+// split over its warps; to P.top ([group][box][NC][NVT][P]).  (Within k_hier_far every segment
+// of a 2048-box would repeat it: fine for a few boxes, 3/4 of that kernel at 512 of them.)
+template <typename T, int NC, int NVT, bool RAGGED>
+__global__ void __launch_bounds__(kThreads) k_hier_top(const __grid_constant__ HierParams<T> P) {
+    using F = FarShape<T, NC, NVT>;
+    constexpr int NP = F::NP, VTL = F::VTL, VPT = F::VPT, erow = F::erow;
+    constexpr int TOP = kHierLevels - 1;
+    __shared__ T part[kWarps * erow];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_trigger();
+    const int i = blockIdx.x % P.ntop;
+    const int64_t grp = blockIdx.x / P.ntop, g0 = grp * NVT;
+    pdl_wait();  // the moments were written by the previous kernel
+    const int leaves = group_leaves<T, NC, RAGGED>(P, g0);
+    const int nb = (leaves + kHierTopLeaves - 1) / kHierTopLeaves;
+    if (i >= nb) return;
+    const int64_t boxrow = (int64_t)NC * P.bpad * NP;
+    const int p = lane % NP, vt = (lane / NP) % VTL, c = lane / (NP * VTL);
+    if (c < NC) {
+        int xp = 0;
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+            if (q == p) xp = hier_point<NP>(TOP, q);
+        T acc[VPT];
+#pragma unroll
+        for (int u = 0; u < VPT; ++u) acc[u] = T(0);
+        far_box<T, NC, VPT, TOP>(P.s - xp, P.hh + (int64_t)2 * i * hier_size(TOP) + xp + c,
+                                 P.mom[TOP] + i * boxrow + ((int64_t)c * P.bpad + g0 + vt * VPT) * NP,
+                                 boxrow, 2 + warp, nb - i, kWarps, acc);
+#pragma unroll
+        for (int u = 0; u < VPT; ++u) part[warp * erow + (c * NVT + vt * VPT + u) * NP + p] = acc[u];
+    }
+    __syncthreads();
+    for (int e = tid; e < erow; e += kThreads) {
+        T a = part[e];
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) a += part[w * erow + e];
+        P.top[(grp * P.ntop + i) * erow + e] = a;
+    }
+}
+
+template <typename T, int NC, int NVT, bool RAGGED>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_hier_far(
+    const __grid_constant__ HierParams<T> P) {
+    using F = FarShape<T, NC, NVT>;
+    constexpr int NP = F::NP, VTL = F::VTL, VPT = F::VPT, erow = F::erow;
+    constexpr int QV = Vec16<T>::N;
+    constexpr int TOP = kHierLevels - 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int xn[kHierLevels][NP];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nseg = P.nseg, SL = P.seg_leaves, NVT = P.nvt;
+    pdl_trigger();
+    const int nseg = P.nseg, SL = P.seg_leaves;
     const int seg = blockIdx.x % nseg;
     const int64_t g0 = (int64_t)(blockIdx.x / nseg) * NVT;
     const int leaves = group_leaves<T, NC, RAGGED>(P, g0);
@@ -247,226 +512,485 @@ __global__ void __launch_bounds__(kThreads, 2) k_hier_down(const __grid_constant
         return;
     }
     const int a0 = l0 * kHierLeaf;
-    const int XW = NC * (SL + 1) * kHierLeaf;  // inputs staged: the segment and one leaf more
-    const int XS = XW + 16 / (int)sizeof(T);
-    // shared memory: inputs, s window [-32, 256), h window, leaf weights, expansions
-    T* xs = reinterpret_cast<T*>(smem_raw);
-    T* sw = xs + (size_t)NVT * XS + kHierSZero;
+    // shared memory: s window [-32, 256), h window, transfer weights, expansions
+    T* sw = reinterpret_cast<T*>(smem_raw) + kHierSZero;
     constexpr int SW = 8 * kHierLeaf;
     T* hw = sw + SW;
     const int HW = 2 * SL * kHierLeaf + 10 * kHierLeaf;
-    T* lw = hw + HW;                           // [P][32]
-    const int erow = NC * NVT * NP;
-    int nloc[kHierLevels];                     // boxes of the segment (or its path) per level
-    T* ex[kHierLevels];
-    {
-        T* e = lw + NP * kHierLeaf;
-        for (int l = kHierLevels - 1; l >= 0; --l) {
-            nloc[l] = max(1, SL >> (2 * l));
-            ex[l] = e;
-            e += (size_t)(l == kHierLevels - 1 ? kTopSplit : nloc[l]) * erow;
-        }
-    }
-    // the launch's first vector group decides the boxes in play
-    if (tid < kHierLevels * NP) xn[tid / NP][tid % NP] = P.x[tid / NP][tid % NP];
+    T* tw = hw + HW;
+    const int n1 = max(1, SL / 4), n2 = max(1, SL / 16);
+    // leaves' moments [box][channel][NVT][P], rows of a box padded so that the lanes' vector
+    // groups and channels meet other banks
+    constexpr int MG = F::MG, MC = VTL * MG;   // a lane group's vectors, one channel's row
+    T* mw = tw + F::trw;
+    T* e3 = mw + (SL + 7) * NC * MC;            // [kTopSplit] parts of the 2048-box's
+    T* e2 = e3 + kTopSplit * erow;
+    T* e1 = e2 + n2 * erow;
+    T* e0 = e1 + n1 * erow;
     for (int i = tid; i < SW + kHierSZero; i += kThreads) sw[i - kHierSZero] = P.s[i - kHierSZero];
     for (int i = tid; i < HW; i += kThreads) {
         const int64_t g = 2 * (int64_t)a0 + i;
         hw[i] = g < 2 * (P.npk / NC) + kHierHPad - 1 ? P.hh[g] : T(0);
     }
-    for (int i = tid; i < NP * kHierLeaf; i += kThreads) lw[i] = P.lw[i];
-    for (int i = tid; i < XW; i += kThreads) {
-        const int64_t kp = (int64_t)NC * a0 + i;
-        const int64_t k = P.rev ? P.npk - 1 - kp : kp;
-        T d = T(0);
-        if (k >= 0 && (RAGGED || k < P.n)) {
-            // ragged: k may pass the tables' end in the last leaf; no vector reaches it
-            d = k < P.n ? P.din[k] : T(0);
-            if (P.sign_in && (k & 1)) d = -d;
+    for (int i = tid; i < F::trw; i += kThreads) tw[i] = P.tr[i];
+    if (tid == 0)
+#pragma unroll
+        for (int i = 0; i < kHierLevels * NP; ++i) xn[i / NP][i % NP] = hier_point<NP>(i / NP, i % NP);
+    __syncthreads();
+    pdl_wait();  // the moments were written by the previous kernel
+    // ---- exchange: leaves, their parents, ..., the parts of the 2048-box
+    const int64_t boxrow = (int64_t)NC * P.bpad * NP;
+    {
+        constexpr int CPC = NVT * NP / QV;      // 16-byte chunks of a channel's row
+        const int nbox = min(SL + 7, leaves - l0);
+        for (int i = tid; i < nbox * NC * CPC; i += kThreads) {
+            const int q = i % CPC, bc = i / CPC;
+            constexpr int CPG = VPT * NP / QV;  // chunks of a lane group
+            cp_async16(mw + bc * MC + q / CPG * MG + q % CPG * QV,
+                       P.mom[0] + (l0 + bc / NC) * boxrow +
+                           ((int64_t)(bc % NC) * P.bpad + g0) * NP + q * QV);
         }
-#pragma unroll 4
-        for (int v = 0; v < NVT; ++v) {
-            int64_t base, len;
-            vector_at<T, RAGGED>(P, g0 + v, &base, &len);
-            xs[(size_t)v * XS + i] = (k >= 0 && k < len) ? P.in[base + k] * d : T(0);
+        cp_async_wait_all();
+        __syncthreads();
+    }
+    const int p = lane % NP, vt = (lane / NP) % VTL, c = lane / (NP * VTL);
+    const int nbx = SL + n1 + n2 + (P.top ? 0 : kTopSplit);
+    for (int bx = warp; bx < nbx && c < NC; bx += kWarps) {
+        T acc[VPT];
+#pragma unroll
+        for (int u = 0; u < VPT; ++u) acc[u] = T(0);
+        const int64_t mo = ((int64_t)c * P.bpad + g0 + vt * VPT) * NP;
+        T* e;
+        if (bx < SL) {
+            const int i = l0 + bx;
+            far_box<T, NC, VPT, 0>(sw - xn[0][p], hw + 2 * bx * kHierLeaf + xn[0][p] + c,
+                                   mw + (bx * NC + c) * MC + vt * MG, NC * MC, 2,
+                                   min(8 - (i & 3), leaves - i), 1, acc);
+            e = e0 + bx * erow;
+        } else if (bx < SL + n1) {
+            const int i = (l0 >> 2) + bx - SL, nb = (leaves + 3) >> 2;
+            far_box<T, NC, VPT, 1>(P.s - xn[1][p], P.hh + (int64_t)2 * i * hier_size(1) + xn[1][p] + c,
+                                   P.mom[1] + i * boxrow + mo, boxrow, 2,
+                                   min(8 - (i & 3), nb - i), 1, acc);
+            e = e1 + (bx - SL) * erow;
+        } else if (bx < SL + n1 + n2) {
+            const int i = (l0 >> 4) + bx - SL - n1, nb = (leaves + 15) >> 4;
+            far_box<T, NC, VPT, 2>(P.s - xn[2][p], P.hh + (int64_t)2 * i * hier_size(2) + xn[2][p] + c,
+                                   P.mom[2] + i * boxrow + mo, boxrow, 2,
+                                   min(8 - (i & 3), nb - i), 1, acc);
+            e = e2 + (bx - SL - n1) * erow;
+        } else {
+            const int i = l0 >> 6, nb = (leaves + 63) >> 6, part = bx - SL - n1 - n2;
+            far_box<T, NC, VPT, 3>(P.s - xn[3][p], P.hh + (int64_t)2 * i * hier_size(3) + xn[3][p] + c,
+                                   P.mom[3] + i * boxrow + mo, boxrow, 2 + part, nb - i, kTopSplit,
+                                   acc);
+            e = e3 + part * erow;
+        }
+        e += (c * NVT + vt * VPT) * NP + p;
+#pragma unroll
+        for (int u = 0; u < VPT; ++u) e[u * NP] = acc[u];
+    }
+    __syncthreads();
+    for (int i = tid; i < erow; i += kThreads) {
+        T a;
+        if (P.top) {
+            a = P.top[(g0 / NVT * P.ntop + (l0 >> 6)) * erow + i];
+        } else {
+            a = e3[i];
+#pragma unroll
+            for (int k = 1; k < kTopSplit; ++k) a += e3[k * erow + i];
+        }
+        e3[i] = a;
+    }
+    // ---- parents into children; the leaves' expansions go out
+#pragma unroll 1
+    for (int l = TOP - 1; l >= 0; --l) {
+        __syncthreads();
+        const T* from = l == 2 ? e3 : l == 1 ? e2 : e1;
+        T* to = l == 2 ? e2 : l == 1 ? e1 : e0;
+        const int nb = l == 2 ? n2 : l == 1 ? n1 : SL, np = l == 2 ? 1 : l == 1 ? n2 : n1;
+        for (int it = tid; it < nb * NC * NVT; it += kThreads) {
+            const int v = it % NVT, cc = (it / NVT) % NC, bl = it / (NVT * NC);
+            const int i = (l0 >> (2 * l)) + bl;
+            const T* par = from + (np > 1 ? bl / 4 : 0) * erow + (cc * NVT + v) * NP;
+            T* ch = to + bl * erow + (cc * NVT + v) * NP;
+            const T* w = tw + (l * 4 + (i & 3)) * NP * NP;
+            T out[NP], x[NP];
+#pragma unroll
+            for (int q = 0; q < NP; q += QV) {
+                Vec16<T> o, f;
+                o.load(ch + q);
+                f.load(par + q);
+#pragma unroll
+                for (int j = 0; j < QV; ++j) {
+                    out[q + j] = o.v[j];
+                    x[q + j] = f.v[j];
+                }
+            }
+#pragma unroll
+            for (int pp = 0; pp < NP; ++pp) {
+#pragma unroll
+                for (int q = 0; q < NP; q += QV) {
+                    Vec16<T> o;
+                    o.load(w + pp * NP + q);
+#pragma unroll
+                    for (int j = 0; j < QV; ++j) out[q + j] += o.v[j] * x[pp];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < NP; q += QV) {
+                Vec16<T> o;
+#pragma unroll
+                for (int j = 0; j < QV; ++j) o.v[j] = out[q + j];
+                o.store(ch + q);
+            }
         }
     }
     __syncthreads();
-    // ---- exchange: every level's boxes at once
-    const int64_t boxrow = (int64_t)NC * P.bpad * NP;
-    const int vts = NVT / VPT;
-    pdl_wait();  // the moments were written by the previous kernel
-    if (leaves > 2) {
-        for (int l = kHierLevels - 1; l >= 0; --l) {
-            const bool topl = l == kHierLevels - 1;
-            const int size = hier_size(l);
-            const int nb = (leaves + (1 << (2 * l)) - 1) >> (2 * l);
-            const int split = topl ? kTopSplit : 1;
-            const int per = vts * NC * NP;
-            const int items = nloc[l] * split * per;
-            for (int it = tid; it < items; it += kThreads) {
-                const int p = it % NP;
-                const int vt = (it / NP) % vts;
-                const int c = (it / (NP * vts)) % NC;
-                const int bs = it / per;
-                const int bl = topl ? 0 : bs;
-                const int sp = topl ? bs : 0;
-                const int i = (l0 >> (2 * l)) + bl;
-                const int xp = xn[l][p];
-                T acc[VPT];
+    {
+        // out in whole 16-byte pieces: [leaf][vector][P][NC]
+        constexpr int PPV = NC * NP / QV;       // pieces of a vector
+        const int pieces = min(SL, leaves - l0) * NVT * PPV;
+        for (int it = tid; it < pieces; it += kThreads) {
+            const int w = it % PPV, v = (it / PPV) % NVT, bl = it / (PPV * NVT);
+            Vec16<T> o;
 #pragma unroll
-                for (int u = 0; u < VPT; ++u) acc[u] = T(0);
-                const int d1 = topl ? nb - i : min(8 - (i & 3), nb - i);
-                const T* mrow = P.mom[l] + ((int64_t)c * P.bpad + g0 + vt * VPT) * NP;
-                for (int d = 2 + sp; d < d1; d += split) {
-                    const T* m = mrow + (int64_t)(i + d) * boxrow;
-                    const T* sp0 = (l == 0 ? sw : P.s) + d * size - xp;
-                    const T* hp0 = (l == 0 ? hw + (2 * bl + d) * size
-                                           : P.hh + (int64_t)(2 * i + d) * size) + xp + c;
-#pragma unroll
-                    for (int q0 = 0; q0 < NP; q0 += QV) {
-                        T cf[QV];
-#pragma unroll
-                        for (int j = 0; j < QV; ++j) {
-                            const int x = xn[l][q0 + j];
-                            cf[j] = sp0[x] * hp0[x];
-                        }
-#pragma unroll
-                        for (int u = 0; u < VPT; ++u) {
-                            Vec16<T> mv;
-                            mv.load(m + u * NP + q0);
-#pragma unroll
-                            for (int j = 0; j < QV; ++j) acc[u] += cf[j] * mv.v[j];
-                        }
-                    }
-                }
-                T* e = ex[l] + (size_t)bs * erow + (c * NVT + vt * VPT) * NP + p;
-#pragma unroll
-                for (int u = 0; u < VPT; ++u) e[u * NP] = acc[u];
+            for (int j = 0; j < QV; ++j) {
+                const int e = w * QV + j, q = e / NC, cc = P.rev ? NC - 1 - e % NC : e % NC;
+                o.v[j] = e0[bl * erow + (cc * NVT + v) * NP + q];
             }
+            o.store(P.loc + ((int64_t)(l0 + bl) * P.bpad + g0 + v) * (NC * NP) + w * QV);
         }
-        __syncthreads();
-        for (int i = tid; i < erow; i += kThreads) {
-            T a = ex[kHierLevels - 1][i];
-            for (int k = 1; k < kTopSplit; ++k) a += ex[kHierLevels - 1][(size_t)k * erow + i];
-            ex[kHierLevels - 1][i] = a;
-        }
-        // ---- local expansions down
-        for (int l = kHierLevels - 2; l >= 0; --l) {
-            __syncthreads();
-            for (int it = tid; it < nloc[l] * erow; it += kThreads) {
-                const int bl = it / erow, e = it % erow;
-                const int q = e % NP, cv = e / NP;
-                const int i = (l0 >> (2 * l)) + bl;
-                const T* par = ex[l + 1] + (size_t)(nloc[l + 1] > 1 ? bl / 4 : 0) * erow + cv * NP;
-                const T* w = P.tr + (l * 4 + (i & 3)) * NP * NP + q;
-                T acc = ex[l][it];
-#pragma unroll
-                for (int p = 0; p < NP; ++p) acc += w[p * NP] * par[p];
-                ex[l][it] = acc;
-            }
-        }
-        __syncthreads();
     }
-    // ---- near field, local expansions at the rows, output
+}
+
+// ----------------------------------------------------------------------------- near field
+//
+// A warp walks `run` leaves of NV vectors: leaf j's scaled inputs come into its own shared
+// memory, give the off-diagonal block of leaf j - 1's rows, which are then complete (local
+// expansion, output scaling, store), and the triangle of leaf j's.  No barrier between warps.
+//
+// The two half-warps take half of the vectors each, a lane rows r and r + 16.  Values are taken
+// in pairs (two parities of one packed index, or two neighbouring indices), so one 16-byte
+// broadcast of inputs feeds four pair operations per row pair, and the entries s h a lane forms
+// serve all of its vectors.  Bound by the FP32 (FP64) pipe.
+template <typename T, int NC, int NV>
+struct NearShape {
+    static constexpr int NP = HierP<T>::P;
+    static constexpr int NPR = NC * kHierLeaf / 2;             // pairs of a leaf
+    static constexpr int CH = 16 / (int)sizeof(T);             // coefficients of a 16-byte chunk
+    static constexpr int CPR = 2 * NPR / CH;                   // chunks of a leaf's row
+    static constexpr int XS = NPR + (sizeof(T) == 4 ? 2 : 1);  // row stride, in pairs
+    static constexpr int LS = NC * NP / 2;                     // pairs of an expansion, per vector
+    static constexpr int HP = 3 * kHierLeaf;                   // Hankel window per step, in pairs
+    static constexpr int LW = (NC == 2 ? NP : NP / 2) * kHierLeaf;
+    // one CTA per SM
+    static constexpr int warps = NV * (int)sizeof(T) >= 128 ? 8 : 16;
+    // pairs of shared memory: of a warp (two input buffers), and of the CTA's tables (s pairs,
+    // leaf weights)
+    static constexpr int warp_pairs(bool ragged) {
+        return 2 * NV * XS + HP + NV * LS + (ragged ? NV * 16 / (int)(2 * sizeof(T)) : 0);
+    }
+    static constexpr int table_pairs = 3 * kHierLeaf + LW;
+};
+
+template <typename T, int NC, int NV, bool REV, bool RAGGED>
+__global__ void __launch_bounds__(32 * NearShape<T, NC, NV>::warps, 1) k_hier_near(
+    const __grid_constant__ HierParams<T> P) {
+    using S = NearShape<T, NC, NV>;
+    using P2 = typename PairOf<T>::t;
+    constexpr int KV = NV / 2;                       // vectors per half-warp
+    constexpr int NPR = S::NPR, XS = S::XS, LS = S::LS, HP = S::HP, LW = S::LW;
+    constexpr int CS = NC == 2 ? 1 : 2;              // packed indices per pair
+    constexpr int CH = S::CH, CPR = S::CPR, RPI = 32 / CPR;
+    constexpr int NIT = NV > RPI ? NV / RPI : 1;     // chunks per lane and leaf
+    constexpr int NTH = 32 * S::warps;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    P2* sp = reinterpret_cast<P2*>(smem_raw) + kHierLeaf;  // s pairs [-32, 64)
+    P2* lw = sp + 2 * kHierLeaf;                           // leaf weights [.][32]
+    P2* xs = lw + LW + (size_t)warp * S::warp_pairs(RAGGED);
+    P2* hp = xs + 2 * NV * XS;
+    P2* lc = hp + HP;
+    longlong2* vt = reinterpret_cast<longlong2*>(lc + NV * LS);  // ragged: {start, length}
+    for (int i = tid; i < 3 * kHierLeaf; i += NTH) {
+        const int m = i - kHierLeaf;
+        const T s0 = P.s[m], s1 = P.s[m + 1];
+        sp[m] = NC == 2 ? pair_make(s0, s0) : (REV ? pair_make(s1, s0) : pair_make(s0, s1));
+    }
+    for (int i = tid; i < LW; i += NTH) {
+        const int q = i / kHierLeaf, a = i % kHierLeaf;
+        lw[i] = NC == 2 ? pair_make(P.lw[i], P.lw[i])
+                        : pair_make(P.lw[2 * q * kHierLeaf + a], P.lw[(2 * q + 1) * kHierLeaf + a]);
+    }
+    __syncthreads();
+    const int64_t task = (int64_t)blockIdx.x * S::warps + warp;
+    const int64_t g0 = task / P.runs * NV;
+    int i0 = (int)(task % P.runs) * P.run;
+    bool far = false;
+    int leaves = 0;
+    if (g0 < P.batch) {
+        leaves = group_leaves<T, NC, RAGGED>(P, g0);
+        // a group's far field was formed with the leaves of the far kernel's group
+        far = P.loc && group_leaves<T, NC, RAGGED>(P, g0 / P.nvt * P.nvt) > 2;
+    }
+    const int i1 = min(i0 + P.run, leaves);
+    i0 = max(i0, P.leaf0);
+    if (i0 >= i1) {
+        pdl_wait();  // the launch must not complete before the previous one does
+        return;
+    }
+    if constexpr (RAGGED) {
+        for (int v = lane; v < NV; v += 32) {
+            int64_t base, len;
+            vector_at<T, true>(P, g0 + v, &base, &len);
+            vt[v] = make_longlong2(base, len);
+        }
+        __syncwarp();
+    }
+    auto vec = [&](int v, int64_t* base, int64_t* len) {
+        if constexpr (RAGGED) {
+            const longlong2 q = vt[v];
+            *base = q.x;
+            *len = q.y;
+        } else {
+            vector_at<T, false>(P, g0 + v, base, len);
+        }
+    };
+    // half-warp h takes vectors 2 k + h: neighbouring rows, whose broadcasts meet other banks
     const int half = lane >> 4, r = lane & 15;
-    const int gvs = NVT / NV;
-    for (int item = warp; item < SL * gvs; item += kWarps) {
-        const int li = item / gvs, gv = item % gvs;
-        const int leaf = l0 + li;
-        if (leaf >= leaves || leaf < P.leaf0) continue;
-        const int v0 = gv * NV + half * KV;
-        const T* xv = xs + (size_t)v0 * XS + NC * li * kHierLeaf;
-        const T* hb = hw + 2 * li * kHierLeaf + r;
-        T acc[KV][2][NC];
+    const int hmax = (int)(2 * (P.npk / NC)) + kHierHPad - 2;
+    const int col = lane % CPR, rv = lane / CPR;  // a lane's chunk column and first row
+    const int nv = RAGGED ? NV : (int)min((int64_t)NV, P.batch - g0);
+    // natural index of a lane's chunk of leaf j
+    auto chunk_at = [&](int j) -> int64_t {
+        return (REV ? P.npk - (int64_t)(j + 1) * 2 * NPR : (int64_t)j * 2 * NPR) + col * CH;
+    };
+    // start the copy of leaf j's inputs (unscaled) into its buffer
+    auto fetch = [&](int j) {
+        const int64_t k = chunk_at(j);
+        P2* xb = xs + (j & 1) * NV * XS;
+        if (!RAGGED && P.aligned && k >= 0 && k + CH <= P.n) {
+            const T* x = P.in + (g0 + rv) * P.n + k;
+            T* to = reinterpret_cast<T*>(xb + rv * XS) + col * CH;
 #pragma unroll
-        for (int k = 0; k < KV; ++k)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) acc[k][0][c] = acc[k][1][c] = T(0);
-        // columns b0 .. b0 + NB - 1: NB x NC = 4 inputs per vector
-        constexpr int NB = 4 / NC;
-        // rows r + 16 meet no column below 16 (s is zero left of the diagonal)
-#pragma unroll 2
-        for (int b0 = 0; b0 < 2 * kHierLeaf; b0 += NB) {
-            T A0[NB][NC], A1[NB][NC];
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                const T s0 = sw[b0 + j - r], s1 = sw[b0 + j - r - 16];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    A0[j][c] = s0 * hb[b0 + j + c];
-                    A1[j][c] = s1 * hb[b0 + j + c + 16];
-                }
+            for (int i = 0; i < NIT; ++i) {
+                if (i * RPI + rv < nv) cp_async16(to, x);
+                x += RPI * P.n;
+                to += RPI * 2 * XS;
             }
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                T x[4];
-#pragma unroll
-                for (int q = 0; q < 4; q += QV) {
-                    Vec16<T> t;
-                    t.load(xv + (size_t)k * XS + NC * b0 + q);
-#pragma unroll
-                    for (int j = 0; j < QV; ++j) x[q + j] = t.v[j];
-                }
-#pragma unroll
-                for (int j = 0; j < NB; ++j)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        acc[k][0][c] += A0[j][c] * x[j * NC + c];
-                        acc[k][1][c] += A1[j][c] * x[j * NC + c];
-                    }
-            }
-        }
-        if (leaves > 2) {
-            const T* e = ex[0] + (size_t)li * erow;
-#pragma unroll
-            for (int q = 0; q < NP; q += QV) {
-                T w0[QV], w1[QV];
-#pragma unroll
-                for (int j = 0; j < QV; ++j) {
-                    w0[j] = lw[(q + j) * kHierLeaf + r];
-                    w1[j] = lw[(q + j) * kHierLeaf + r + 16];
-                }
-#pragma unroll
-                for (int k = 0; k < KV; ++k)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        Vec16<T> t;
-                        t.load(e + (c * NVT + v0 + k) * NP + q);
-#pragma unroll
-                        for (int j = 0; j < QV; ++j) {
-                            acc[k][0][c] += w0[j] * t.v[j];
-                            acc[k][1][c] += w1[j] * t.v[j];
-                        }
-                    }
-            }
-        }
-#pragma unroll
-        for (int rr = 0; rr < 2; ++rr) {
-            const int64_t kp = (int64_t)NC * ((int64_t)leaf * kHierLeaf + r + 16 * rr);
-            // packed pair -> coefficients k .. k + NC - 1 (components swapped when reversed)
-            const int64_t k0 = P.rev ? P.npk - NC - kp : kp;
-            T d[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const int64_t k = k0 + c;
-                d[c] = (k >= 0 && k < P.n) ? P.dout[k] : T(0);
-                if (P.sign_out && (k & 1)) d[c] = -d[c];
-            }
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
+        } else {
+#pragma unroll 1
+            for (int v = rv; v < NV; v += RPI) {
                 int64_t base, len;
-                vector_at<T, RAGGED>(P, g0 + v0 + k, &base, &len);
-                T y[NC];
+                vec(v, &base, &len);
+                const T* x = P.in + base + k;
+                T* to = reinterpret_cast<T*>(xb + v * XS) + col * CH;
+                if (k >= 0 && k + CH <= len && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+                    cp_async16(to, x);
+                } else {
 #pragma unroll
-                for (int c = 0; c < NC; ++c) y[c] = acc[k][rr][P.rev ? NC - 1 - c : c] * d[c];
-                if (k0 == 0 && len > 0 && P.a00) y[0] += P.a00[0] * P.in[base];
-                T* o = P.out + base + k0;
-#pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (k0 + c >= 0 && k0 + c < len) o[c] = y[c];
+                    for (int u = 0; u < CH; ++u) {
+                        const bool in = k + u >= 0 && k + u < len;
+                        cp_async_small<(int)sizeof(T)>(to + u, in ? x + u : P.in, in);
+                    }
+                }
             }
         }
+    };
+    // a lane's input scaling of leaf j, and its entries of leaf j's Hankel window (from 64 j - 32)
+    T d[CH], hl[HP / 32], hh[HP / 32];
+    auto tables = [&](int j) {
+        const int64_t k = chunk_at(j);
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+            const int64_t kk = k + u;
+            d[u] = kk >= 0 && kk < P.n ? P.din[kk] : T(0);
+            if (P.sign_in && (kk & 1)) d[u] = -d[u];
+        }
+        const int hb = 2 * j * kHierLeaf - kHierLeaf + lane;
+#pragma unroll
+        for (int i = 0; i < HP / 32; ++i) {
+            const int g = hb + 32 * i;
+            hl[i] = g >= 0 && g < hmax ? P.hh[g] : T(0);
+            hh[i] = g >= -1 && g < hmax ? P.hh[g + 1] : T(0);
+        }
+    };
+    const P2* xv = xs;
+    // primed pair q is natural pair q, or NPR - 1 - q when reversed
+    auto two = [&](int k, int q, P2& x0, P2& x1) {
+        if constexpr (REV)
+            pair_load2(xv + 2 * k * XS + NPR - 2 - q, x1, x0);
+        else
+            pair_load2(xv + 2 * k * XS + q, x0, x1);
+    };
+    P2 acc[KV][2];
+    // acc += entries of columns CS q ... (pairs q0 <= q < NPR) for rows r and r + 16
+    auto both_rows = [&](const P2* s0, const P2* h0, int q0) {
+#pragma unroll 1
+        for (int q = q0; q < NPR; q += 2) {
+            const int b = CS * q;
+            const P2 a00 = pair_mul(s0[b], h0[b]);
+            const P2 a01 = pair_mul(s0[b + CS], h0[b + CS]);
+            const P2 a10 = pair_mul(s0[b - 16], h0[b + 16]);
+            const P2 a11 = pair_mul(s0[b + CS - 16], h0[b + CS + 16]);
+#pragma unroll
+            for (int k = 0; k < KV; ++k) {
+                P2 x0, x1;
+                two(k, q, x0, x1);
+                pair_fma(acc[k][0], a00, x0);
+                pair_fma(acc[k][1], a10, x0);
+                pair_fma(acc[k][0], a01, x1);
+                pair_fma(acc[k][1], a11, x1);
+            }
+        }
+    };
+    fetch(i0);
+    cp_async_commit();
+    tables(i0);
+#pragma unroll 1
+    for (int j = i0; j <= i1; ++j) {
+        // ---- leaf j's inputs are here: scale what this lane copied
+        cp_async_wait<0>();
+        if (j < leaves) {
+            T* to = reinterpret_cast<T*>(xs + (j & 1) * NV * XS + rv * XS) + col * CH;
+#pragma unroll
+            for (int i = 0; i < NIT; ++i) {
+                if (i * RPI + rv < NV) {
+                    Vec16<T> q;
+                    q.load(to);
+#pragma unroll
+                    for (int u = 0; u < CH; ++u) q.v[u] *= d[u];
+                    q.store(to);
+                }
+                to += RPI * 2 * XS;
+            }
+#pragma unroll
+            for (int i = 0; i < HP / 32; ++i)
+                hp[32 * i + lane] = REV ? pair_make(hh[i], hl[i]) : pair_make(hl[i], hh[i]);
+        }
+        __syncwarp();
+        // ---- start what comes next: leaf j - 1's expansions and scaling, leaf j + 1's inputs
+        T da[2], db[2];
+        if (j > i0) {
+            if (j == i0 + 1) pdl_wait();  // the expansions were written by the previous kernel
+            if (far) {
+                const T* e = P.loc + ((int64_t)(j - 1) * P.bpad + g0) * (NC * S::NP);
+#pragma unroll
+                for (int i = lane; i < NV * NC * S::NP / CH; i += 32)
+                    cp_async16(reinterpret_cast<T*>(lc) + i * CH, e + i * CH);
+            }
+#pragma unroll
+            for (int rr = 0; rr < 2; ++rr) {
+                const int64_t kp = (int64_t)NC * ((int64_t)(j - 1) * kHierLeaf + r + 16 * rr);
+                const int64_t k0 = REV ? P.npk - NC - kp : kp;
+                da[rr] = db[rr] = T(0);
+                if constexpr (NC == 2)
+                    load_two(P.dout, k0, P.n, da[rr], db[rr]);
+                else if (k0 >= 0 && k0 < P.n)
+                    da[rr] = P.dout[k0];
+                if (P.sign_out) {
+                    if (k0 & 1)
+                        da[rr] = -da[rr];
+                    else
+                        db[rr] = -db[rr];
+                }
+            }
+        }
+        cp_async_commit();
+        if (j < i1 && j + 1 < leaves) {
+            fetch(j + 1);
+            tables(j + 1);
+        }
+        cp_async_commit();
+        xv = xs + (j & 1) * NV * XS + half * XS;
+        if (j > i0) {
+            // ---- off-diagonal block, rows of leaf j - 1 and columns of leaf j:
+            // l = 32 (j-1) + r + 32 j + b, window from 64 j - 32
+            if (j < leaves) both_rows(sp + kHierLeaf - r, hp + r, 0);
+            // ---- rows of leaf j - 1 are complete but for the far field
+            if (far) {
+                cp_async_wait<1>();
+                __syncwarp();
+#pragma unroll 1
+                for (int q = 0; q < LS; q += 2) {
+                    const P2 w00 = lw[q * kHierLeaf + r], w10 = lw[q * kHierLeaf + r + 16];
+                    const P2 w01 = lw[(q + 1) * kHierLeaf + r];
+                    const P2 w11 = lw[(q + 1) * kHierLeaf + r + 16];
+#pragma unroll
+                    for (int k = 0; k < KV; ++k) {
+                        P2 x0, x1;
+                        pair_load2(lc + (2 * k + half) * LS + q, x0, x1);
+                        pair_fma(acc[k][0], w00, x0);
+                        pair_fma(acc[k][1], w10, x0);
+                        pair_fma(acc[k][0], w01, x1);
+                        pair_fma(acc[k][1], w11, x1);
+                    }
+                }
+            }
+#pragma unroll
+            for (int rr = 0; rr < 2; ++rr) {
+                const int64_t kp = (int64_t)NC * ((int64_t)(j - 1) * kHierLeaf + r + 16 * rr);
+                const int64_t k0 = REV ? P.npk - NC - kp : kp;
+                const bool direct = k0 == 0 && P.a00;
+                if (!RAGGED && P.aligned && !direct && k0 >= 0 && k0 + NC <= P.n) {
+                    T* o = P.out + (g0 + half) * P.n + k0;
+#pragma unroll
+                    for (int k = 0; k < KV; ++k) {
+                        if (2 * k + half < nv) {
+                            if constexpr (NC == 2)
+                                *reinterpret_cast<P2*>(o) =
+                                    pair_mul(acc[k][rr], pair_make(da[rr], db[rr]));
+                            else
+                                *o = (pair_x(acc[k][rr]) + pair_y(acc[k][rr])) * da[rr];
+                        }
+                        o += 2 * P.n;
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < KV; ++k) {
+                        int64_t base, len;
+                        vec(2 * k + half, &base, &len);
+                        T* o = P.out + base;
+                        T ya, yb = T(0);
+                        if constexpr (NC == 2) {
+                            ya = pair_x(acc[k][rr]) * da[rr];
+                            yb = pair_y(acc[k][rr]) * db[rr];
+                        } else {
+                            ya = (pair_x(acc[k][rr]) + pair_y(acc[k][rr])) * da[rr];
+                        }
+                        if (direct && len > 0) ya += P.a00[0] * P.in[base];
+                        if constexpr (NC == 2)
+                            store_two(o, k0, len, ya, yb);
+                        else if (k0 >= 0 && k0 < len)
+                            o[k0] = ya;
+                    }
+                }
+            }
+        }
+        if (j < i1) {
+            // ---- triangle of leaf j: l = 64 j + r + b (s is zero left of the diagonal; rows
+            // r + 16 meet no column below 16)
+#pragma unroll
+            for (int k = 0; k < KV; ++k) acc[k][0] = acc[k][1] = pair_zero(T(0));
+            const P2* s0 = sp - r;
+            const P2* h0 = hp + kHierLeaf + r;
+#pragma unroll 1
+            for (int q = 0; q < NPR / 2; q += 2) {
+                const int b = CS * q;
+                const P2 a00 = pair_mul(s0[b], h0[b]);
+                const P2 a01 = pair_mul(s0[b + CS], h0[b + CS]);
+#pragma unroll
+                for (int k = 0; k < KV; ++k) {
+                    P2 x0, x1;
+                    two(k, q, x0, x1);
+                    pair_fma(acc[k][0], a00, x0);
+                    pair_fma(acc[k][0], a01, x1);
+                }
+            }
+            both_rows(s0, h0, NPR / 2);
+        }
+        __syncwarp();  // every lane is done with the buffers this step read
     }
 }
 
@@ -624,16 +1148,6 @@ __global__ void k_hier_scatter(const int64_t* __restrict__ offs, int64_t batch, 
 
 // ------------------------------------------------------------------------------ host side
 
-// Chebyshev points of a box of `size` packed indices, rounded to distinct integers.
-void hier_points(int size, int P, int* x) {
-    const double pi = 3.14159265358979323846;
-    for (int i = 0; i < P; ++i)
-        x[i] = (int)std::lrint(0.5 * size - 0.5 -
-                               0.5 * (size - 1) * std::cos(pi * (2 * i + 1) / (2.0 * P)));
-    for (int i = 1; i < P; ++i) x[i] = std::max(x[i], x[i - 1] + 1);
-    for (int i = P - 1; i >= 0; --i) x[i] = std::min(x[i], size - P + i);
-}
-
 double lagrange(const int* x, int P, int i, double at) {
     double v = 1.0;
     for (int j = 0; j < P; ++j)
@@ -689,7 +1203,8 @@ int prepare_typed(Step& st, cudaStream_t s) {
             sym, sym + N, H.mpad, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
             static_cast<T*>(H.hr));
         int x[kHierLevels][P];
-        for (int l = 0; l < kHierLevels; ++l) hier_points(hier_size(l), P, x[l]);
+        for (int l = 0; l < kHierLevels; ++l)
+            for (int p = 0; p < P; ++p) x[l][p] = hier_point<P>(l, p);
         for (int p = 0; p < P; ++p)
             for (int a = 0; a < kHierLeaf; ++a)
                 w[(size_t)p * kHierLeaf + a] = (T)lagrange(x[0], P, p, a);
@@ -714,22 +1229,19 @@ int prepare_typed(Step& st, cudaStream_t s) {
     return rc;
 }
 
-// Launch shape of one execute.
-struct Shape {
-    int NV;           // vectors per warp of the down kernel
-    int gv, gu;       // warp groups of vectors per CTA (down, up)
-    int seg_leaves;
-    int64_t chunk;    // vectors per pass over the moment scratch
-};
-
-template <typename T>
-size_t down_smem(int NC, int SL, int NVT) {
-    constexpr int P = HierP<T>::P;
-    size_t e = (size_t)NVT * (NC * (SL + 1) * kHierLeaf + 16 / sizeof(T));
-    e += kHierSZero + 8 * kHierLeaf + 2 * SL * kHierLeaf + 10 * kHierLeaf + P * kHierLeaf;
+template <typename T, int NC, int NVT>
+size_t far_smem(int SL) {
+    using F = FarShape<T, NC, NVT>;
     size_t boxes = kTopSplit;
     for (int l = 0; l < kHierLevels - 1; ++l) boxes += std::max(1, SL >> (2 * l));
-    return sizeof(T) * (e + boxes * NC * NVT * P);
+    return sizeof(T) * (kHierSZero + 8 * kHierLeaf + 2 * SL * kHierLeaf + 10 * kHierLeaf + F::trw +
+                        (SL + 7) * NC * F::VTL * F::MG + boxes * F::erow);
+}
+
+template <typename T, int NC, int NV, bool RAGGED>
+constexpr size_t near_smem() {
+    using S = NearShape<T, NC, NV>;
+    return 2 * sizeof(T) * (size_t)(S::table_pairs + S::warps * S::warp_pairs(RAGGED));
 }
 
 template <typename T>
@@ -738,39 +1250,19 @@ size_t up_smem(int NC, int NVT) {
     constexpr int VW = 32 / P;
     return sizeof(T) * ((size_t)kWarps * VW * (NC * kHierLeaf + 16 / sizeof(T)) +
                         (size_t)(kHierTopLeaves + kHierTopLeaves / 4 + kHierTopLeaves / 16) * NC *
-                            NVT * P);
+                            NVT * P +
+                        (size_t)12 * P * P);
 }
 
 constexpr size_t kMaxSmem = 227 * 1024;
 
 template <typename T>
-Shape choose_shape(int NC, int64_t leaves, int64_t batch) {
-    Shape sh{};
-    const int vmax = sizeof(T) == 4 ? 16 : 8;
-    sh.NV = batch >= vmax * 3 / 4 ? vmax : (batch > 2 ? 8 : 2);
-    const int64_t groups = (batch + sh.NV - 1) / sh.NV;
-    // the longest segments that still give every SM a few CTAs
-    const int64_t want = 4 * (int64_t)sm_count();
-    sh.seg_leaves = 16;
-    while (sh.seg_leaves > 1 &&
-           (sh.seg_leaves >= 4 * leaves || (leaves / sh.seg_leaves) * groups < want))
-        sh.seg_leaves /= 4;
-    // short segments: several vector groups per CTA, so that all eight warps have a leaf
-    sh.gv = 1;
-    const int64_t per = std::min<int64_t>(leaves, sh.seg_leaves);
-    while (per * sh.gv < kWarps && (int64_t)(2 * sh.gv) * want <= groups * ((leaves + per - 1) / per))
-        sh.gv *= 2;
-    while (sh.gv > 1 && down_smem<T>(NC, sh.seg_leaves, sh.NV * sh.gv) > kMaxSmem) sh.gv /= 2;
-    sh.gu = 1;
-    return sh;
-}
-
-template <typename T>
 cudaError_t launch_cfg(void (*kern)(const HierParams<T>), unsigned grid, size_t smem,
-                       cudaStream_t s, bool pdl, const HierParams<T>& P) {
+                       cudaStream_t s, bool pdl, const HierParams<T>& P,
+                       int threads = kThreads) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute a[1];
@@ -783,7 +1275,8 @@ cudaError_t launch_cfg(void (*kern)(const HierParams<T>), unsigned grid, size_t 
 
 template <typename T, int NC, bool RAGGED>
 int launch_up(const HierParams<T>& P, unsigned grid, cudaStream_t s) {
-    auto kern = k_hier_up<T, NC, RAGGED>;
+    auto kern = k_hier_up<T, NC, RAGGED>;  // launched without overlap: its input may be the
+                                           // previous step's output
     static PerDevice once;
     cudaError_t e = per_device(once, [&](int*) {
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -798,30 +1291,71 @@ int launch_up(const HierParams<T>& P, unsigned grid, cudaStream_t s) {
     return TDH_OK;
 }
 
-template <typename T, int NC, int NV, bool RAGGED>
-int launch_down_nv(const HierParams<T>& P, unsigned grid, bool pdl, cudaStream_t s) {
-    auto kern = k_hier_down<T, NC, NV, RAGGED>;
+template <typename T, int NC, int NVT, bool RAGGED>
+int launch_far(const HierParams<T>& P, unsigned grid, cudaStream_t s) {
+    auto kern = k_hier_far<T, NC, NVT, RAGGED>;
     static PerDevice once;
     cudaError_t e = per_device(once, [&](int*) {
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kMaxSmem - 1024);
     });
     if (e == cudaSuccess)
-        e = launch_cfg<T>(kern, grid, down_smem<T>(NC, P.seg_leaves, P.nvt), s, pdl, P);
+        e = launch_cfg<T>(kern, grid, far_smem<T, NC, NVT>(P.seg_leaves), s, true, P);
     if (e != cudaSuccess) {
-        set_error("hierarchical product: %s", cudaGetErrorString(e));
+        set_error("hierarchical far field: %s", cudaGetErrorString(e));
         return TDH_ERR_CUDA;
     }
     note_launches(1);
     return TDH_OK;
 }
 
+template <typename T, int NC, int NVT, bool RAGGED>
+int launch_top(const HierParams<T>& P, unsigned grid, cudaStream_t s) {
+    const cudaError_t e = launch_cfg<T>(k_hier_top<T, NC, NVT, RAGGED>, grid, 0, s, true, P);
+    if (e != cudaSuccess) {
+        set_error("hierarchical far field: %s", cudaGetErrorString(e));
+        return TDH_ERR_CUDA;
+    }
+    note_launches(1);
+    return TDH_OK;
+}
+
+template <typename T, int NC, int NV, bool REV, bool RAGGED>
+int launch_near_rev(const HierParams<T>& P, unsigned grid, bool pdl, cudaStream_t s) {
+    constexpr size_t smem = near_smem<T, NC, NV, RAGGED>();
+    static_assert(smem <= kMaxSmem, "shared memory budget");
+    auto kern = k_hier_near<T, NC, NV, REV, RAGGED>;
+    static PerDevice once;
+    cudaError_t e = per_device(once, [&](int*) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
+    if (e == cudaSuccess)
+        e = launch_cfg<T>(kern, grid, smem, s, pdl, P, 32 * NearShape<T, NC, NV>::warps);
+    if (e != cudaSuccess) {
+        set_error("hierarchical near field: %s", cudaGetErrorString(e));
+        return TDH_ERR_CUDA;
+    }
+    note_launches(1);
+    return TDH_OK;
+}
+
+template <typename T, int NC, int NV, bool RAGGED>
+int launch_near_nv(const HierParams<T>& P, int64_t nb, bool pdl, cudaStream_t s) {
+    const int64_t tasks = (nb + NV - 1) / NV * P.runs;
+    constexpr int W = NearShape<T, NC, NV>::warps;
+    const unsigned grid = (unsigned)((tasks + W - 1) / W);
+    if constexpr (!RAGGED)
+        if (P.rev) return launch_near_rev<T, NC, NV, true, false>(P, grid, pdl, s);
+    return launch_near_rev<T, NC, NV, false, RAGGED>(P, grid, pdl, s);
+}
+
 template <typename T, int NC, bool RAGGED>
-int launch_down(const HierParams<T>& P, int NV, unsigned grid, bool pdl, cudaStream_t s) {
-    if constexpr (sizeof(T) == 4)
-        if (NV == 16) return launch_down_nv<T, NC, 16, RAGGED>(P, grid, pdl, s);
-    if (NV == 8) return launch_down_nv<T, NC, 8, RAGGED>(P, grid, pdl, s);
-    return launch_down_nv<T, NC, 2, RAGGED>(P, grid, pdl, s);
+int launch_near(const HierParams<T>& P, int NV, int64_t nb, bool pdl, cudaStream_t s) {
+    constexpr int VMAX = sizeof(T) == 4 ? 32 : 16;
+    if (NV == VMAX) return launch_near_nv<T, NC, VMAX, RAGGED>(P, nb, pdl, s);
+    if (NV == 16) return launch_near_nv<T, NC, 16, RAGGED>(P, nb, pdl, s);
+    if (NV == 8) return launch_near_nv<T, NC, 8, RAGGED>(P, nb, pdl, s);
+    return launch_near_nv<T, NC, 2, RAGGED>(P, nb, pdl, s);
 }
 
 // The direct product's shared memory, and whether it is the faster way: its work is m^2 B
@@ -876,6 +1410,7 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     P.dout = static_cast<const T*>(adjoint ? st.d2x : st.d1x);
     P.a00 = st.j0 == 1 ? static_cast<const T*>(st.row0) : nullptr;
     P.rev = adjoint;
+    P.aligned = st.n * (int64_t)sizeof(T) % 16 == 0;
     P.sign_in = st.sign_in;
     P.sign_out = st.sign_out;
     if (adjoint) {
@@ -885,11 +1420,6 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         P.leaf0 = 0;
         P.leaves = (int)((m + kHierLeaf - 1) / kHierLeaf);
     }
-    for (int l = 0; l < kHierLevels; ++l) {
-        int x[NP];
-        hier_points(hier_size(l), NP, x);
-        for (int p = 0; p < NP; ++p) P.x[l][p] = (short)x[p];
-    }
     const int64_t real_leaves = (m + kHierLeaf - 1) / kHierLeaf;
     if (!RAGGED && direct_serves<T>(NC, m, batch)) {
         P.batch = batch;
@@ -897,20 +1427,46 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         P.out = static_cast<T*>(out);
         return batch == 1 ? launch_direct<T, NC, 1>(P, m, s) : launch_direct<T, NC, 4>(P, m, s);
     }
-    const Shape sh = choose_shape<T>(NC, real_leaves, batch);
-    P.seg_leaves = sh.seg_leaves;
-    P.nvt = sh.NV * sh.gv;
+    // vectors of a near-field warp, and of a far-field CTA
+    constexpr int VMAX = sizeof(T) == 4 ? 32 : 16;
+    constexpr int FMAX = sizeof(T) == 4 ? 16 : 8;
+    P.nvt = batch > 2 ? FMAX : 2;
     P.unvt = 32 / NP;
-    P.nseg = (P.leaves + sh.seg_leaves - 1) / sh.seg_leaves;
+    // Near field: vectors of a warp (twice as many on half as many warps do the same work per SM
+    // and step with fewer loads, about 15 % less time) and leaves it walks (a walk loads one leaf
+    // more than it completes).  One CTA per SM is resident: the waves should be full.
+    int NV = 2;
+    double best = 0;
+    for (int nv = batch > 2 ? VMAX / (sizeof(T) == 4 ? 4 : 2) : 2; nv <= VMAX; nv *= 2) {
+        const int64_t slots = (nv == VMAX ? 8 : 16) * (int64_t)sm_count();
+        const int64_t vgroups = (batch + nv - 1) / nv;
+        const double step = nv == VMAX ? 1.0 : nv == 16 || sizeof(T) == 8 ? 1.15 * nv / (VMAX / 2) : 0.8;
+        for (int run = 16; run >= 1; --run) {
+            const int64_t tasks = (real_leaves + run - 1) / run * vgroups;
+            const double cost = (double)((tasks + slots - 1) / slots) * (run + 0.4) * step;
+            if (best == 0 || cost < best) {
+                best = cost;
+                P.run = run;
+                NV = nv;
+            }
+        }
+        if (batch <= 2) break;
+    }
+    P.runs = (P.leaves + P.run - 1) / P.run;
+    P.seg_leaves = real_leaves > 4 ? 16 : 4;
+    P.nseg = (P.leaves + P.seg_leaves - 1) / P.seg_leaves;
     const int64_t ntop = (P.leaves + kHierTopLeaves - 1) / kHierTopLeaves;
-    // moments of every box of a vector; at most about 1 GB of them at a time
+    // moments of every box and expansions of every leaf of a vector; about 1 GB at a time
     int64_t boxes[kHierLevels], total = 0;
     for (int l = 0; l < kHierLevels; ++l) total += boxes[l] = (H.mpad / kHierLeaf) >> (2 * l);
     const bool far = real_leaves > 2;
-    const int64_t per_vec = total * NC * NP * (int64_t)sizeof(T);
+    P.ntop = (int)ntop;
+    const bool top = ntop >= kTopKernel;
+    const int64_t per_vec =
+        (total + boxes[0] + (top ? ntop : 0)) * NC * NP * (int64_t)sizeof(T);
+    const int unit = std::max(std::max(P.nvt, P.unvt), NV);  // powers of two
     int64_t chunk = std::max<int64_t>(1, ((int64_t)1 << 30) / per_vec);
-    chunk = std::min(chunk, (int64_t)INT32_MAX / 2 / std::max<int64_t>(P.nseg, ntop));
-    const int unit = std::max(P.nvt, P.unvt);  // both powers of two
+    chunk = std::min(chunk, (int64_t)INT32_MAX / 4 / std::max<int64_t>(P.runs, ntop));
     chunk = std::max<int64_t>(unit, chunk / unit * unit);
     chunk = std::min<int64_t>(chunk, (batch + unit - 1) / unit * unit);
     T* mom = nullptr;
@@ -920,6 +1476,8 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         P.mom[l] = mom;
         if (mom) mom += boxes[l] * NC * NP * chunk;
     }
+    P.loc = mom;
+    P.top = top ? mom + boxes[0] * NC * NP * chunk : nullptr;
     int rc = TDH_OK;
     for (int64_t b0 = 0; rc == TDH_OK && b0 < batch; b0 += chunk) {
         const int64_t nb = std::min(chunk, batch - b0);
@@ -936,12 +1494,19 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
             P.out += b0 * st.n;
         }
         if (far) {
-            const int64_t gu = ((nb + P.nvt - 1) / P.nvt * P.nvt + P.unvt - 1) / P.unvt;
-            rc = launch_up<T, NC, RAGGED>(P, (unsigned)(gu * ntop), s);
+            const int64_t groups = (nb + P.nvt - 1) / P.nvt;
+            rc = launch_up<T, NC, RAGGED>(
+                P, (unsigned)((groups * P.nvt + P.unvt - 1) / P.unvt * ntop), s);
+            const unsigned grid = (unsigned)(groups * P.nseg);
+            if (rc == TDH_OK && top)
+                rc = P.nvt == FMAX
+                         ? launch_top<T, NC, FMAX, RAGGED>(P, (unsigned)(groups * ntop), s)
+                         : launch_top<T, NC, 2, RAGGED>(P, (unsigned)(groups * ntop), s);
+            if (rc == TDH_OK)
+                rc = P.nvt == FMAX ? launch_far<T, NC, FMAX, RAGGED>(P, grid, s)
+                                   : launch_far<T, NC, 2, RAGGED>(P, grid, s);
         }
-        if (rc == TDH_OK)
-            rc = launch_down<T, NC, RAGGED>(
-                P, sh.NV, (unsigned)((nb + P.nvt - 1) / P.nvt * P.nseg), far, s);
+        if (rc == TDH_OK) rc = launch_near<T, NC, RAGGED>(P, NV, nb, far, s);
     }
     if (far) scratch_free(P.mom[0], s);
     return rc;

@@ -39,6 +39,26 @@ struct HierP {
     static constexpr int P = sizeof(T) == 4 ? 8 : 16;
 };
 
+// The points of a box, per level: round((size - 1)/2 (1 - cos(pi (2i + 1) / (2P)))), kept distinct.
+template <int P>
+__host__ __device__ constexpr int hier_point(int level, int i) {
+    static_assert(P == 8 || P == 16, "points per box");
+    if constexpr (P == 8) {
+        constexpr int x[kHierLevels][8] = {{0, 3, 7, 12, 19, 24, 28, 31},
+                                           {1, 11, 28, 51, 76, 99, 116, 126},
+                                           {5, 43, 114, 206, 305, 397, 468, 506},
+                                           {20, 172, 455, 824, 1223, 1592, 1875, 2027}};
+        return x[level][i];
+    } else {
+        constexpr int x[kHierLevels][16] = {
+            {0, 1, 2, 4, 6, 8, 11, 14, 17, 20, 23, 25, 27, 29, 30, 31},
+            {0, 3, 7, 14, 23, 34, 45, 57, 70, 82, 93, 104, 113, 120, 124, 127},
+            {1, 11, 30, 58, 93, 135, 181, 230, 281, 330, 376, 418, 453, 481, 500, 510},
+            {5, 44, 121, 232, 374, 541, 726, 923, 1124, 1321, 1506, 1673, 1815, 1926, 2003, 2042}};
+        return x[level][i];
+    }
+}
+
 __host__ __device__ constexpr int hier_size(int level) { return kHierLeaf << (2 * level); }
 
 }  // namespace tdh
