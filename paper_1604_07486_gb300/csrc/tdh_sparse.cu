@@ -845,7 +845,8 @@ __global__ void k_sum_tables(FactorSpec F, int f, const double* __restrict__ g, 
     const double so = f == F.M - 1 && sout ? sout[j] : 1.0;
     const double si = f == 0 && sin ? sin[j] : 1.0;
     from_double(t[j], so * W * sign);
-    from_double(t[F.ld + j], sign * si / (p * W));
+    from_double(t[F.ld + j],
+                sign * si * (F.family == SP_ULTRA ? 1.0 / (par * scale) : 1.0 / (p * W)));
 }
 
 unsigned blocks_for(int64_t count) { return (unsigned)((count + kThreads - 1) / kThreads); }
@@ -1100,9 +1101,12 @@ int sum_tables(const Step& st, const FactorSpec& F, cudaStream_t s) {
         const double par = F.par0 + F.dir * (double)f;
         if (g) rc = gamma_ratio_launch(par + F.b + 1.0, F.b + 1.0, count, g, s);
         if (rc != TDH_OK) break;
-        k_sum_tables<A><<<blocks_for(F.ld), kThreads, 0, s>>>(F, f, g, std::exp(-0.5 * (lo + hi)),
-                                                              st.scale_out, st.scale_in,
-                                                              static_cast<A*>(st.sp_tab));
+        // ultraspherical U is the constant 1 / (l scale): a power of two, so that rounding it
+        // leaves no error common to all terms
+        double scale = std::exp(-0.5 * (lo + hi));
+        if (F.family == SP_ULTRA) scale = std::exp2(std::round(std::log2(scale * par))) / par;
+        k_sum_tables<A><<<blocks_for(F.ld), kThreads, 0, s>>>(
+            F, f, g, scale, st.scale_out, st.scale_in, static_cast<A*>(st.sp_tab));
         if (cudaGetLastError() != cudaSuccess) {
             set_error("back-substitution tables: launch failed");
             rc = TDH_ERR_CUDA;
