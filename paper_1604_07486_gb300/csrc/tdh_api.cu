@@ -170,9 +170,10 @@ void release_step(Step& st) {
 }
 
 // Build one conversion step: symbols (a1), pivoted Cholesky (a2), execute tables (a3).
-// Relative stop threshold of the Cholesky of an accuracy-targeted plan: run to the rounding
-// floor, then keep the prefix the truncation bound asks for.
+// Relative stop threshold of the Cholesky of an accuracy-targeted plan: down to the rounding
+// floor, unless the truncation bound is met first.
 constexpr double kTargetRelTol = 1e-18;
+constexpr int64_t kFirstRank = 64;
 
 // Steps whose T and H are smooth away from the diagonal, as the hierarchical product needs: every
 // T o H step of a parameter change below one (Cases 2 and 3), and Legendre / Chebyshev.  A
@@ -201,24 +202,31 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
         int64_t kcap = std::min<int64_t>(kmax, n - st.j0);
         double* ubig = nullptr;
         TDH_TRY(dev_alloc_t(&st.piv, (size_t)kcap));
-        TDH_TRY(dev_alloc_t(&ubig, (size_t)kcap * n));
         int64_t K = 0;
         // accuracy-targeted plans pivot on the congruent W H W, w_j = sqrt(|D1_j D2_j|): the
         // same A (D1 W^-1 (T o W H W) W^-1 D2), with the greedy step chasing the residual the
         // output error weighs; the factors are converted back to factors of H (u_r / w)
-        double* w = nullptr;
+        double* w = nullptr;  // weights, then the truncation bound's arrays
         int rc = TDH_OK;
+        PcholTarget goal{};
         if (target) {
-            rc = dev_alloc_t(&w, (size_t)n);
+            rc = dev_alloc_t(&w, (size_t)(3 * n + 1));
+            goal = PcholTarget{w + n, w + 2 * n, w + 3 * n, tol};
             if (rc == TDH_OK)
-                rc = pchol_weights(st.d1, st.d2, st.scale_out, st.scale_in, n, w, s);
+                rc = pchol_weights(st.t, st.d1, st.d2, st.scale_out, st.scale_in, n, st.j0, w,
+                                   w + n, w + 2 * n, w + 3 * n, s);
         }
-        if (rc == TDH_OK)
-            rc = pchol_run(st.h, w, n, st.j0, target ? kTargetRelTol : tol, kcap, ubig, st.piv,
-                           &K, s);
-        if (rc == TDH_OK && target && K > 0)
-            rc = pchol_truncate(st.h, w, ubig, n, st.j0, K, st.t, st.d1, st.d2, st.scale_out,
-                                st.scale_in, tol, &K, nullptr, s);
+        // room for kFirstRank terms first (no plan of the common kinds needs more); a run that
+        // fills it starts again with all of kcap
+        for (int64_t cap = std::min(kcap, kFirstRank); rc == TDH_OK; cap = kcap) {
+            dev_free(ubig);
+            ubig = nullptr;
+            rc = dev_alloc_t(&ubig, (size_t)(cap * n));
+            if (rc == TDH_OK)
+                rc = pchol_run(st.h, w, n, st.j0, target ? kTargetRelTol : tol, cap,
+                               target ? &goal : nullptr, ubig, st.piv, &K, s);
+            if (K < cap || cap == kcap) break;
+        }
         if (rc == TDH_OK && target && K > 0) rc = pchol_unweight(ubig, w, K, n, s);
         if (w) {
             cudaStreamSynchronize(s);

@@ -38,77 +38,101 @@ struct State {
     int done;
 };
 
+// What a block publishes of its slice after a step: the largest residual diagonal entry and,
+// for accuracy-targeted runs, the factors of the truncation bound.
+struct Part {
+    ArgMax best;
+    double b1, b2;  // max |D1_j| sqrt(d_j) / w_j, max |D2_j| sqrt(d_j) / w_j
+};
+
+// Accuracy target of a run (a1 null: none): a1_j = |D1_j| / w_j, a2_j = |D2_j| / w_j (with the
+// step's scalings), tmax = max |t|.
+struct TargetSpec {
+    const double* a1;
+    const double* a2;
+    const double* tmax;
+    double target;
+};
+
 __device__ __forceinline__ ArgMax amax(ArgMax a, ArgMax b) {
     return (b.v > a.v || (b.v == a.v && b.i < a.i)) ? b : a;
 }
 
-__device__ ArgMax block_argmax(ArgMax x) {
-    __shared__ double sv[kThreads / 32];
-    __shared__ int64_t si[kThreads / 32];
+__device__ __forceinline__ Part pmax(Part a, Part b) {
+    return Part{amax(a.best, b.best), fmax(a.b1, b.b1), fmax(a.b2, b.b2)};
+}
+
+// The block's maximum, the same in every thread.
+__device__ Part block_max(Part x) {
+    __shared__ Part s[kThreads / 32];
     for (int off = 16; off > 0; off >>= 1) {
-        ArgMax o;
-        o.v = __shfl_down_sync(0xffffffffu, x.v, off);
-        o.i = __shfl_down_sync(0xffffffffu, x.i, off);
-        x = amax(x, o);
+        Part o;
+        o.best.v = __shfl_xor_sync(0xffffffffu, x.best.v, off);
+        o.best.i = __shfl_xor_sync(0xffffffffu, x.best.i, off);
+        o.b1 = __shfl_xor_sync(0xffffffffu, x.b1, off);
+        o.b2 = __shfl_xor_sync(0xffffffffu, x.b2, off);
+        x = pmax(x, o);
     }
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) {
-        sv[w] = x.v;
-        si[w] = x.i;
-    }
+    __syncthreads();  // earlier readers of s are done
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = x;
     __syncthreads();
-    if (w == 0) {
-        x.v = (l < kThreads / 32) ? sv[l] : -INFINITY;
-        x.i = (l < kThreads / 32) ? si[l] : INT64_MAX;
-        for (int off = 16; off > 0; off >>= 1) {
-            ArgMax o;
-            o.v = __shfl_down_sync(0xffffffffu, x.v, off);
-            o.i = __shfl_down_sync(0xffffffffu, x.i, off);
-            x = amax(x, o);
-        }
-        if (l == 0) {
-            sv[0] = x.v;
-            si[0] = x.i;
-        }
-    }
-    __syncthreads();
-    ArgMax r{sv[0], si[0]};
-    __syncthreads();
+    Part r = s[0];
+    for (int w = 1; w < kThreads / 32; ++w) r = pmax(r, s[w]);
     return r;
 }
 
-// d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf); publish block argmax.
+__device__ __forceinline__ Part part_none() {
+    return Part{ArgMax{-INFINITY, INT64_MAX}, 0.0, 0.0};
+}
+
+// Entry j's share of the block's maxima, residual diagonal dj (j >= j0).
+__device__ __forceinline__ Part part_of(const TargetSpec& T, int64_t j, double dj, bool in) {
+    Part p{ArgMax{dj, j}, 0.0, 0.0};
+    if (T.a1 && in) {
+        const double sq = sqrt(fmax(dj, 0.0));
+        p.b1 = T.a1[j] * sq;
+        p.b2 = T.a2[j] * sq;
+    }
+    return p;
+}
+
+// d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf); publish the block's maxima.
 __global__ void __launch_bounds__(kThreads) pchol_init(const double* __restrict__ h, int64_t n,
                                                        int64_t j0, const double* __restrict__ w,
-                                                       double* __restrict__ d,
-                                                       ArgMax* __restrict__ part) {
-    ArgMax best{-INFINITY, INT64_MAX};
+                                                       TargetSpec T, double* __restrict__ d,
+                                                       Part* __restrict__ part) {
+    Part best = part_none();
     for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * kThreads) {
         double v = (j >= j0) ? h[2 * j] * (w ? w[j] * w[j] : 1.0) : -INFINITY;
         d[j] = v;
-        best = amax(best, ArgMax{v, j});
+        best = pmax(best, part_of(T, j, v, j >= j0));
     }
-    best = block_argmax(best);
+    best = block_max(best);
     if (threadIdx.x == 0) part[blockIdx.x] = best;
 }
 
+// One step.  Latency-bound: at most a few hundred KB move.  The column's dot products read the
+// earlier factors kBatch at a time (independent loads in flight), and subtract in order.
+constexpr int kBatch = 8;
+
 __global__ void __launch_bounds__(kThreads) pchol_step(
     const double* __restrict__ h, int64_t n, int64_t j0, const double* __restrict__ w, double tol,
-    int r, double* __restrict__ u, int64_t* __restrict__ piv, double* __restrict__ d,
-    const ArgMax* __restrict__ part_in, ArgMax* __restrict__ part_out, int nparts,
+    TargetSpec T, int r, double* __restrict__ u, int64_t* __restrict__ piv, double* __restrict__ d,
+    const Part* __restrict__ part_in, Part* __restrict__ part_out, int nparts,
     State* __restrict__ st) {
     __shared__ double s_up[kKmaxShared];
     __shared__ double s_a;
     if (st->done) return;
     // every block reduces the same partials: identical pivot and decision everywhere
-    ArgMax best{-INFINITY, INT64_MAX};
-    for (int i = threadIdx.x; i < nparts; i += kThreads) best = amax(best, part_in[i]);
-    best = block_argmax(best);
-    double thresh = (r == 0) ? tol * best.v : st->thresh;
+    Part best = part_none();
+    for (int i = threadIdx.x; i < nparts; i += kThreads) best = pmax(best, part_in[i]);
+    best = block_max(best);
+    double thresh = (r == 0) ? tol * best.best.v : st->thresh;
     if (r == 0 && blockIdx.x == 0 && threadIdx.x == 0) st->thresh = thresh;
-    const int64_t p = best.i;
-    if (!(best.v > thresh) || p < j0 || p >= n) {
+    const int64_t p = best.best.i;
+    const bool met = T.a1 && *T.tmax * best.b1 * best.b2 <= T.target;
+    if (met || !(best.best.v > thresh) || p < j0 || p >= n) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             st->K = r;
             st->done = 1;
@@ -133,7 +157,7 @@ __global__ void __launch_bounds__(kThreads) pchol_step(
         return;
     }
     const double inv = 1.0 / sqrt(a);
-    ArgMax nb{-INFINITY, INT64_MAX};
+    Part nb = part_none();
     double* ur = u + (int64_t)r * n;
     for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * kThreads) {
@@ -141,15 +165,24 @@ __global__ void __launch_bounds__(kThreads) pchol_step(
         double dj = -INFINITY;
         if (j >= j0) {
             double c = h[j + p] * (w ? w[j] * wp : 1.0);
-            for (int i = 0; i < r; ++i) c -= u[(int64_t)i * n + j] * s_up[i];
+            const double* uj = u + j;
+            int i = 0;
+            for (; i + kBatch <= r; i += kBatch) {
+                double v[kBatch];
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) v[b] = uj[(int64_t)(i + b) * n];
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) c -= v[b] * s_up[i + b];
+            }
+            for (; i < r; ++i) c -= uj[(int64_t)i * n] * s_up[i];
             val = c * inv;
             dj = d[j] - val * val;
             d[j] = dj;
         }
         ur[j] = val;
-        nb = amax(nb, ArgMax{dj, j});
+        nb = pmax(nb, part_of(T, j, dj, j >= j0));
     }
-    nb = block_argmax(nb);
+    nb = block_max(nb);
     if (threadIdx.x == 0) part_out[blockIdx.x] = nb;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         piv[r] = p;
@@ -159,41 +192,53 @@ __global__ void __launch_bounds__(kThreads) pchol_step(
 
 }  // namespace
 
+namespace {
+
+// The steps of a factorisation on stream s: state, residual diagonal and partials given.
+cudaError_t pchol_steps(const double* h, const double* w, int64_t n, int64_t j0, double tol,
+                        int64_t kmax, const TargetSpec& T, double* u, int64_t* pivots, double* d,
+                        Part* part, int nblk, State* st, State* host, cudaStream_t s) {
+    *host = State{0.0, 0, 0};
+    cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
+    if (e == cudaSuccess) {
+        pchol_init<<<nblk, kThreads, 0, s>>>(h, n, j0, w, T, d, part);
+        e = cudaGetLastError();
+    }
+    for (int64_t r = 0; e == cudaSuccess && r < kmax; ++r) {
+        pchol_step<<<nblk, kThreads, 0, s>>>(h, n, j0, w, tol, T, (int)r, u, pivots, d,
+                                             part + (r & 1) * nblk, part + ((r + 1) & 1) * nblk,
+                                             nblk, st);
+        e = cudaGetLastError();
+        if (e == cudaSuccess && ((r & 7) == 7 || r + 1 == kmax)) {
+            e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e == cudaSuccess && host->done) break;
+        }
+    }
+    return e;
+}
+
+}  // namespace
+
 int pchol_run(const double* h, const double* w, int64_t n, int64_t j0, double tol, int64_t kmax,
-              double* u, int64_t* pivots, int64_t* K, cudaStream_t s) {
+              const PcholTarget* target, double* u, int64_t* pivots, int64_t* K, cudaStream_t s) {
     if (kmax > kKmaxShared) kmax = kKmaxShared;
     if (kmax > n - j0) kmax = n - j0;
     int nblk = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 4 * (int64_t)sm_count());
     if (nblk < 1) nblk = 1;
     double* d = nullptr;
-    ArgMax* part = nullptr;
+    Part* part = nullptr;
     State* st = nullptr;
     int rc = TDH_OK;
     State host{0.0, 0, 0};
+    TargetSpec T{};
+    if (target) T = TargetSpec{target->a1, target->a2, target->tmax, target->tol};
     if ((rc = dev_alloc_t(&d, (size_t)n)) != TDH_OK) goto done;
     if ((rc = dev_alloc_t(&part, (size_t)2 * nblk)) != TDH_OK) goto done;
     if ((rc = dev_alloc_t(&st, 1)) != TDH_OK) goto done;
     {
-        cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
-        if (e == cudaSuccess) {
-            pchol_init<<<nblk, kThreads, 0, s>>>(h, n, j0, w, d, part);
-            e = cudaGetLastError();
-        }
-        for (int64_t r = 0; e == cudaSuccess && r < kmax; ++r) {
-            pchol_step<<<nblk, kThreads, 0, s>>>(h, n, j0, w, tol, (int)r, u, pivots, d,
-                                                 part + (r & 1) * nblk,
-                                                 part + ((r + 1) & 1) * nblk, nblk, st);
-            e = cudaGetLastError();
-            if (e == cudaSuccess && ((r & 7) == 7 || r + 1 == kmax)) {
-                e = cudaMemcpyAsync(&host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-                if (e == cudaSuccess && host.done) break;
-            }
-        }
-        if (e == cudaSuccess) {
-            e = cudaMemcpyAsync(&host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        }
+        const cudaError_t e =
+            pchol_steps(h, w, n, j0, tol, kmax, T, u, pivots, d, part, nblk, st, &host, s);
         if (e != cudaSuccess) {
             set_error("pivoted Cholesky: %s", cudaGetErrorString(e));
             rc = TDH_ERR_CUDA;
@@ -214,58 +259,32 @@ done:
 // 2 x 2 principal minor gives |R_jk| <= sqrt(d_j d_k) with d = diag(R).  In A = D1 (T o H) D2
 // the truncation error is then |(A - A_K)_jk| <= max|t| |D1_j| sqrt(d_j) |D2_k| sqrt(d_k), and
 // max |beta_K - beta| <= B(K) ||alpha||_1 with B(K) = max|t| max_j |D1_j| sqrt(d_j)
-// max_k |D2_k| sqrt(d_k).  One pass over j evaluates B for every prefix K' <= K.
+// max_k |D2_k| sqrt(d_k).  A run with a target stops at the first K whose B(K) meets it: every
+// step publishes B's two maxima beside the next pivot, so the steps beyond K, up to the rounding
+// floor, are never taken (128 steps and 3.7 ms at n = 1024 where 11 are kept).
 namespace {
 
-// Non-negative doubles order like their bit patterns: atomicMax on the bits.
-__device__ __forceinline__ void atomic_max_nonneg(unsigned long long* m, double v) {
-    atomicMax(m, (unsigned long long)__double_as_longlong(v));
-}
-
-__device__ __forceinline__ double warp_max(double v) {
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-    return v;
-}
-
-// m[0] = max|t|; m[1 + k] = max_j |D1_j| sqrt(d_j^(k)), m[2 + K + k] = max_j |D2_j| sqrt(d_j^(k))
-// for k = 0..K (d^(k): residual diagonal after k steps, indices j >= j0).
-__global__ void __launch_bounds__(kThreads) k_trunc_bound(
-    const double* __restrict__ h, const double* __restrict__ u, int64_t n, int64_t j0, int K,
+// w_j = sqrt(|D1_j D2_j|) (with the step's scalings), 1 where that is 0 or not finite; a1_j =
+// |D1_j| / w_j, a2_j = |D2_j| / w_j (0 for j < j0); *tmax = max |t_j| (cleared before the
+// launch; non-negative doubles order like their bit patterns).
+__global__ void __launch_bounds__(kThreads) k_pivot_weights(
     const double* __restrict__ t, const double* __restrict__ d1, const double* __restrict__ d2,
-    const double* __restrict__ so, const double* __restrict__ si, const double* __restrict__ w,
-    unsigned long long* __restrict__ m) {
+    const double* __restrict__ so, const double* __restrict__ si, int64_t n, int64_t j0,
+    double* __restrict__ w, double* __restrict__ a1, double* __restrict__ a2,
+    unsigned long long* __restrict__ tmax) {
     const int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    const bool in = j < n;
-    const bool blk = in && j >= j0;
-    const int lane = threadIdx.x & 31;
-    const double tm = warp_max(in ? fabs(t[j]) : 0.0);
-    if (lane == 0) atomic_max_nonneg(&m[0], tm);
-    const double wj = (blk && w) ? w[j] : 1.0;
-    const double a1 = blk ? fabs(d1[j] * (so ? so[j] : 1.0)) / wj : 0.0;
-    const double a2 = blk ? fabs(d2[j] * (si ? si[j] : 1.0)) / wj : 0.0;
-    double dj = blk ? h[2 * j] * wj * wj : 0.0;
-    for (int k = 0; k <= K; ++k) {
-        const double sq = sqrt(fmax(dj, 0.0));
-        const double v1 = warp_max(a1 * sq), v2 = warp_max(a2 * sq);
-        if (lane == 0) {
-            atomic_max_nonneg(&m[1 + k], v1);
-            atomic_max_nonneg(&m[2 + K + k], v2);
-        }
-        if (k < K && blk) {
-            const double x = u[(int64_t)k * n + j];
-            dj -= x * x;
-        }
+    double tm = 0.0;
+    if (j < n) {
+        const double x1 = fabs(d1[j] * (so ? so[j] : 1.0)), x2 = fabs(d2[j] * (si ? si[j] : 1.0));
+        const double v = sqrt(fabs(d1[j] * (so ? so[j] : 1.0) * d2[j] * (si ? si[j] : 1.0)));
+        const double wj = (v > 0.0 && isfinite(v)) ? v : 1.0;
+        w[j] = wj;
+        a1[j] = j >= j0 ? x1 / wj : 0.0;
+        a2[j] = j >= j0 ? x2 / wj : 0.0;
+        tm = fabs(t[j]);
     }
-}
-
-// w_j = sqrt(|D1_j D2_j|) (with the step's scalings), 1 where that is 0 or not finite.
-__global__ void k_pivot_weights(const double* __restrict__ d1, const double* __restrict__ d2,
-                                const double* __restrict__ so, const double* __restrict__ si,
-                                int64_t n, double* __restrict__ w) {
-    const int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (j >= n) return;
-    const double v = sqrt(fabs(d1[j] * (so ? so[j] : 1.0) * d2[j] * (si ? si[j] : 1.0)));
-    w[j] = (v > 0.0 && isfinite(v)) ? v : 1.0;
+    for (int off = 16; off > 0; off >>= 1) tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, off));
+    if ((threadIdx.x & 31) == 0) atomicMax(tmax, (unsigned long long)__double_as_longlong(tm));
 }
 
 // u[r][j] /= w_j: factors of W H W -> factors of H
@@ -277,10 +296,12 @@ __global__ void k_unweight(double* __restrict__ u, const double* __restrict__ w,
 
 }  // namespace
 
-int pchol_weights(const double* d1, const double* d2, const double* so, const double* si,
-                  int64_t n, double* w, cudaStream_t s) {
-    k_pivot_weights<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(d1, d2, so, si,
-                                                                                  n, w);
+int pchol_weights(const double* t, const double* d1, const double* d2, const double* so,
+                  const double* si, int64_t n, int64_t j0, double* w, double* a1, double* a2,
+                  double* tmax, cudaStream_t s) {
+    TDH_CUDA(cudaMemsetAsync(tmax, 0, sizeof(double), s));
+    k_pivot_weights<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+        t, d1, d2, so, si, n, j0, w, a1, a2, reinterpret_cast<unsigned long long*>(tmax));
     TDH_CUDA(cudaGetLastError());
     return TDH_OK;
 }
@@ -289,48 +310,6 @@ int pchol_unweight(double* u, const double* w, int64_t K, int64_t n, cudaStream_
     if (K <= 0) return TDH_OK;
     k_unweight<<<(unsigned)((K * n + kThreads - 1) / kThreads), kThreads, 0, s>>>(u, w, K, n);
     TDH_CUDA(cudaGetLastError());
-    return TDH_OK;
-}
-
-int pchol_truncate(const double* h, const double* w, const double* u, int64_t n, int64_t j0,
-                   int64_t K, const double* t, const double* d1, const double* d2,
-                   const double* so, const double* si, double target, int64_t* Kout,
-                   double* bound, cudaStream_t s) {
-    *Kout = K;
-    if (K <= 0) return TDH_OK;
-    const size_t words = 2 * (size_t)K + 3;
-    unsigned long long* m = nullptr;
-    TDH_TRY(dev_alloc_t(&m, words));
-    std::vector<unsigned long long> host(words);
-    cudaError_t e = cudaMemsetAsync(m, 0, sizeof(unsigned long long) * words, s);
-    if (e == cudaSuccess) {
-        const unsigned blocks = (unsigned)((n + kThreads - 1) / kThreads);
-        k_trunc_bound<<<blocks, kThreads, 0, s>>>(h, u, n, j0, (int)K, t, d1, d2, so, si, w, m);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(host.data(), m, sizeof(unsigned long long) * words,
-                            cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    dev_free(m);
-    if (e != cudaSuccess) {
-        set_error("truncation bound: %s", cudaGetErrorString(e));
-        return TDH_ERR_CUDA;
-    }
-    auto as_d = [&](size_t i) {
-        double v;
-        std::memcpy(&v, &host[i], sizeof(double));
-        return v;
-    };
-    const double tmax = as_d(0);
-    for (int64_t k = 0; k <= K; ++k) {
-        const double b = tmax * as_d(1 + (size_t)k) * as_d(2 + (size_t)K + (size_t)k);
-        if (bound) *bound = b;
-        if (b <= target) {
-            *Kout = k;
-            return TDH_OK;
-        }
-    }
     return TDH_OK;
 }
 
@@ -344,7 +323,8 @@ extern "C" int tdh_pchol(const double* h, int64_t n, int64_t j0, double tol, int
         tdh::set_error("tdh_pchol: need n >= 1, j0 in {0,1} < n, tol > 0, kmax >= 1, non-NULL");
         return TDH_ERR_INVALID_ARG;
     }
-    return tdh::pchol_run(h, nullptr, n, j0, tol, kmax, u, pivots, K, tdh::as_stream(stream));
+    return tdh::pchol_run(h, nullptr, n, j0, tol, kmax, nullptr, u, pivots, K,
+                          tdh::as_stream(stream));
 }
 
 // ----------------------------------------------------------------------------------------
@@ -370,7 +350,7 @@ namespace {
 constexpr int64_t kNoAllocMaxN = 65536;
 constexpr int kNoAllocMaxParts = (int)((kNoAllocMaxN + kThreads - 1) / kThreads);
 constexpr size_t kNoAllocDBytes = sizeof(double) * (size_t)kNoAllocMaxN;
-constexpr size_t kNoAllocPartBytes = sizeof(ArgMax) * 2 * (size_t)kNoAllocMaxParts;
+constexpr size_t kNoAllocPartBytes = sizeof(Part) * 2 * (size_t)kNoAllocMaxParts;
 constexpr size_t kNoAllocBytes = kNoAllocDBytes + kNoAllocPartBytes + 256;
 
 static __device__ __align__(256) unsigned char g_pchol_scratch[kNoAllocBytes];
@@ -408,7 +388,7 @@ extern "C" int tdh_pchol_noalloc(const double* h, int64_t n, int64_t j0, double 
     TDH_TRY(noalloc_scratch(&base));
     cudaStream_t s = as_stream(stream);
     double* d = reinterpret_cast<double*>(base);
-    ArgMax* part = reinterpret_cast<ArgMax*>(base + kNoAllocDBytes);
+    Part* part = reinterpret_cast<Part*>(base + kNoAllocDBytes);
     State* st = reinterpret_cast<State*>(base + kNoAllocDBytes + kNoAllocPartBytes);
     if (kmax > kKmaxShared) kmax = kKmaxShared;
     if (kmax > n - j0) kmax = n - j0;
@@ -416,26 +396,8 @@ extern "C" int tdh_pchol_noalloc(const double* h, int64_t n, int64_t j0, double 
     int nblk = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 4 * (int64_t)sm_count());
     if (nblk < 1) nblk = 1;
     State host{0.0, 0, 0};
-    cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
-    if (e == cudaSuccess) {
-        pchol_init<<<nblk, kThreads, 0, s>>>(h, n, j0, nullptr, d, part);
-        e = cudaGetLastError();
-    }
-    for (int64_t r = 0; e == cudaSuccess && r < kmax; ++r) {
-        pchol_step<<<nblk, kThreads, 0, s>>>(h, n, j0, nullptr, tol, (int)r, u, pivots, d,
-                                             part + (r & 1) * nblk, part + ((r + 1) & 1) * nblk,
-                                             nblk, st);
-        e = cudaGetLastError();
-        if (e == cudaSuccess && ((r & 7) == 7 || r + 1 == kmax)) {
-            e = cudaMemcpyAsync(&host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e == cudaSuccess && host.done) break;
-        }
-    }
-    if (e == cudaSuccess) {
-        e = cudaMemcpyAsync(&host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    }
+    const cudaError_t e = pchol_steps(h, nullptr, n, j0, tol, kmax, TargetSpec{}, u, pivots, d, part,
+                                      nblk, st, &host, s);
     if (e != cudaSuccess) {
         set_error("tdh_pchol_noalloc: %s", cudaGetErrorString(e));
         return TDH_ERR_CUDA;
