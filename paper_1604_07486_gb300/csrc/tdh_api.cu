@@ -174,6 +174,7 @@ void release_step(Step& st) {
 // floor, unless the truncation bound is met first.
 constexpr double kTargetRelTol = 1e-18;
 constexpr int64_t kFirstRank = 64;
+constexpr size_t kKeepBytes = (size_t)64 << 20;
 
 // Steps whose T and H are smooth away from the diagonal, as the hierarchical product needs: every
 // T o H step of a parameter change below one (Cases 2 and 3), and Legendre / Chebyshev.  A
@@ -188,11 +189,15 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
     const int64_t n = st.n;
     if (st.sp_M > 0)  // sparse factors: only their tables
         return sparse_prepare(st, prec, s);
-    TDH_TRY(dev_alloc_t(&st.t, n));
-    TDH_TRY(dev_alloc_t(&st.h, 2 * n - 1));
-    TDH_TRY(dev_alloc_t(&st.d1, n));
-    TDH_TRY(dev_alloc_t(&st.d2, n));
-    TDH_TRY(symbols_launch(st.kind, n, st.p, st.t, st.h, st.d1, st.d2, s));
+    TDH_TRY(exec_choose(st, prec));
+    // split-bfloat16 steps run their tensor-core FFT passes
+    const bool hier = hier_serves(st) && !st.ex.g.tc;
+    const int64_t ns = hier ? hier_length(st) : n;
+    TDH_TRY(dev_alloc_t(&st.t, ns));
+    TDH_TRY(dev_alloc_t(&st.h, 2 * ns - 1));
+    TDH_TRY(dev_alloc_t(&st.d1, ns));
+    TDH_TRY(dev_alloc_t(&st.d2, ns));
+    TDH_TRY(symbols_launch(st.kind, ns, st.p, st.t, st.h, st.d1, st.d2, s));
     // row 0 applied directly, Hankel block on indices >= 1: Chebyshev-to-Legendre (Sec. 5.1)
     // and Jacobi Case 3, a + b <= -1 (Sec. 5.3)
     st.j0 = (st.kind == TDH_CHEB2LEG || (st.kind == TDH_JAC2JAC && !(st.p[0] + st.p[1] > -1.0)))
@@ -233,8 +238,12 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
             dev_free(w);
         }
         if (rc == TDH_OK && K > 0) {
-            rc = dev_alloc_t(&st.u64, (size_t)K * n);
-            if (rc == TDH_OK) {
+            if (sizeof(double) * (size_t)(kFirstRank * n) <= kKeepBytes) {
+                std::swap(st.u64, ubig);  // small: kept with its spare rows
+            } else {
+                rc = dev_alloc_t(&st.u64, (size_t)K * n);
+            }
+            if (rc == TDH_OK && ubig) {
                 cudaError_t e = cudaMemcpyAsync(st.u64, ubig, sizeof(double) * K * n,
                                                 cudaMemcpyDeviceToDevice, s);
                 if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -248,10 +257,8 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
         TDH_TRY(rc);
         st.K = K;
     }
-    TDH_TRY(exec_prepare(st, prec, s));
-    // split-bfloat16 steps run their tensor-core FFT passes
-    if (hier_serves(st) && !st.ex.g.tc) return hier_prepare(st, prec, s);
-    return exec_build(st, prec, s);
+    TDH_TRY(exec_diagonals(st, prec, s));
+    return hier ? hier_prepare(st, prec, s) : exec_build(st, prec, s);
 }
 
 void destroy_plan_streams(tdh_plan_s* plan) {

@@ -504,7 +504,7 @@ int launch_typed(const Step& st, const void* in, void* out, int64_t batch, int a
 
 }  // namespace
 
-int exec_prepare(Step& st, int prec, cudaStream_t s) {
+int exec_choose(Step& st, int prec) {
     ExecData& ex = st.ex;
     ex.m = st.full ? st.n : (st.n + 1) / 2;
     int logL = 8;
@@ -514,6 +514,10 @@ int exec_prepare(Step& st, int prec, cudaStream_t s) {
                   (long long)st.n, logL);
         return TDH_ERR_UNSUPPORTED;
     }
+    return TDH_OK;
+}
+
+int exec_diagonals(Step& st, int prec, cudaStream_t s) {
     return prec != TDH_FP64 ? prepare_diagonals<float>(st, s) : prepare_diagonals<double>(st, s);
 }
 

@@ -1180,17 +1180,10 @@ int prepare_typed(Step& st, cudaStream_t s) {
     constexpr int P = HierP<T>::P;
     HierData& H = st.hier;
     const int NC = st.full ? 1 : 2;
-    const int64_t m = (st.n + NC - 1) / NC;
-    H.mpad = (m + kHierTop - 1) / kHierTop * kHierTop;
-    // symbols of the padded length: the boxes at the end reach past n
-    const int64_t N = NC * H.mpad + 2;
-    double* sym = nullptr;  // t[N], h[2N-1], d1[N], d2[N]
-    TDH_TRY(dev_alloc_t(&sym, (size_t)(5 * N)));
+    H.mpad = (hier_length(st) - 2) / NC;
     const size_t ns = (size_t)(H.mpad + kHierSZero), nh = (size_t)(2 * H.mpad + kHierHPad);
     const size_t nw = (size_t)P * kHierLeaf + 12 * P * P;
     int rc = dev_alloc(&H.tab, sizeof(T) * (ns + 2 * nh + nw));
-    if (rc == TDH_OK)
-        rc = symbols_launch(st.kind, N, st.p, sym, sym + N, sym + 3 * N, sym + 4 * N, s);
     std::vector<T> w(nw);
     if (rc == TDH_OK) {
         T* tab = static_cast<T*>(H.tab);
@@ -1200,7 +1193,7 @@ int prepare_typed(Step& st, cudaStream_t s) {
         H.w = tab + ns + 2 * nh;
         const int64_t cnt = 2 * H.mpad + kHierHPad;
         k_hier_tables<T><<<(unsigned)((cnt + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-            sym, sym + N, H.mpad, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
+            st.t, st.h, H.mpad, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
             static_cast<T*>(H.hr));
         int x[kHierLevels][P];
         for (int l = 0; l < kHierLevels; ++l)
@@ -1223,7 +1216,6 @@ int prepare_typed(Step& st, cudaStream_t s) {
             rc = TDH_ERR_CUDA;
         }
     }
-    dev_free(sym);
     if (rc == TDH_OK) H.on = H.use = 1;
     H.use_ragged = H.use && NC == 2;
     return rc;
@@ -1545,6 +1537,13 @@ int ragged_typed(const Step& st, const void* in, void* out, const int64_t* offs,
 }
 
 }  // namespace
+
+// The boxes at the end reach past n: whole 2048-boxes per channel.
+int64_t hier_length(const Step& st) {
+    const int NC = st.full ? 1 : 2;
+    const int64_t m = (st.n + NC - 1) / NC;
+    return NC * ((m + kHierTop - 1) / kHierTop * kHierTop) + 2;
+}
 
 int hier_prepare(Step& st, int prec, cudaStream_t s) {
     return prec != TDH_FP64 ? prepare_typed<float>(st, s) : prepare_typed<double>(st, s);

@@ -179,6 +179,7 @@ struct Step {
     // diag(scale_in) (float64 device arrays of n entries, owned by the step, may be null)
     double* scale_out = nullptr;
     double* scale_in = nullptr;
+    // symbols: of n coefficients, or of the hierarchical product's padded length
     double* t = nullptr;   // [n]
     double* h = nullptr;   // [2n-1]
     double* d1 = nullptr;  // [n]
@@ -238,8 +239,9 @@ int gamma_ratio_launch(double a, double b, int64_t count, double* out, cudaStrea
 // P_k^(-1/2,-1/2)(1) = Gamma(k+1/2)/(Gamma(1/2) Gamma(k+1)), k < n (its reciprocal if
 // `inverse`), float64 device array: T_k = P_k^(-1/2,-1/2) / P_k^(-1/2,-1/2)(1).
 int chebyshev_scale_launch(int64_t n, int inverse, double* out, cudaStream_t s);
-// Choose the FFT geometry of `st` for precision `prec` and build its diagonals.
-int exec_prepare(Step& st, int prec, cudaStream_t s);
+// Choose the FFT geometry of `st` for precision `prec`; build its diagonals.
+int exec_choose(Step& st, int prec);
+int exec_diagonals(Step& st, int prec, cudaStream_t s);
 // The tables of its FFT configurations (spectrum, twiddles, factors) that are not there yet:
 // at creation for steps that run their FFTs, else when a schedule is asked for.
 int exec_build(Step& st, int prec, cudaStream_t s);
@@ -252,6 +254,7 @@ int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, cons
                        const std::vector<cudaEvent_t>& ev);
 // Hierarchical product: tables of a step it serves (hier.on says whether it does), dense and
 // ragged executes.  in and out must not overlap.
+int64_t hier_length(const Step& st);  // coefficients its symbols cover
 int hier_prepare(Step& st, int prec, cudaStream_t s);
 void hier_release(HierData& h);
 int hier_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,

@@ -9,11 +9,12 @@
 // <= tol * max(diag H).  u_r = l_r / sqrt(a_r) in the paper's notation, so
 // H ~ sum_r l_r l_r^T / a_r = sum_r u_r u_r^T.
 //
-// One launch per step over a grid of blocks; each block owns a fixed slice of indices and
-// also publishes the argmax of its slice of the updated d, which every block of the next
-// step reduces (a few hundred entries) to find the next pivot.  Every block takes the same
-// stop decision from the same data, so no grid-wide wait is needed.  The host reads the
-// "done" flag every few steps and stops launching.
+// One cooperative launch for all steps: every block owns a fixed slice of indices and after each
+// step publishes the argmax of its slice of the updated d; a grid-wide barrier later every block
+// reduces the few hundred entries to the next pivot and takes the same stop decision from the
+// same data.  Latency-bound: a step is two barriers' worth of dependent loads (one launch per
+// step, with the host reading a stop flag every eight, took about 19 us a step at n = 2^16; the
+// barrier's waits are bounded, and a wait that ran out is reported as an error).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -27,26 +28,26 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kKmaxShared = 1024;  // u_i[p] for i < r staged in shared memory
 
-struct ArgMax {
-    double v;
-    int64_t i;
-};
-
 struct State {
-    double thresh;  // tol * d0
-    int64_t K;      // steps taken so far
-    int done;
+    int64_t K;      // steps taken
+    int done;       // stopped before the last step it may take, or by its target
+    int timeout;    // a barrier's wait ran out
+    unsigned count; // the barrier
 };
 
-// What a block publishes of its slice after a step: the largest residual diagonal entry and,
-// for accuracy-targeted runs, the factors of the truncation bound.
+// What a block publishes of its slice after a step: the largest residual diagonal entry (its
+// value as an ordered integer, the lowest index on ties) and, for accuracy-targeted runs, the
+// factors of the truncation bound as bit patterns.  All comparisons are integer ones: a float64
+// comparison takes the SM's two float64 lanes sixteen cycles a warp, and the reductions need
+// hundreds of them.
 struct Part {
-    ArgMax best;
-    double b1, b2;  // max |D1_j| sqrt(d_j) / w_j, max |D2_j| sqrt(d_j) / w_j
+    int64_t key;
+    int64_t i;
+    int64_t b1, b2;  // max (D1_j / w_j)^2 d_j, max (D2_j / w_j)^2 d_j (not below 0)
 };
 
-// Accuracy target of a run (a1 null: none): a1_j = |D1_j| / w_j, a2_j = |D2_j| / w_j (with the
-// step's scalings), tmax = max |t|.
+// Accuracy target of a run (a1 null: none): a1_j = (D1_j / w_j)^2, a2_j = (D2_j / w_j)^2 (with
+// the step's scalings), tmax = max |t|.
 struct TargetSpec {
     const double* a1;
     const double* a2;
@@ -54,139 +55,196 @@ struct TargetSpec {
     double target;
 };
 
-__device__ __forceinline__ ArgMax amax(ArgMax a, ArgMax b) {
-    return (b.v > a.v || (b.v == a.v && b.i < a.i)) ? b : a;
+// Doubles in the order of signed integers (NaN below everything), and back.
+__device__ __forceinline__ int64_t order_key(double v) {
+    const int64_t b = __double_as_longlong(v);
+    return v == v ? b ^ ((b >> 63) & INT64_MAX) : INT64_MIN;
+}
+__device__ __forceinline__ double order_value(int64_t k) {
+    return __longlong_as_double(k ^ ((k >> 63) & INT64_MAX));
 }
 
 __device__ __forceinline__ Part pmax(Part a, Part b) {
-    return Part{amax(a.best, b.best), fmax(a.b1, b.b1), fmax(a.b2, b.b2)};
+    const bool second = b.key > a.key || (b.key == a.key && b.i < a.i);
+    Part r;
+    r.key = second ? b.key : a.key;
+    r.i = second ? b.i : a.i;
+    r.b1 = b.b1 > a.b1 ? b.b1 : a.b1;
+    r.b2 = b.b2 > a.b2 ? b.b2 : a.b2;
+    return r;
 }
 
-// The block's maximum, the same in every thread.
-__device__ Part block_max(Part x) {
-    __shared__ Part s[kThreads / 32];
+__device__ __forceinline__ Part part_none() { return Part{INT64_MIN, INT64_MAX, 0, 0}; }
+
+__device__ __forceinline__ Part warp_max(Part x) {
     for (int off = 16; off > 0; off >>= 1) {
         Part o;
-        o.best.v = __shfl_xor_sync(0xffffffffu, x.best.v, off);
-        o.best.i = __shfl_xor_sync(0xffffffffu, x.best.i, off);
+        o.key = __shfl_xor_sync(0xffffffffu, x.key, off);
+        o.i = __shfl_xor_sync(0xffffffffu, x.i, off);
         o.b1 = __shfl_xor_sync(0xffffffffu, x.b1, off);
         o.b2 = __shfl_xor_sync(0xffffffffu, x.b2, off);
         x = pmax(x, o);
     }
-    __syncthreads();  // earlier readers of s are done
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = x;
-    __syncthreads();
-    Part r = s[0];
-    for (int w = 1; w < kThreads / 32; ++w) r = pmax(r, s[w]);
-    return r;
-}
-
-__device__ __forceinline__ Part part_none() {
-    return Part{ArgMax{-INFINITY, INT64_MAX}, 0.0, 0.0};
+    return x;
 }
 
 // Entry j's share of the block's maxima, residual diagonal dj (j >= j0).
 __device__ __forceinline__ Part part_of(const TargetSpec& T, int64_t j, double dj, bool in) {
-    Part p{ArgMax{dj, j}, 0.0, 0.0};
-    if (T.a1 && in) {
-        const double sq = sqrt(fmax(dj, 0.0));
-        p.b1 = T.a1[j] * sq;
-        p.b2 = T.a2[j] * sq;
+    Part p{order_key(dj), j, 0, 0};
+    if (T.a1 && in && dj > 0.0) {  // (a negative rounding residue counts as 0)
+        p.b1 = __double_as_longlong(T.a1[j] * dj);
+        p.b2 = __double_as_longlong(T.a2[j] * dj);
     }
     return p;
 }
 
-// d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf); publish the block's maxima.
-__global__ void __launch_bounds__(kThreads) pchol_init(const double* __restrict__ h, int64_t n,
-                                                       int64_t j0, const double* __restrict__ w,
-                                                       TargetSpec T, double* __restrict__ d,
-                                                       Part* __restrict__ part) {
-    Part best = part_none();
-    for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * kThreads) {
-        double v = (j >= j0) ? h[2 * j] * (w ? w[j] * w[j] : 1.0) : -INFINITY;
-        d[j] = v;
-        best = pmax(best, part_of(T, j, v, j >= j0));
+// Grid-wide barrier of a cooperative launch: block 0 ... gridDim.x - 1 count up to gen *
+// gridDim.x.  Returns false when the wait ran out (a second; the other blocks then run out too).
+constexpr long long kBarrierNs = 1000000000ll;
+__device__ __forceinline__ long long global_ns() {
+    long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ bool grid_barrier(unsigned* count, unsigned gen) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(count, 1u);
+        const unsigned goal = gen * gridDim.x;
+        const long long t0 = global_ns();
+        int good = 1;
+        while (*(volatile unsigned*)count < goal) {
+            if (global_ns() - t0 > kBarrierNs) {
+                good = 0;
+                break;
+            }
+        }
+        __threadfence();
+        ok = good;
     }
-    best = block_max(best);
-    if (threadIdx.x == 0) part[blockIdx.x] = best;
+    __syncthreads();
+    return ok != 0;
 }
 
-// One step.  Latency-bound: at most a few hundred KB move.  The column's dot products read the
-// earlier factors kBatch at a time (independent loads in flight), and subtract in order.
+// All steps.  The column's dot products read the earlier factors kBatch at a time (independent
+// loads in flight), and subtract in order.  part: [2][gridDim.x], alternating between steps.
 constexpr int kBatch = 8;
 
-__global__ void __launch_bounds__(kThreads) pchol_step(
+__global__ void __launch_bounds__(kThreads, 2) pchol_all(
     const double* __restrict__ h, int64_t n, int64_t j0, const double* __restrict__ w, double tol,
-    TargetSpec T, int r, double* __restrict__ u, int64_t* __restrict__ piv, double* __restrict__ d,
-    const Part* __restrict__ part_in, Part* __restrict__ part_out, int nparts,
-    State* __restrict__ st) {
+    TargetSpec T, int kmax, double* u, int64_t* __restrict__ piv, double* __restrict__ d,
+    Part* part, State* st) {
     __shared__ double s_up[kKmaxShared];
-    __shared__ double s_a;
-    if (st->done) return;
-    // every block reduces the same partials: identical pivot and decision everywhere
-    Part best = part_none();
-    for (int i = threadIdx.x; i < nparts; i += kThreads) best = pmax(best, part_in[i]);
-    best = block_max(best);
-    double thresh = (r == 0) ? tol * best.best.v : st->thresh;
-    if (r == 0 && blockIdx.x == 0 && threadIdx.x == 0) st->thresh = thresh;
-    const int64_t p = best.best.i;
-    const bool met = T.a1 && *T.tmax * best.b1 * best.b2 <= T.target;
-    if (met || !(best.best.v > thresh) || p < j0 || p >= n) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            st->K = r;
-            st->done = 1;
-        }
-        return;
-    }
-    for (int i = threadIdx.x; i < r; i += kThreads) s_up[i] = u[(int64_t)i * n + p];
-    __syncthreads();
-    const double wp = w ? w[p] : 1.0;
-    if (threadIdx.x == 0) {
-        double a = h[2 * p] * wp * wp;
-        for (int i = 0; i < r; ++i) a -= s_up[i] * s_up[i];
-        s_a = a;
-    }
-    __syncthreads();
-    const double a = s_a;
-    if (!(a > thresh)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            st->K = r;
-            st->done = 1;
-        }
-        return;
-    }
-    const double inv = 1.0 / sqrt(a);
-    Part nb = part_none();
-    double* ur = u + (int64_t)r * n;
+    __shared__ Part s_part[kThreads / 32];
+    __shared__ double s_inv, s_wp;
+    __shared__ int64_t s_p;
+    const int nparts = gridDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    unsigned gen = 0;
+    // d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf)
+    Part own = part_none();
     for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * kThreads) {
-        double val = 0.0;
-        double dj = -INFINITY;
-        if (j >= j0) {
-            double c = h[j + p] * (w ? w[j] * wp : 1.0);
-            const double* uj = u + j;
-            int i = 0;
-            for (; i + kBatch <= r; i += kBatch) {
-                double v[kBatch];
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) v[b] = uj[(int64_t)(i + b) * n];
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) c -= v[b] * s_up[i + b];
-            }
-            for (; i < r; ++i) c -= uj[(int64_t)i * n] * s_up[i];
-            val = c * inv;
-            dj = d[j] - val * val;
-            d[j] = dj;
-        }
-        ur[j] = val;
-        nb = pmax(nb, part_of(T, j, dj, j >= j0));
+        const double v = (j >= j0) ? h[2 * j] * (w ? w[j] * w[j] : 1.0) : -INFINITY;
+        d[j] = v;
+        own = pmax(own, part_of(T, j, v, j >= j0));
     }
-    nb = block_max(nb);
-    if (threadIdx.x == 0) part_out[blockIdx.x] = nb;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        piv[r] = p;
-        st->K = r + 1;
+    double thresh = 0.0;  // warp 0, lane 0
+    for (int r = 0;; ++r) {
+        own = warp_max(own);
+        if (lane == 0) s_part[warp] = own;
+        __syncthreads();
+        Part* pub = part + (r & 1) * nparts;
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < kThreads / 32; ++i) own = pmax(own, s_part[i]);
+            pub[blockIdx.x] = own;
+        }
+        if (!grid_barrier(&st->count, ++gen)) {
+            if (threadIdx.x == 0) st->timeout = 1;
+            return;
+        }
+        // warp 0 of every block reduces the same partials (identical pivot and decision
+        // everywhere), gathers the pivot row of the factors and forms its scale
+        if (warp == 0) {
+            Part best = part_none();
+            for (int i = lane; i < nparts; i += 32) {
+                const volatile Part* q = pub + i;
+                Part o;
+                o.key = q->key;
+                o.i = q->i;
+                o.b1 = q->b1;
+                o.b2 = q->b2;
+                best = pmax(best, o);
+            }
+            best = warp_max(best);
+            const int64_t p = best.i;
+            int stop = 0;  // 1: done, 2: the last step taken
+            if (lane == 0) {
+                const double v = order_value(best.key);
+                if (r == 0) thresh = tol * v;
+                const bool met = T.a1 && *T.tmax * sqrt(__longlong_as_double(best.b1)) *
+                                                 sqrt(__longlong_as_double(best.b2)) <= T.target;
+                if (met || !(v > thresh) || p < j0 || p >= n)
+                    stop = 1;
+                else if (r == kmax)
+                    stop = 2;
+            }
+            stop = __shfl_sync(0xffffffffu, stop, 0);
+            if (!stop) {
+                // (factors of this launch are read past L1, which other SMs' writes do not reach)
+                for (int i = lane; i < r; i += 32) s_up[i] = __ldcg(u + (int64_t)i * n + p);
+                __syncwarp();
+                if (lane == 0) {
+                    const double wp = w ? w[p] : 1.0;
+                    double a = h[2 * p] * wp * wp;
+                    for (int i = 0; i < r; ++i) a -= s_up[i] * s_up[i];
+                    if (!(a > thresh)) stop = 1;
+                    s_wp = wp;
+                    s_inv = 1.0 / sqrt(a);
+                }
+            }
+            if (lane == 0) {
+                s_p = stop ? -1 : p;
+                if (stop && blockIdx.x == 0) {
+                    st->K = r;
+                    st->done = stop == 1;
+                }
+            }
+        }
+        __syncthreads();
+        const int64_t p = s_p;
+        if (p < 0) return;
+        const double inv = s_inv, wp = s_wp;
+        own = part_none();
+        double* ur = u + (int64_t)r * n;
+        for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
+             j += (int64_t)gridDim.x * kThreads) {
+            double val = 0.0;
+            double dj = -INFINITY;
+            if (j >= j0) {
+                double c = h[j + p] * (w ? w[j] * wp : 1.0);
+                const double dold = d[j];
+                const double* uj = u + j;  // this thread's own writes
+                int i = 0;
+                for (; i + kBatch <= r; i += kBatch) {
+                    double v[kBatch];
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b) v[b] = __ldcg(uj + (int64_t)(i + b) * n);
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b) c -= v[b] * s_up[i + b];
+                }
+                for (; i < r; ++i) c -= __ldcg(uj + (int64_t)i * n) * s_up[i];
+                val = c * inv;
+                dj = dold - val * val;
+                d[j] = dj;
+            }
+            ur[j] = val;
+            own = pmax(own, part_of(T, j, dj, j >= j0));
+        }
+        if (lead) piv[r] = p;
     }
 }
 
@@ -198,39 +256,40 @@ namespace {
 cudaError_t pchol_steps(const double* h, const double* w, int64_t n, int64_t j0, double tol,
                         int64_t kmax, const TargetSpec& T, double* u, int64_t* pivots, double* d,
                         Part* part, int nblk, State* st, State* host, cudaStream_t s) {
-    *host = State{0.0, 0, 0};
+    *host = State{};
+    int kk = (int)kmax;
     cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
     if (e == cudaSuccess) {
-        pchol_init<<<nblk, kThreads, 0, s>>>(h, n, j0, w, T, d, part);
-        e = cudaGetLastError();
+        TargetSpec TT = T;
+        void* args[] = {&h, &n, &j0, &w, &tol, &TT, &kk, &u, &pivots, &d, &part, &st};
+        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pchol_all), dim3(nblk),
+                                        dim3(kThreads), args, 0, s);
     }
-    for (int64_t r = 0; e == cudaSuccess && r < kmax; ++r) {
-        pchol_step<<<nblk, kThreads, 0, s>>>(h, n, j0, w, tol, T, (int)r, u, pivots, d,
-                                             part + (r & 1) * nblk, part + ((r + 1) & 1) * nblk,
-                                             nblk, st);
-        e = cudaGetLastError();
-        if (e == cudaSuccess && ((r & 7) == 7 || r + 1 == kmax)) {
-            e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e == cudaSuccess && host->done) break;
-        }
-    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && host->timeout) e = cudaErrorLaunchTimeout;
     return e;
 }
 
 }  // namespace
 
+// Blocks of the launch: all resident at once (two of at most 128 registers a thread per SM).
+int pchol_blocks(int64_t n) {
+    return (int)std::max<int64_t>(
+        1, std::min<int64_t>((n + kThreads - 1) / kThreads, 2 * (int64_t)sm_count()));
+}
+
 int pchol_run(const double* h, const double* w, int64_t n, int64_t j0, double tol, int64_t kmax,
               const PcholTarget* target, double* u, int64_t* pivots, int64_t* K, cudaStream_t s) {
     if (kmax > kKmaxShared) kmax = kKmaxShared;
     if (kmax > n - j0) kmax = n - j0;
-    int nblk = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 4 * (int64_t)sm_count());
-    if (nblk < 1) nblk = 1;
+    const int nblk = pchol_blocks(n);
     double* d = nullptr;
     Part* part = nullptr;
     State* st = nullptr;
     int rc = TDH_OK;
-    State host{0.0, 0, 0};
+    State host{};
     TargetSpec T{};
     if (target) T = TargetSpec{target->a1, target->a2, target->tmax, target->tol};
     if ((rc = dev_alloc_t(&d, (size_t)n)) != TDH_OK) goto done;
@@ -265,7 +324,7 @@ done:
 namespace {
 
 // w_j = sqrt(|D1_j D2_j|) (with the step's scalings), 1 where that is 0 or not finite; a1_j =
-// |D1_j| / w_j, a2_j = |D2_j| / w_j (0 for j < j0); *tmax = max |t_j| (cleared before the
+// (D1_j / w_j)^2, a2_j = (D2_j / w_j)^2 (0 for j < j0); *tmax = max |t_j| (cleared before the
 // launch; non-negative doubles order like their bit patterns).
 __global__ void __launch_bounds__(kThreads) k_pivot_weights(
     const double* __restrict__ t, const double* __restrict__ d1, const double* __restrict__ d2,
@@ -279,8 +338,9 @@ __global__ void __launch_bounds__(kThreads) k_pivot_weights(
         const double v = sqrt(fabs(d1[j] * (so ? so[j] : 1.0) * d2[j] * (si ? si[j] : 1.0)));
         const double wj = (v > 0.0 && isfinite(v)) ? v : 1.0;
         w[j] = wj;
-        a1[j] = j >= j0 ? x1 / wj : 0.0;
-        a2[j] = j >= j0 ? x2 / wj : 0.0;
+        const double r1 = x1 / wj, r2 = x2 / wj;
+        a1[j] = j >= j0 ? r1 * r1 : 0.0;
+        a2[j] = j >= j0 ? r2 * r2 : 0.0;
         tm = fabs(t[j]);
     }
     for (int off = 16; off > 0; off >>= 1) tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, off));
@@ -392,10 +452,9 @@ extern "C" int tdh_pchol_noalloc(const double* h, int64_t n, int64_t j0, double 
     State* st = reinterpret_cast<State*>(base + kNoAllocDBytes + kNoAllocPartBytes);
     if (kmax > kKmaxShared) kmax = kKmaxShared;
     if (kmax > n - j0) kmax = n - j0;
-    // the same grid as tdh_pchol (at most 4 blocks per SM), within the array's partials
-    int nblk = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 4 * (int64_t)sm_count());
-    if (nblk < 1) nblk = 1;
-    State host{0.0, 0, 0};
+    // the same grid as tdh_pchol, within the array's partials
+    const int nblk = pchol_blocks(n);
+    State host{};
     const cudaError_t e = pchol_steps(h, nullptr, n, j0, tol, kmax, TargetSpec{}, u, pivots, d, part,
                                       nblk, st, &host, s);
     if (e != cudaSuccess) {
