@@ -40,6 +40,8 @@ struct HierParams {
     int nseg, seg_leaves, nvt, unvt;  // far segments; vectors per CTA (far, moments)
     T* top;             // 2048-boxes' exchange, [group][ntop][NC][nvt][P] (null: by k_hier_far)
     int ntop;           // 2048-boxes of a vector
+    const T* st;        // s and h at the 2048-boxes' points (k_hier_top)
+    const T* ht;
     int run;            // leaves a warp of the near kernel walks
     int64_t runs;       // such walks per vector group
     const int64_t* offs;  // ragged: vector i of the launch is list[i]
@@ -451,7 +453,9 @@ __device__ __forceinline__ void far_box(const T* sp, const T* hp, const T* m0, i
 
 // Long vectors: the exchange of the 2048-boxes, one CTA per box and NVT vectors, the far boxes
 // split over its warps; to P.top ([group][box][NC][NVT][P]).  (Within k_hier_far every segment
-// of a 2048-box would repeat it: fine for a few boxes, 3/4 of that kernel at 512 of them.)
+// of a 2048-box would repeat it: fine for a few boxes, 3/4 of that kernel at 512 of them.)  The
+// points lie a sector or more apart in s and h, so the factors are read from tables of their
+// own (16 lanes' rows contiguous): 105 -> 44 us at n = 2^20 x 16 float32.
 template <typename T, int NC, int NVT, bool RAGGED>
 __global__ void __launch_bounds__(kThreads) k_hier_top(const __grid_constant__ HierParams<T> P) {
     using F = FarShape<T, NC, NVT>;
@@ -469,18 +473,34 @@ __global__ void __launch_bounds__(kThreads) k_hier_top(const __grid_constant__ H
     const int64_t boxrow = (int64_t)NC * P.bpad * NP;
     const int p = lane % NP, vt = (lane / NP) % VTL, c = lane / (NP * VTL);
     if (c < NC) {
-        int xp = 0;
+        using P2 = typename PairOf<T>::t;
+        const T* st = P.st + p * NP;
+        const T* ht = P.ht + (((int64_t)2 * i * NC + c) * NP + p) * NP;
+        const T* m = P.mom[TOP] + i * boxrow + ((int64_t)c * P.bpad + g0 + vt * VPT) * NP;
+        P2 acc[VPT];  // sums over the even and the odd points
 #pragma unroll
-        for (int q = 0; q < NP; ++q)
-            if (q == p) xp = hier_point<NP>(TOP, q);
-        T acc[VPT];
+        for (int u = 0; u < VPT; ++u) acc[u] = pair_zero(T(0));
+#pragma unroll 1
+        for (int64_t d = 2 + warp; d < nb - i; d += kWarps) {
 #pragma unroll
-        for (int u = 0; u < VPT; ++u) acc[u] = T(0);
-        far_box<T, NC, VPT, TOP>(P.s - xp, P.hh + (int64_t)2 * i * hier_size(TOP) + xp + c,
-                                 P.mom[TOP] + i * boxrow + ((int64_t)c * P.bpad + g0 + vt * VPT) * NP,
-                                 boxrow, 2 + warp, nb - i, kWarps, acc);
+            for (int q = 0; q < NP; q += 4) {
+                P2 s0, s1, h0, h1;
+                pair_load2(reinterpret_cast<const P2*>(st + d * (NP * NP) + q), s0, s1);
+                pair_load2(reinterpret_cast<const P2*>(ht + d * (NC * NP * NP) + q), h0, h1);
+                s0 = pair_mul(s0, h0);
+                s1 = pair_mul(s1, h1);
 #pragma unroll
-        for (int u = 0; u < VPT; ++u) part[warp * erow + (c * NVT + vt * VPT + u) * NP + p] = acc[u];
+                for (int u = 0; u < VPT; ++u) {
+                    P2 y0, y1;
+                    pair_load2(reinterpret_cast<const P2*>(m + d * boxrow + u * NP + q), y0, y1);
+                    pair_fma(acc[u], s0, y0);
+                    pair_fma(acc[u], s1, y1);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < VPT; ++u)
+            part[warp * erow + (c * NVT + vt * VPT + u) * NP + p] = pair_x(acc[u]) + pair_y(acc[u]);
     }
     __syncthreads();
     for (int e = tid; e < erow; e += kThreads) {
@@ -1175,6 +1195,31 @@ __global__ void k_hier_tables(const double* __restrict__ t, const double* __rest
     }
 }
 
+// s at the points of the 2048-boxes, [distance][P][P], then h forward and reversed,
+// [sum of indices][NC][P][P].
+template <typename T>
+__global__ void k_hier_points(const T* __restrict__ s, const T* __restrict__ hf,
+                              const T* __restrict__ hr, int nc, int64_t ns, int64_t nh,
+                              T* __restrict__ out) {
+    constexpr int P = HierP<T>::P, TOP = kHierLevels - 1;
+    __shared__ int x[P];
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int i = 0; i < P; ++i) x[i] = hier_point<P>(TOP, i);
+    __syncthreads();
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (i >= ns + 2 * nh) return;
+    const int xq = x[i % P], xp = x[i / P % P];  // every table is whole [P][P] blocks
+    if (i < ns) {
+        const int64_t at = i / (P * P) * kHierTop + xq - xp;
+        out[i] = at >= 0 ? s[at] : T(0);
+    } else {
+        const bool rev = i >= ns + nh;
+        const int64_t b = (i - ns - (rev ? nh : 0)) / (P * P);
+        out[i] = (rev ? hr : hf)[b / nc * kHierTop + xp + xq + b % nc];
+    }
+}
+
 template <typename T>
 int prepare_typed(Step& st, cudaStream_t s) {
     constexpr int P = HierP<T>::P;
@@ -1183,7 +1228,12 @@ int prepare_typed(Step& st, cudaStream_t s) {
     H.mpad = (hier_length(st) - 2) / NC;
     const size_t ns = (size_t)(H.mpad + kHierSZero), nh = (size_t)(2 * H.mpad + kHierHPad);
     const size_t nw = (size_t)P * kHierLeaf + 12 * P * P;
-    int rc = dev_alloc(&H.tab, sizeof(T) * (ns + 2 * nh + nw));
+    // long vectors: the 2048-boxes' point tables (k_hier_top)
+    const int64_t ntop = H.mpad / kHierTop;
+    const bool top = ntop >= kTopKernel;
+    const int64_t nps = top ? ntop * P * P : 0, nph = top ? (2 * ntop - 1) * NC * P * P : 0;
+    const size_t at = (ns + 2 * nh + nw + 3) / 4 * 4;  // 16-byte aligned
+    int rc = dev_alloc(&H.tab, sizeof(T) * (at + (size_t)(nps + 2 * nph)));
     std::vector<T> w(nw);
     if (rc == TDH_OK) {
         T* tab = static_cast<T*>(H.tab);
@@ -1195,6 +1245,15 @@ int prepare_typed(Step& st, cudaStream_t s) {
         k_hier_tables<T><<<(unsigned)((cnt + kThreads - 1) / kThreads), kThreads, 0, s>>>(
             st.t, st.h, H.mpad, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
             static_cast<T*>(H.hr));
+        if (top) {
+            H.st = tab + at;
+            H.ht[0] = tab + at + nps;
+            H.ht[1] = tab + at + nps + nph;
+            // (reversed full kinds start one entry on, as in run_typed)
+            k_hier_points<T><<<(unsigned)((nps + 2 * nph + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+                static_cast<const T*>(H.s), static_cast<const T*>(H.hf),
+                static_cast<const T*>(H.hr) + (NC == 1 ? 1 : 0), NC, nps, nph, tab + at);
+        }
         int x[kHierLevels][P];
         for (int l = 0; l < kHierLevels; ++l)
             for (int p = 0; p < P; ++p) x[l][p] = hier_point<P>(l, p);
@@ -1396,6 +1455,8 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     P.s = static_cast<const T*>(H.s);
     // reversed: packed index a' + b' meets hf[2 (mpad - 1) - a' - b' (+ 1 in channel 0)]
     P.hh = static_cast<const T*>(adjoint ? H.hr : H.hf) + (adjoint && NC == 1 ? 1 : 0);
+    P.st = static_cast<const T*>(H.st);
+    P.ht = static_cast<const T*>(H.ht[adjoint ? 1 : 0]);
     P.lw = static_cast<const T*>(H.w);
     P.tr = P.lw + NP * kHierLeaf;
     P.din = static_cast<const T*>(adjoint ? st.d1x : st.d2x);

@@ -148,6 +148,8 @@ struct HierData {
     void* hf = nullptr;   // Hankel table, forward
     void* hr = nullptr;   // Hankel table, reversed (transpose)
     void* w = nullptr;    // Lagrange weights: leaf [P][32], then transfers [3][4][P][P]
+    void* st = nullptr;   // long vectors: s at the 2048-boxes' points, [distance][P][P]
+    void* ht[2] = {};     // and h, forward and reversed, [sum of indices][NC][P][P]
 };
 
 // One T o H conversion step of a plan.
