@@ -312,10 +312,13 @@ def precision_comparison(tdh, args, flush, stream, world, rank, n=1 << 20, batch
 
 def dense_arm_bf16x3(tdh, args, alpha, flush, stream, world, rank, rows):
     """Both directions at n = 2^16, batch 256 with the split-bfloat16 tensor-core DFT passes
-    (TDH_BF16X3), tuned, timed like the float32 line; errors against the oracle."""
+    (the tuned FFT schedule of TDH_BF16X3 plans, which run the hierarchical product unless asked
+    for it), timed like the float32 line; errors against the oracle."""
     import torch
     plans = {k: tdh.Plan(k, N, prec="bf16x3") for k in KINDS}
     sched = {k: tune(plans[k], BATCH, args)[1] for k in KINDS}
+    for k in KINDS:
+        plans[k].set_schedule(plans[k].schedules()[0]["index"])
     x = torch.tensor(alpha, dtype=torch.float32, device="cuda")
     y = {k: torch.empty_like(x) for k in KINDS}
     for _ in range(args.warmup):
@@ -342,8 +345,9 @@ def dense_arm_bf16x3(tdh, args, alpha, flush, stream, world, rank, rows):
 
 def ragged_arm_bf16x3(tdh, args, xv, offs, lengths, flops, fp32_peak, apeaks, flush, stream,
                       world, dist, rank):
-    """Config 3's second arm: the same ragged batch with the split-bfloat16 tensor-core DFT
-    passes (TDH_BF16X3), tuned, replayed from one CUDA graph, timed like the float32 arm."""
+    """Config 3's second arm: the same ragged batch with a TDH_BF16X3 plan, tuned (its
+    tensor-core FFT schedules against the hierarchical product), replayed from one CUDA graph,
+    timed like the float32 arm."""
     import numpy as np
     import torch
     import oracle
@@ -393,8 +397,8 @@ def ragged_arm_bf16x3(tdh, args, xv, offs, lengths, flops, fp32_peak, apeaks, fl
                          "unit": "TFLOP/s", "frac": achieved / fp32_peak,
                          "peak_note": "same algorithmic flops as the float32 arm, against the "
                                       "FP32 FFMA " + apeaks["note"]},
-            "note": "radix-16/8 middle FFT passes as split-bfloat16 tcgen05 DFT products; "
-                    "other passes float32"}
+            "note": "the faster of the hierarchical product (float32) and the FFT schedules with "
+                    "split-bfloat16 tcgen05 DFT products, by tdh_plan_autotune"}
 
 
 def workloads_coefficients(n, batch, seed):

@@ -7,11 +7,11 @@
  * H ~ sum_r l_r l_r^T / a_r (Sec. 2.1, Fig. 2); and beta = A alpha is computed as
  * D1 sum_r D_{u_r} T D_{u_r} D2 alpha with u_r = l_r / sqrt(a_r) (Eq. (5)),
  * each Toeplitz product by zero-padded FFTs of length about 2N (Sec. 1).
- * T o H itself is also smooth away from the diagonal, and the float32 and float64 executes use
- * that instead where it holds (every conversion but Laguerre changes of one or more): its far
- * blocks by interpolation in a tree of boxes, its near ones entry by entry, in O(N) operations
- * and without a truncation (the hierarchical product).  The FFT form runs TDH_BF16X3 plans, and
- * any plan whose FFT schedule is asked for (tdh_plan_set_schedule).
+ * T o H itself is also smooth away from the diagonal, and executes use that instead where it
+ * holds (every conversion but Laguerre changes of one or more): its far blocks by interpolation
+ * in a tree of boxes, its near ones entry by entry, in O(N) operations and without a truncation
+ * (the hierarchical product).  The FFT form runs any plan whose FFT schedule is asked for
+ * (tdh_plan_set_schedule) or found the faster one (tdh_plan_autotune).
  *
  * Conventions for every entry point
  *   - Pointers named d_* or documented as "device" are CUDA device pointers on the current
@@ -51,12 +51,13 @@ extern "C" {
 /* ---------------------------------------------------------------- execute precisions */
 #define TDH_FP64  0 /* float64 in/out, float64 FFT                                             */
 #define TDH_FP32  1 /* float32 in/out, float32 FFT (plan factors rounded once from float64)    */
-/* float32 in/out; within one thread-block cluster (FFTs of up to 2^17 points) the radix-16
+/* float32 in/out; steps the hierarchical product serves run it in float32, as TDH_FP32 plans do
+ * (faster than the FFTs below at every length); in the FFT form, within one thread-block cluster (FFTs of up to 2^17 points) the radix-16
  * (radix-8 for short FFTs) middle passes of every FFT run on the tensor cores as DFT matrix
  * products in split bfloat16: each operand x = hi + lo (bfloat16 parts) and the three products
  * hi*hi + lo*hi + hi*lo accumulate in float32 (tcgen05, tensor memory); every other pass and
  * the multi-pass FFTs beyond one cluster are float32.  The split keeps about 16 bits of each
- * operand, so errors are larger than TDH_FP32's.                                              */
+ * operand, so the FFT form's errors are larger than TDH_FP32's.                               */
 #define TDH_BF16X3 2
 
 /* ---------------------------------------------------------------- plan flags */
@@ -342,8 +343,8 @@ int tdh_test_fail_alloc(int64_t k);
 
 /*
  * tdh_test_tc_stall -- failure injection for tests (the paper has no counterpart): while on
- * (on != 0), executes enqueued from then on with TDH_BF16X3 plans issue none of their
- * tensor-core products, so the first bounded wait of every CTA runs out after about one
+ * (on != 0), executes enqueued from then on with TDH_BF16X3 plans run the FFT form (where it has
+ * tensor-core passes) and issue none of their tensor-core products, so the first bounded wait of every CTA runs out after about one
  * second; the kernels then skip their remaining waits, finish, free their tensor memory and
  * record TDH_STATUS_TIMEOUT (tdh_plan_status).  Their outputs are not valid.  The setting is
  * process-wide and read when an execute is enqueued (a captured CUDA graph keeps the value it

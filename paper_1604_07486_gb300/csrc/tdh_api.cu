@@ -190,8 +190,10 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
     if (st.sp_M > 0)  // sparse factors: only their tables
         return sparse_prepare(st, prec, s);
     TDH_TRY(exec_choose(st, prec));
-    // split-bfloat16 steps run their tensor-core FFT passes
-    const bool hier = hier_serves(st) && !st.ex.g.tc;
+    // Whatever the precision and the length: split-bfloat16 plans' tensor-core FFTs take 28 us at
+    // n = 512 x 16 and 3267 us at 65536 x 256, the float32 hierarchical product 9.4 and 161 us with
+    // smaller errors.  Their FFT tables are built with the plan all the same (tdh_test_tc_stall).
+    const bool hier = hier_serves(st);
     const int64_t ns = hier ? hier_length(st) : n;
     TDH_TRY(dev_alloc_t(&st.t, ns));
     TDH_TRY(dev_alloc_t(&st.h, 2 * ns - 1));
@@ -258,7 +260,8 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
         st.K = K;
     }
     TDH_TRY(exec_diagonals(st, prec, s));
-    return hier ? hier_prepare(st, prec, s) : exec_build(st, prec, s);
+    if (hier) TDH_TRY(hier_prepare(st, prec, s));
+    return hier && !st.ex.g.tc ? TDH_OK : exec_build(st, prec, s);
 }
 
 void destroy_plan_streams(tdh_plan_s* plan) {
@@ -747,7 +750,7 @@ int tdh_plan_create(int kind, int64_t n_max, const tdh_params* params, double to
             rc = TDH_ERR_UNSUPPORTED;
         } else {
             rc = exec_prepare_ragged(plan->steps[0], params->prec);
-            if (rc == TDH_OK && !plan->steps[0].hier.use_ragged)
+            if (rc == TDH_OK && (!plan->steps[0].hier.use_ragged || params->prec == TDH_BF16X3))
                 rc = exec_build(plan->steps[0], params->prec, s);
         }
         const size_t ncls = plan->steps.empty() ? 0 : plan->steps[0].rcls.size();

@@ -705,17 +705,26 @@ int launch_ragged_typed(const Step& st, const void* in, void* out, const int64_t
 
 }  // namespace
 
+// While the stall hook is on, split-bfloat16 steps run the tensor-core FFT it stalls (ragged: the
+// length classes').
+static bool tc_stalled(const Step& st) {
+    if (!tc_stall_enabled()) return false;
+    bool tc = st.ex.built && st.ex.g.tc;
+    for (const ExecData& ex : st.rcls) tc = tc || (ex.built && ex.g.tc);
+    return tc;
+}
+
 int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s, const std::vector<cudaStream_t>& side,
                        const std::vector<cudaEvent_t>& ev) {
-    if (st.hier.use_ragged) return hier_launch_ragged(st, prec, in, out, offs, batch, s);
+    if (st.hier.use_ragged && !tc_stalled(st)) return hier_launch_ragged(st, prec, in, out, offs, batch, s);
     if (prec != TDH_FP64) return launch_ragged_typed<float>(st, in, out, offs, batch, s, side, ev);
     return launch_ragged_typed<double>(st, in, out, offs, batch, s, side, ev);
 }
 
 int exec_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
                 cudaStream_t s) {
-    if (st.hier.use) return hier_launch(st, prec, in, out, batch, adjoint, s);
+    if (st.hier.use && !tc_stalled(st)) return hier_launch(st, prec, in, out, batch, adjoint, s);
     return fft_launch(st, prec, in, out, batch, adjoint, s);
 }
 

@@ -124,6 +124,25 @@ def test_ragged_edges(tdh, prec):
     assert plan.status() == set()
 
 
+@pytest.mark.parametrize("n", [5, 1000, 20001])
+def test_bf16x3_plans_run_it_in_float32(tdh, n):
+    """Split-bfloat16 plans: the float32 plan's results bit for bit (dense, transpose, ragged)
+    until an FFT schedule is set, whose results differ and stay within the stated tolerance."""
+    import torch
+    a = tdh.Plan("leg2cheb", n, prec="bf16x3", ragged=True)
+    b = tdh.Plan("leg2cheb", n, prec="fp32", ragged=True)
+    x = torch.tensor(workloads.coefficients(n, 9, decay=0.5, seed=4), dtype=torch.float32,
+                     device="cuda")
+    offs = torch.arange(10, device="cuda") * n
+    y = a.execute(x)
+    assert torch.equal(y, b.execute(x)) and torch.equal(a.adjoint(x), b.adjoint(x))
+    assert torch.equal(a.execute_ragged(x.flatten(), offs), b.execute_ragged(x.flatten(), offs))
+    a.set_schedule(0)
+    z = a.execute(x)
+    assert n < 64 or not torch.equal(z, y)
+    assert float(((z - y).abs().amax(1) / x.abs().sum(1)).max()) <= 5e-6 + TOL["fp32"]
+
+
 def test_unaligned_rows_and_nonfinite_inputs(tdh):
     """Odd lengths put every other vector at an odd offset; a NaN reaches exactly the outputs
     that depend on it (same parity, lower index) and no other vector."""
