@@ -717,7 +717,11 @@ static bool tc_stalled(const Step& st) {
 int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s, const std::vector<cudaStream_t>& side,
                        const std::vector<cudaEvent_t>& ev) {
-    if (st.hier.use_ragged && !tc_stalled(st)) return hier_launch_ragged(st, prec, in, out, offs, batch, s);
+    // A few short float64 vectors: the tree's latency (125 to 190 us, whatever the lengths) is
+    // longer than the FFTs take (41 us at 1024 x 2, 128 us at 4000 x 4; 270 us at 8000 x 4).
+    const bool few = prec == TDH_FP64 && st.n <= kRaggedFftLen && st.n * batch <= 32768;
+    if (st.hier.use_ragged && !few && !tc_stalled(st))
+        return hier_launch_ragged(st, prec, in, out, offs, batch, s);
     if (prec != TDH_FP64) return launch_ragged_typed<float>(st, in, out, offs, batch, s, side, ev);
     return launch_ragged_typed<double>(st, in, out, offs, batch, s, side, ev);
 }

@@ -1,8 +1,12 @@
 // Kernels and host side of the hierarchical T o H product (tdh_hier.cuh).
 //
-// Two launches per step: k_hier_up forms the moments of every box, k_hier_down exchanges them,
-// passes the local expansions down and adds the near field.  Vectors are independent; a CTA
-// takes a segment of rows of a few vectors, so every table entry it forms serves all of them.
+// Launches of a step: k_hier_up forms the moments of every box, k_hier_top (long vectors)
+// exchanges those of the 2048-boxes, k_hier_far the smaller boxes' and passes the local
+// expansions down, k_hier_near adds the near field and writes the result; each starts while the
+// one before it drains (programmatic dependent launch).  Short vectors, few of them: one
+// launch of k_hier_direct.  Vectors are independent; a CTA or warp takes a few of them, so every
+// table entry it forms serves all of them.  n = 2^16 x 256 float32: 160 us (the FFT form: 2120;
+// a copy of the batch: 20), n = 2^16 x 32 float64: 818 us (21760).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -240,7 +244,8 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // A CTA forms the moments of one 2048-box (64 leaves, their parents, ...) for unvt vectors.  A
 // warp takes one leaf of VW vectors at a time: lane (p, v) holds the 32 weights L_p in
 // registers, so each 16-byte shared load of inputs feeds 16 bytes' worth of multiply-adds; the
-// next leaf's inputs are loaded meanwhile.
+// next leaf's inputs are loaded meanwhile.  Bound by the latency of those loads (one leaf
+// ahead, four CTAs per SM): 41 us at n = 2^16 x 256 float32, whose inputs take 10 us to read.
 template <typename T, int NC, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_hier_up(const __grid_constant__ HierParams<T> P) {
     constexpr int NP = HierP<T>::P;
@@ -408,7 +413,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_hier_up(co
 // Exchange: a warp takes one box, its lanes the box's points, channels and VTL groups of VPT
 // vectors, so a coefficient s h that a lane forms (table offsets of the points are constants of
 // the level) serves VPT vectors.  Children: a thread takes one box of one vector whole, its
-// weights broadcast from shared memory.
+// weights broadcast from shared memory.  Bound by shared-memory reads (the staged moments) and,
+// in float64, the FP64 pipe: 52 us at n = 2^16 x 256 float32, 364 us at 2^16 x 32 float64.
 template <typename T, int NC, int NVT>
 struct FarShape {
     static constexpr int NP = HierP<T>::P;
@@ -693,7 +699,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_hier_far(
 // The two half-warps take half of the vectors each, a lane rows r and r + 16.  Values are taken
 // in pairs (two parities of one packed index, or two neighbouring indices), so one 16-byte
 // broadcast of inputs feeds four pair operations per row pair, and the entries s h a lane forms
-// serve all of its vectors.  Bound by the FP32 (FP64) pipe.
+// serve all of its vectors.  n = 2^16 x 256 float32: 76 us, the FP32 pipe 48 % busy and the LSU
+// 64 % (fused with the far field the whole product took 291 us against 160); two warps a
+// scheduler leave the latency of the shared loads exposed, but four of half as many
+// vectors load more and take 15 % longer.  n = 2^16 x 32 float64: 339 us, bound by the FP64 pipe.
 template <typename T, int NC, int NV>
 struct NearShape {
     static constexpr int NP = HierP<T>::P;
@@ -1019,10 +1028,12 @@ __global__ void __launch_bounds__(32 * NearShape<T, NC, NV>::warps, 1) k_hier_ne
 // Short vectors, few of them: every entry of the triangle once, no far field (one launch).  A
 // CTA stages the scaled inputs and the tables in shared memory; a warp takes one packed row
 // of V vectors, lanes along the columns (s from the diagonal on, h and the inputs all read with
-// consecutive lanes on consecutive places).
-template <typename T, int NC, int V>
+// consecutive lanes on consecutive places); where the rows are few, WR warps share one.  Bound by
+// its launch in float32 (2.6 to 6 us), by the FP64 pipe in float64.
+template <typename T, int NC, int V, int WR>  // WR warps share a row
 __global__ void __launch_bounds__(kThreads) k_hier_direct(const __grid_constant__ HierParams<T> P,
-                                                          int m, int rows) {
+                                                          int m) {
+    constexpr int rows = kWarps / WR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nrow = (m + rows - 1) / rows;
@@ -1034,6 +1045,7 @@ __global__ void __launch_bounds__(kThreads) k_hier_direct(const __grid_constant_
     T* sm = reinterpret_cast<T*>(smem_raw);     // s[0 .. w)
     T* hm = sm + w;                             // hh[l0 .. l0 + w + rows + 1)
     T* xm = hm + w + rows + 1;                  // [V][NC w]
+    T* sums = xm + V * NC * w;                  // [warp][V][NC]
     for (int i = tid; i < w; i += kThreads) sm[i] = P.s[i];
     for (int i = tid; i < w + rows + 1; i += kThreads) hm[i] = P.hh[l0 + i];
     for (int i = tid; i < NC * w; i += kThreads) {
@@ -1046,44 +1058,49 @@ __global__ void __launch_bounds__(kThreads) k_hier_direct(const __grid_constant_
         }
     }
     __syncthreads();
-    for (int r = warp; r < rows && a0 + r < m; r += kWarps) {
-        T acc[V][NC];
+    const int r = warp / WR, part = warp % WR;
+    T acc[V][NC];
 #pragma unroll
-        for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) acc[v][c] = T(0);
-        for (int b = r + lane; b < w; b += 32) {
-            const T s = sm[b - r];
+        for (int c = 0; c < NC; ++c) acc[v][c] = T(0);
+    for (int b = r + lane + 32 * part; b < w; b += 32 * WR) {
+        const T s = sm[b - r];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const T e = s * hm[r + b + c];
+        for (int c = 0; c < NC; ++c) {
+            const T e = s * hm[r + b + c];
 #pragma unroll
-                for (int v = 0; v < V; ++v) acc[v][c] += e * xm[v * NC * w + NC * b + c];
-            }
+            for (int v = 0; v < V; ++v) acc[v][c] += e * xm[v * NC * w + NC * b + c];
         }
+    }
 #pragma unroll
-        for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v)
 #pragma unroll
-            for (int c = 0; c < NC; ++c)
+        for (int c = 0; c < NC; ++c)
 #pragma unroll
-                for (int k = 16; k > 0; k >>= 1)
-                    acc[v][c] += __shfl_xor_sync(0xffffffffu, acc[v][c], k);
-        if (lane < NC * V) {
-            T y = T(0);
+            for (int k = 16; k > 0; k >>= 1)
+                acc[v][c] += __shfl_xor_sync(0xffffffffu, acc[v][c], k);
+    T y = T(0);
 #pragma unroll
-            for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v)
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (lane == v * NC + c) y = acc[v][c];
-            const int64_t g = g0 + lane / NC;
-            const int64_t kp = k0 + (int64_t)NC * (a0 + r) + lane % NC;
-            const int64_t k = P.rev ? P.npk - 1 - kp : kp;
-            if (g < P.batch && k < P.n) {
-                y *= P.dout[k];
-                if (P.sign_out && (k & 1)) y = -y;
-                if (k == 0 && P.a00) y += P.a00[0] * P.in[g * P.n];
-                P.out[g * P.n + k] = y;
-            }
+        for (int c = 0; c < NC; ++c)
+            if (lane == v * NC + c) y = acc[v][c];
+    if constexpr (WR > 1) {
+        if (lane < NC * V) sums[warp * (NC * V) + lane] = y;
+        __syncthreads();
+    }
+    if (part == 0 && lane < NC * V && a0 + r < m) {
+#pragma unroll
+        for (int i = 1; i < WR; ++i) y += sums[(warp + i) * (NC * V) + lane];
+        const int64_t g = g0 + lane / NC;
+        const int64_t kp = k0 + (int64_t)NC * (a0 + r) + lane % NC;
+        const int64_t k = P.rev ? P.npk - 1 - kp : kp;
+        if (g < P.batch && k < P.n) {
+            y *= P.dout[k];
+            if (P.sign_out && (k & 1)) y = -y;
+            if (k == 0 && P.a00) y += P.a00[0] * P.in[g * P.n];
+            P.out[g * P.n + k] = y;
         }
     }
 }
@@ -1409,30 +1426,41 @@ int launch_near(const HierParams<T>& P, int NV, int64_t nb, bool pdl, cudaStream
     return launch_near_nv<T, NC, 2, RAGGED>(P, nb, pdl, s);
 }
 
-// The direct product's shared memory, and whether it is the faster way: its work is m^2 B
-// multiply-adds, that of the tree a few launches and some hundred operations per coefficient.
+// The direct product's shared memory, the vectors a CTA takes (0: too long for it), and whether it
+// is the faster way.
 template <typename T>
-size_t direct_smem(int NC, int64_t m, int rows, int V) {
-    return sizeof(T) * (size_t)(2 * m + rows + 1 + V * NC * m);
+size_t direct_smem(int NC, int64_t m, int V) {
+    return sizeof(T) * (size_t)(2 * m + kWarps + 1 + V * NC * (m + kWarps));
+}
+template <typename T>
+int direct_vectors(int NC, int64_t m, int64_t batch) {
+    int V = batch == 1 ? 1 : batch == 2 ? 2 : 4;
+    while (V > 0 && direct_smem<T>(NC, m, V) > kMaxSmem) V = V == 4 ? 2 : 0;
+    return V;
 }
 template <typename T>
 bool direct_serves(int NC, int64_t m, int64_t batch) {
-    const double work = (double)m * (double)m * (double)batch * NC;
-    return m <= 4096 && work <= (sizeof(T) == 4 ? 1 << 24 : 1 << 20);
+    const int V = direct_vectors<T>(NC, m, batch);
+    if (V == 0) return false;
+    // Multiply-adds, the entries' products among them, against the tree's few launches, which take
+    // about the same time for any short vectors (Leg->Cheb and Jacobi: float32 21 and 16 us,
+    // float64 185 and 125 us).  Measured: float64 113 us at 40e6 (Jacobi 4000 x 4), 118 us at
+    // 41e6 (Leg->Cheb 5700 x 4); float32 13.5 us at 21e6 (Leg->Cheb 1024 x 64), 15 us at 32e6
+    // (8000 x 1), but 23 us at 40e6 (2000 x 32).
+    const double ops = 0.5 * NC * (double)m * (double)m * (double)((batch + V - 1) / V) * (V + 1);
+    return ops <= (sizeof(T) == 4 ? (batch <= 2 ? 33e6 : 24e6) : NC == 2 ? 64e6 : 40e6);
 }
 
-template <typename T, int NC, int V>
-int launch_direct(const HierParams<T>& P, int64_t m, cudaStream_t s) {
-    auto kern = k_hier_direct<T, NC, V>;
+template <typename T, int NC, int V, int WR>
+int launch_direct_wr(const HierParams<T>& P, int64_t m, unsigned grid, cudaStream_t s) {
+    auto kern = k_hier_direct<T, NC, V, WR>;
     static PerDevice once;
     cudaError_t e = per_device(once, [&](int*) {
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kMaxSmem);
     });
-    const int rows = kWarps;
-    const int64_t grid = (m + rows - 1) / rows * ((P.batch + V - 1) / V);
     if (e == cudaSuccess) {
-        kern<<<(unsigned)grid, kThreads, direct_smem<T>(NC, m, rows, V), s>>>(P, (int)m, rows);
+        kern<<<(unsigned)grid, kThreads, direct_smem<T>(NC, m, V), s>>>(P, (int)m);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
@@ -1441,6 +1469,18 @@ int launch_direct(const HierParams<T>& P, int64_t m, cudaStream_t s) {
     }
     note_launches(1);
     return TDH_OK;
+}
+
+// Rows per CTA (8 / WR) halved until every SM has a CTA: the SM that holds the longest rows sets
+// the time, in float64 by its 2 multiply-adds per clock (Leg->Cheb n = 1024 float64: 10.4 us with
+// 64 CTAs of 8 rows, 7.5 us with 256 of 2).
+template <typename T, int NC, int V>
+int launch_direct(const HierParams<T>& P, int64_t m, cudaStream_t s) {
+    const int64_t groups = (P.batch + V - 1) / V;
+    auto grid = [&](int rows) { return (m + rows - 1) / rows * groups; };
+    if (grid(8) >= sm_count()) return launch_direct_wr<T, NC, V, 1>(P, m, (unsigned)grid(8), s);
+    if (grid(4) >= sm_count()) return launch_direct_wr<T, NC, V, 2>(P, m, (unsigned)grid(4), s);
+    return launch_direct_wr<T, NC, V, 4>(P, m, (unsigned)grid(2), s);
 }
 
 template <typename T, int NC, bool RAGGED>
@@ -1478,22 +1518,32 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         P.batch = batch;
         P.in = static_cast<const T*>(in);
         P.out = static_cast<T*>(out);
-        return batch == 1 ? launch_direct<T, NC, 1>(P, m, s) : launch_direct<T, NC, 4>(P, m, s);
+        const int V = direct_vectors<T>(NC, m, batch);
+        return V == 1   ? launch_direct<T, NC, 1>(P, m, s)
+               : V == 2 ? launch_direct<T, NC, 2>(P, m, s)
+                        : launch_direct<T, NC, 4>(P, m, s);
     }
     // vectors of a near-field warp, and of a far-field CTA
     constexpr int VMAX = sizeof(T) == 4 ? 32 : 16;
     constexpr int FMAX = sizeof(T) == 4 ? 16 : 8;
-    P.nvt = batch > 2 ? FMAX : 2;
+    P.seg_leaves = real_leaves > 4 ? 16 : 4;
+    P.nseg = (P.leaves + P.seg_leaves - 1) / P.seg_leaves;
+    // Two vectors per far CTA while such CTAs do not fill the chip: a CTA's time grows with its
+    // vectors, its tables' share only matters once the SMs are full (Leg->Cheb 16000 x 8 float64:
+    // 343 us with 8, 188 us with 2, the near field's vectors chosen alike).
+    P.nvt = batch > 2 && (batch + 1) / 2 * P.nseg > sm_count() ? FMAX : 2;
     P.unvt = 32 / NP;
     // Near field: vectors of a warp (twice as many on half as many warps do the same work per SM
     // and step with fewer loads, about 15 % less time) and leaves it walks (a walk loads one leaf
     // more than it completes).  One CTA per SM is resident: the waves should be full.
     int NV = 2;
     double best = 0;
-    for (int nv = batch > 2 ? VMAX / (sizeof(T) == 4 ? 4 : 2) : 2; nv <= VMAX; nv *= 2) {
+    for (int nv = 2; nv <= VMAX; nv *= nv == 2 ? 4 : 2) {
         const int64_t slots = (nv == VMAX ? 8 : 16) * (int64_t)sm_count();
         const int64_t vgroups = (batch + nv - 1) / nv;
-        const double step = nv == VMAX ? 1.0 : nv == 16 || sizeof(T) == 8 ? 1.15 * nv / (VMAX / 2) : 0.8;
+        const double step = nv == VMAX ? 1.0
+                            : nv == 2  ? 0.65
+                            : nv == 16 || sizeof(T) == 8 ? 1.15 * nv / (VMAX / 2) : 0.8;
         for (int run = 16; run >= 1; --run) {
             const int64_t tasks = (real_leaves + run - 1) / run * vgroups;
             const double cost = (double)((tasks + slots - 1) / slots) * (run + 0.4) * step;
@@ -1506,8 +1556,6 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         if (batch <= 2) break;
     }
     P.runs = (P.leaves + P.run - 1) / P.run;
-    P.seg_leaves = real_leaves > 4 ? 16 : 4;
-    P.nseg = (P.leaves + P.seg_leaves - 1) / P.seg_leaves;
     const int64_t ntop = (P.leaves + kHierTopLeaves - 1) / kHierTopLeaves;
     // moments of every box and expansions of every leaf of a vector; about 1 GB at a time
     int64_t boxes[kHierLevels], total = 0;

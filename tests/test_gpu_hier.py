@@ -88,6 +88,15 @@ def test_vector_groups(tdh, batch, prec):
     _check(tdh, "jacobi", 1300, batch, prec)
 
 
+def test_short_batches(tdh):
+    """Where the direct product takes two vectors per CTA for want of shared memory, and its
+    last sizes before the tree."""
+    for name, n, batch in (("cheb2leg", 5900, 3), ("cheb2leg", 5900, 4), ("cheb2leg", 5400, 4),
+                           ("jacobi", 4400, 3), ("cheb2leg", 400, 70)):
+        _check(tdh, name, n, batch, "fp64")
+        _check(tdh, name, n, batch, "fp32")
+
+
 def test_long_vectors_match_the_fft_schedule(tdh):
     """Several 2048-boxes (the top level's exchange) and the deepest tree, against the FFT schedule
     of the same plan: both within the stated tolerance, so within twice of each other."""
@@ -110,10 +119,17 @@ def test_long_vectors_match_the_fft_schedule(tdh):
 def test_ragged_edges(tdh, prec):
     """Lengths at the tree's edges in one ragged batch, each against the oracle; vectors that
     share a group with longer ones do not see them."""
-    import torch
     lengths = np.array([0, 1, 2, 63, 64, 65, 127, 129, 1000, 4096, 4097, 5000, 3, 0, 64] * 3)
+    _ragged(tdh, lengths, 5000, prec)
+    # a few short vectors (float64: the FFT schedules), and the same plan with more of them
+    _ragged(tdh, np.array([0, 1, 700, 64, 1000]), 1000, prec)
+    _ragged(tdh, np.array([1000, 700, 64, 0] * 20), 1000, prec)
+
+
+def _ragged(tdh, lengths, n_max, prec):
+    import torch
     x, offs = workloads.ragged_coefficients(lengths, decay=0.5, seed=9)
-    plan = tdh.Plan("cheb2leg", 5000, prec=prec, ragged=True)
+    plan = tdh.Plan("cheb2leg", n_max, prec=prec, ragged=True)
     y = plan.execute_ragged(torch.tensor(x, dtype=plan.dtype, device="cuda"),
                             torch.tensor(offs, device="cuda")).double().cpu().numpy()
     for v in range(len(lengths)):
