@@ -36,8 +36,8 @@ GUARANTEE = {"leg2cheb": "tolerance met for every alpha (truncation bound)",
 DECAY = 0.5
 WORKLOAD = "leg2cheb+cheb2leg n=65536 batch=256"
 METRIC = "Leg<->Cheb coefficients/s"
-PROFILE = os.path.join(ROOT, "profiles", "exec_fp32_n65536_b256.txt")
-KERNEL_SOURCES = ["paper_1604_07486_gb300/csrc/tdh_exec.cuh", "paper_1604_07486_gb300/csrc/tdh_fft.cuh"]
+PROFILE = os.path.join(ROOT, "profiles", "hier_fp32_n65536_b256.txt")
+KERNEL_SOURCES = ["paper_1604_07486_gb300/csrc/tdh_hier.cu", "paper_1604_07486_gb300/csrc/tdh_hier.cuh"]
 
 
 def kernel_hash():
@@ -72,16 +72,15 @@ def tune(plan, batch, args):
     return ms, desc
 
 
-def flops_per_vector(K, n):
-    """Algorithmic flops of one vector of n coefficients, the path's per-unit figure: per rank
-    term two real FFTs of length L = nextpow2(2n - 1) (2.5 L log2 L each, 10 n log2 L for the
-    pair) plus 9 flops per coefficient of pointwise work (factor and spectrum products,
-    scalings), i.e. K (10 log2 L + 9) per coefficient.  The kernels compute the same transform
-    with packed complex FFTs (even/odd or rank-pair packing); that is not counted as less
-    work."""
-    import math
-    L = 1 << max(0, math.ceil(math.log2(max(2 * n - 1, 1))))
-    return K * n * (10 * math.log2(L) + 9)
+def flops_per_vector(n, points=8):
+    """Flops of one vector of n coefficients in the hierarchical product, which the plans run:
+    multiply-adds per coefficient of the near field (a leaf of 32 meets itself and its right
+    neighbour: 1552 entries), moments and leaf expansions (2 P), the exchange (4.5 boxes on
+    average, P^2 each) and the two transfers (P^2 each) of every level of boxes.  P = 8 points in
+    float32, 16 in float64.  Table entries (one product per entry and group of vectors) are not
+    counted."""
+    levels = (1 + 1 / 4 + 1 / 16) * points * points / 32
+    return 2 * n * (1552 / 32 + 2 * points + 4.5 * levels + 2 * levels)
 
 
 class ClockSampler:
@@ -502,8 +501,8 @@ def main():
     coeffs_per_step = len(KINDS) * BATCH * N
     value, total_ms = job_throughput(sum(step_ms), coeffs_per_step, args.steps, world, dist)
 
-    # roofline of the execute kernel (the only kernel in the timed region)
-    flops = sum(flops_per_vector(plans32[k].K, N) * BATCH for k in KINDS) * args.steps
+    # roofline of the product's kernels (the only ones in the timed region)
+    flops = len(KINDS) * flops_per_vector(N) * BATCH * args.steps
     achieved = flops / (total_ms / 1e3) / 1e12
     clocks = sampler.summary()
     peaks = measured_peaks()
@@ -549,7 +548,7 @@ def main():
         if rank == 0:
             for k in KINDS:
                 err64[k] = oracle_error(alpha, y64[k].cpu().numpy(), k, [0, BATCH - 1], rows)
-        flops64 = sum(flops_per_vector(plans64[k].K, N) * BATCH for k in KINDS)
+        flops64 = len(KINDS) * flops_per_vector(N, 16) * BATCH
         fp64 = {"value": world * coeffs_per_step * reps / (ms64 / 1e3), "unit": "coeffs/s",
                 "ms_per_step": ms64 / reps, "reps": reps, "K": {k: plans64[k].K for k in KINDS},
                 "plans": PLAN64, "error_vs_oracle": err64, "schedule": tuned64,
@@ -666,7 +665,8 @@ def run_extra(args, rank, world, local):
         y = torch.empty_like(x)
         fn = lambda: plan.execute(x, out=y)
         coeffs, dtype = n * B, "f64"
-        flops = flops_per_vector(plan.K, n) * B
+        # the direct product: every entry s h of the two channels' triangles, times the input
+        flops = 3 * 2 * (n // 2) * (n // 2 + 1) / 2 * B
         bound, peak, unit, pnote = "alu", apeaks["fp64"], "TFLOP/s", "FP64 DFMA " + apeaks["note"]
         config = {"workload": "leg2cheb n=1024 batch=1 fp64 tol=1e-15", "K": plan.K}
         check = lambda: {"leg2cheb": float(np.abs(y.cpu().numpy() - oracle.matvec(oracle.LEG2CHEB, None, alpha)).max() / np.abs(alpha).sum())}
@@ -694,7 +694,7 @@ def run_extra(args, rank, world, local):
         graph_launches = tdh.launch_count() - c0  # kernels in the captured graph
         fn = graph.replay
         coeffs, dtype = int(offs[-1]), "f32"
-        flops = sum(flops_per_vector(plan.K, int(n)) for n in lengths)
+        flops = sum(flops_per_vector(int(n)) for n in lengths)
         bound, peak, unit, pnote = "alu", fp32_peak, "TFLOP/s", "FP32 FFMA " + apeaks["note"]
         config = {"workload": "ragged leg2cheb 4096 vectors, degrees log-uniform [64, 65536), fp32, one CUDA-graph launch",
                   "K": plan.K, "plan": PLAN32["leg2cheb"], "coefficients": coeffs}
@@ -731,9 +731,8 @@ def run_extra(args, rank, world, local):
             ev_mid.append(e)
             pu.execute(x, out=yu)
         coeffs, dtype = 2 * n * B, "f32"
-        # both Jacobi steps (factor count from the plan)
-        flops = 2 * flops_per_vector(pj.K, n) * B
-        bound, peak, unit, pnote = "alu", fp32_peak, "TFLOP/s", "FP32 FFMA " + apeaks["note"] + " (Jacobi multi-pass part)"
+        flops = 2 * flops_per_vector(n) * B  # both Jacobi steps
+        bound, peak, unit, pnote = "alu", fp32_peak, "TFLOP/s", "FP32 FFMA " + apeaks["note"] + " (Jacobi part)"
         config = {"workload": "jacobi (0.1,-0.3)->(0,0) + ultraspherical 0.25->1.25, n=2^20, batch=16, fp32 execute, fp64 plan, tol 1e-13",
                   "K_jacobi_max_step": pj.K}
         def check():
@@ -772,7 +771,7 @@ def run_extra(args, rank, world, local):
             beta = convert(x, plan)
             (wgt * beta * beta).sum().backward()
         coeffs, dtype = n * B, "f32"
-        flops = 2 * flops_per_vector(plan.K, n) * B
+        flops = 2 * flops_per_vector(n) * B
         bound, peak, unit, pnote = "alu", fp32_peak, "TFLOP/s", "FP32 FFMA " + apeaks["note"]
         config = {"workload": "autograd leg2cheb n=8192 batch=1024 fp32: forward + loss + backward (adjoint kernel)",
                   "K": plan.K, "plan": PLAN32["leg2cheb"]}

@@ -244,8 +244,9 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // A CTA forms the moments of one 2048-box (64 leaves, their parents, ...) for unvt vectors.  A
 // warp takes one leaf of VW vectors at a time: lane (p, v) holds the 32 weights L_p in
 // registers, so each 16-byte shared load of inputs feeds 16 bytes' worth of multiply-adds; the
-// next leaf's inputs are loaded meanwhile.  Bound by the latency of those loads (one leaf
-// ahead, four CTAs per SM): 41 us at n = 2^16 x 256 float32, whose inputs take 10 us to read.
+// next leaf's inputs are loaded meanwhile.  Bound by shared-memory reads (LSU 65 % busy, their
+// latency the main stall): 41 us at n = 2^16 x 256 float32, whose inputs take 10 us to read; in
+// float64 by the FP64 pipe (83 % busy): 131 us at 2^16 x 32.
 template <typename T, int NC, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_hier_up(const __grid_constant__ HierParams<T> P) {
     constexpr int NP = HierP<T>::P;
@@ -413,8 +414,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_hier_up(co
 // Exchange: a warp takes one box, its lanes the box's points, channels and VTL groups of VPT
 // vectors, so a coefficient s h that a lane forms (table offsets of the points are constants of
 // the level) serves VPT vectors.  Children: a thread takes one box of one vector whole, its
-// weights broadcast from shared memory.  Bound by shared-memory reads (the staged moments) and,
-// in float64, the FP64 pipe: 52 us at n = 2^16 x 256 float32, 364 us at 2^16 x 32 float64.
+// weights broadcast from shared memory.  Bound by shared-memory reads (LSU 65 % busy) and the
+// barriers between its phases: 52 us at n = 2^16 x 256 float32; in float64 by the FP64 pipe (76 %
+// busy): 364 us at 2^16 x 32.
 template <typename T, int NC, int NVT>
 struct FarShape {
     static constexpr int NP = HierP<T>::P;
