@@ -1444,13 +1444,17 @@ template <typename T>
 bool direct_serves(int NC, int64_t m, int64_t batch) {
     const int V = direct_vectors<T>(NC, m, batch);
     if (V == 0) return false;
-    // Multiply-adds, the entries' products among them, against the tree's few launches, which take
-    // about the same time for any short vectors (Leg->Cheb and Jacobi: float32 21 and 16 us,
-    // float64 185 and 125 us).  Measured: float64 113 us at 40e6 (Jacobi 4000 x 4), 118 us at
-    // 41e6 (Leg->Cheb 5700 x 4); float32 13.5 us at 21e6 (Leg->Cheb 1024 x 64), 15 us at 32e6
-    // (8000 x 1), but 23 us at 40e6 (2000 x 32).
-    const double ops = 0.5 * NC * (double)m * (double)m * (double)((batch + V - 1) / V) * (V + 1);
-    return ops <= (sizeof(T) == 4 ? (batch <= 2 ? 33e6 : 24e6) : NC == 2 ? 64e6 : 40e6);
+    // Lane operations: multiply-adds, the entries' products among them, half a warp of each row
+    // idle on average, and a row's reductions (five adds a lane and sum); against the tree, whose
+    // few launches take about the same time for any short vectors (float32 21 us, Jacobi 16;
+    // float64 185 and 125 us), or its one launch where there is no far field (two leaves: float32
+    // 6 to 9 us, float64 60 to 100).  Measured, direct: float64 113 us at 45e6 (Leg->Cheb 5700 x 4),
+    // 60 us at 21e6 (100 x 1000), 114 us at 52e6 (64 x 4096, the tree 63); float32 13.5 us at 33e6
+    // (1024 x 64, the tree 17.6), 17.7 us at 68e6 (256 x 1024, the tree 14.9).
+    const double cost = NC * (double)m * (double)((batch + V - 1) / V) *
+                        ((V + 1) * (0.5 * (double)m + 16) + 160 * V);
+    if (m <= 2 * kHierLeaf) return cost <= (sizeof(T) == 4 ? 14.5e6 : 22e6);
+    return cost <= (sizeof(T) == 4 ? 35e6 : NC == 2 ? 70e6 : 44e6);
 }
 
 template <typename T, int NC, int V, int WR>
