@@ -714,6 +714,14 @@ static bool tc_stalled(const Step& st) {
     return tc;
 }
 
+// The tables of an FFT launch are there.  They always are on the routes below; a configuration
+// without them is an error on the host, never a launch on null tables.
+static int require_built(const ExecData& ex) {
+    if (ex.built) return TDH_OK;
+    set_error("the FFT tables of this step are not built");
+    return TDH_ERR_UNSUPPORTED;
+}
+
 int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s, const std::vector<cudaStream_t>& side,
                        const std::vector<cudaEvent_t>& ev) {
@@ -722,6 +730,7 @@ int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, cons
     const bool few = prec == TDH_FP64 && st.n <= kRaggedFftLen && st.n * batch <= 32768;
     if (st.hier.use_ragged && !few && !tc_stalled(st))
         return hier_launch_ragged(st, prec, in, out, offs, batch, s);
+    for (const ExecData& ex : st.rcls) TDH_TRY(require_built(ex));
     if (prec != TDH_FP64) return launch_ragged_typed<float>(st, in, out, offs, batch, s, side, ev);
     return launch_ragged_typed<double>(st, in, out, offs, batch, s, side, ev);
 }
@@ -734,6 +743,7 @@ int exec_launch(const Step& st, int prec, const void* in, void* out, int64_t bat
 
 int fft_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
                cudaStream_t s) {
+    TDH_TRY(require_built(st.ex));
     if (st.ex.multipass) return mp_launch(st, prec, in, out, batch, adjoint, s);
     if (prec != TDH_FP64) return launch_typed<float>(st, in, out, batch, adjoint, s);
     return launch_typed<double>(st, in, out, batch, adjoint, s);
@@ -907,7 +917,15 @@ int autotune_typed(tdh_plan_s& plan, int64_t batch, cudaStream_t s) {
         cleanup();
         return TDH_ERR_CUDA;
     }
-    float ragged_fft = 0, ragged_hier = 0;  // length classes together: they run in one call
+    // What the timings say of each step's form.  Applied only once every configuration is timed: a
+    // call that fails half-way leaves the plan on the forms it ran before.
+    struct Choice {
+        Step* st;
+        bool dense = false;            // the dense configuration was timed both ways
+        bool dense_hier = false;
+        float ragged_fft = 0, ragged_hier = 0;  // length classes together: they run in one call
+    };
+    std::vector<Choice> choices;
     for (const ConfigRef& r : cfgs) {
         const std::vector<Geometry> cands =
             schedule_candidates(prec, config_data(r).g.logL, r.cls >= 0);
@@ -926,16 +944,29 @@ int autotune_typed(tdh_plan_s& plan, int64_t batch, cudaStream_t s) {
         if (rc == TDH_OK && r.st->hier.on) {
             float ms = 0;
             rc = time_config<T>(r, batch, tb, true, s, &ms);
+            if (choices.empty() || choices.back().st != r.st) choices.push_back(Choice{r.st});
+            Choice& c = choices.back();
             if (r.cls < 0) {
-                r.st->hier.use = ms <= best_ms;
+                c.dense = true;
+                c.dense_hier = ms <= best_ms;
             } else {
-                ragged_fft += best_ms;
-                ragged_hier += ms;
-                r.st->hier.use_ragged = ragged_hier <= ragged_fft;
+                c.ragged_fft += best_ms;
+                c.ragged_hier += ms;
             }
         }
         if (rc != TDH_OK) break;
     }
+    // a step that goes to its FFTs needs the tables of all its configurations, those with one
+    // schedule (not timed) among them
+    for (const Choice& c : choices) {
+        const bool to_fft = (c.dense && !c.dense_hier) || c.ragged_hier > c.ragged_fft;
+        if (rc == TDH_OK && to_fft) rc = exec_build(*c.st, prec, s);
+    }
+    if (rc == TDH_OK)
+        for (const Choice& c : choices) {
+            if (c.dense) c.st->hier.use = c.dense_hier;
+            if (c.ragged_fft > 0) c.st->hier.use_ragged = c.ragged_hier <= c.ragged_fft;
+        }
     cleanup();
     return rc;
 }

@@ -1,0 +1,73 @@
+"""Which form a call takes (hierarchical product, direct product, FFT schedules, sums or affine
+scans), and what it needs for that (needs a GPU): a plan that stays usable when a call fails
+half-way, scratch that is bounded, results that do not depend on how a call was cut up.
+
+Tolerances: the stated ones (float32 5e-6, float64 1e-12 of ||alpha||_1) unless a test says
+otherwise.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+NOMEM = -3
+TOL = {"fp64": 1e-12, "fp32": 5e-6, "bf16x3": 1e-5}
+
+
+@pytest.fixture(scope="module")
+def tdh():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1604_07486_gb300 as m
+    from paper_1604_07486_gb300 import build
+    build.build()
+    yield m
+    m.inject_alloc_failure(0)
+
+
+@pytest.mark.parametrize("n,prec", [(4096, "fp32"), (700, "fp32"), (9000, "fp64")])
+def test_autotune_that_fails_leaves_the_plan_usable(tdh, n, prec):
+    """Every allocation of autotune in turn (a spread of them) fails: the plan goes on giving the
+    results it gave before, bit for bit, ragged and dense; a whole autotune's choice stays within
+    the tolerance for every length class."""
+    import torch
+    lengths = np.array([n, 1, 100, 0, 257, n // 2, n // 3, 64])
+    x, offs = workloads.ragged_coefficients(lengths, decay=1.0, seed=5)
+    ot = torch.tensor(offs, device="cuda")
+    made, failed = None, 0
+    for k in [0] + list(range(1, 30)):
+        plan = tdh.Plan("leg2cheb", n, prec=prec, ragged=True)
+        xt = torch.tensor(x, dtype=plan.dtype, device="cuda")
+        dense = xt[:n].reshape(1, n).clone()
+        before = plan.execute_ragged(xt, ot), plan.execute(dense), plan.adjoint(dense)
+        if k == 0:
+            a0 = tdh.alloc_stats()[0]
+            plan.autotune(6)
+            made = tdh.alloc_stats()[0] - a0
+            y = plan.execute_ragged(xt, ot).double().cpu().numpy()
+            for v in range(len(lengths)):
+                a, b = int(offs[v]), int(offs[v + 1])
+                if b > a:
+                    ref = oracle.matvec(oracle.LEG2CHEB, None, x[a:b])
+                    assert np.abs(y[a:b] - ref).max() <= TOL[prec] * np.abs(x[a:b]).sum()
+        else:
+            at = 1 + (k - 1) * int(0.85 * made) // 28  # (a choice of schedule costs a few)
+            tdh.inject_alloc_failure(at)
+            try:
+                plan.autotune(6)
+                raised = False
+            except tdh.TdhError as e:
+                assert e.code == NOMEM, at
+                raised = True
+            tdh.inject_alloc_failure(0)
+            failed += raised
+            after = plan.execute_ragged(xt, ot), plan.execute(dense), plan.adjoint(dense)
+            if raised:
+                assert all(torch.equal(a, b) for a, b in zip(before, after)), at
+        assert plan.status() == set()
+        plan.close()
+    assert failed >= 20
