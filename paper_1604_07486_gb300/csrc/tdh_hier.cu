@@ -26,7 +26,7 @@ struct HierParams {
     const T* in;
     T* out;
     int64_t n;       // coefficients per vector (dense)
-    int64_t npk;     // NC * mpad: padded length (index reversal)
+    int64_t npk;     // NC * the padded length per channel (index reversal, table ends)
     int64_t batch;   // vectors of this launch
     int64_t bpad;    // vectors per box row of the moment arrays
     const T* s;
@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(32 * NearShape<T, NC, NV>::warps, 1) k_hier_ne
     __syncthreads();
     const int64_t task = (int64_t)blockIdx.x * S::warps + warp;
     const int64_t g0 = task / P.runs * NV;
-    int i0 = (int)(task % P.runs) * P.run;
+    const int i0 = P.leaf0 + (int)(task % P.runs) * P.run;
     bool far = false;
     int leaves = 0;
     if (g0 < P.batch) {
@@ -766,7 +766,6 @@ __global__ void __launch_bounds__(32 * NearShape<T, NC, NV>::warps, 1) k_hier_ne
         far = P.loc && group_leaves<T, NC, RAGGED>(P, g0 / P.nvt * P.nvt) > 2;
     }
     const int i1 = min(i0 + P.run, leaves);
-    i0 = max(i0, P.leaf0);
     if (i0 >= i1) {
         pdl_wait();  // the launch must not complete before the previous one does
         return;
@@ -1195,20 +1194,20 @@ double lagrange(const int* x, int P, int i, double at) {
 }
 
 // table copies in execute precision: s_m = t[stride m] (32 zeros before, zero past mpad),
-// hf_l = h[stride l], hr_i = hf[2 mpad - 1 - i]; entry 0 of h dropped where (0, 0) is direct
+// hf_l = h[stride l], hr_i = hf[2 mrev - 1 - i] (zero past 2 mrev); entry 0 of h dropped where
+// (0, 0) is direct
 template <typename T>
 __global__ void k_hier_tables(const double* __restrict__ t, const double* __restrict__ h,
-                              int64_t mpad, int stride, int j0, T* __restrict__ s,
+                              int64_t mpad, int64_t mrev, int stride, int j0, T* __restrict__ s,
                               T* __restrict__ hf, T* __restrict__ hr) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i < kHierSZero) s[i - kHierSZero] = T(0);
     if (i < mpad) s[i] = (T)t[stride * i];
     if (i < 2 * mpad + kHierHPad) {
-        const bool in = i < 2 * mpad;
-        const T v = (!in || (j0 == 1 && i == 0)) ? T(0) : (T)h[stride * i];
+        const T v = (i >= 2 * mpad || (j0 == 1 && i == 0)) ? T(0) : (T)h[stride * i];
         hf[i] = v;
-        if (in)
-            hr[2 * mpad - 1 - i] = v;
+        if (i < 2 * mrev)
+            hr[2 * mrev - 1 - i] = v;
         else
             hr[i] = T(0);
     }
@@ -1239,12 +1238,24 @@ __global__ void k_hier_points(const T* __restrict__ s, const T* __restrict__ hf,
     }
 }
 
+// Packed length of a reversed vector of m indices: whole boxes of the largest size that exchanges
+// anything (three boxes or more), so that its last one ends at index 0, beyond which h is not
+// smooth, and the padding lies before its first leaf.  (Whole 2048-boxes for every length made
+// transposes of short vectors form moments and launch warps for up to 63 empty leaves: Leg->Cheb
+// 200 x 1024 float32 41 us, now 18; the FFTs take 29.)
+int64_t reversed_length(int64_t m) {
+    int l = kHierLevels - 1;
+    while (l > 0 && m <= 2 * hier_size(l)) --l;
+    return (m + hier_size(l) - 1) / hier_size(l) * hier_size(l);
+}
+
 template <typename T>
 int prepare_typed(Step& st, cudaStream_t s) {
     constexpr int P = HierP<T>::P;
     HierData& H = st.hier;
     const int NC = st.full ? 1 : 2;
     H.mpad = (hier_length(st) - 2) / NC;
+    H.mrev = reversed_length((st.n + NC - 1) / NC);
     const size_t ns = (size_t)(H.mpad + kHierSZero), nh = (size_t)(2 * H.mpad + kHierHPad);
     const size_t nw = (size_t)P * kHierLeaf + 12 * P * P;
     // long vectors: the 2048-boxes' point tables (k_hier_top)
@@ -1262,7 +1273,7 @@ int prepare_typed(Step& st, cudaStream_t s) {
         H.w = tab + ns + 2 * nh;
         const int64_t cnt = 2 * H.mpad + kHierHPad;
         k_hier_tables<T><<<(unsigned)((cnt + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-            st.t, st.h, H.mpad, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
+            st.t, st.h, H.mpad, H.mrev, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
             static_cast<T*>(H.hr));
         if (top) {
             H.st = tab + at;
@@ -1497,9 +1508,9 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     const int64_t m = (st.n + NC - 1) / NC;
     HierParams<T> P{};
     P.n = st.n;
-    P.npk = NC * H.mpad;
+    P.npk = NC * (adjoint ? H.mrev : H.mpad);
     P.s = static_cast<const T*>(H.s);
-    // reversed: packed index a' + b' meets hf[2 (mpad - 1) - a' - b' (+ 1 in channel 0)]
+    // reversed: packed index a' + b' meets hf[2 (mrev - 1) - a' - b' (+ 1 in channel 0)]
     P.hh = static_cast<const T*>(adjoint ? H.hr : H.hf) + (adjoint && NC == 1 ? 1 : 0);
     P.st = static_cast<const T*>(H.st);
     P.ht = static_cast<const T*>(H.ht[adjoint ? 1 : 0]);
@@ -1513,8 +1524,8 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     P.sign_in = st.sign_in;
     P.sign_out = st.sign_out;
     if (adjoint) {
-        P.leaf0 = (int)((H.mpad - m) / kHierLeaf);
-        P.leaves = (int)(H.mpad / kHierLeaf);
+        P.leaf0 = (int)((H.mrev - m) / kHierLeaf);
+        P.leaves = (int)(H.mrev / kHierLeaf);
     } else {
         P.leaf0 = 0;
         P.leaves = (int)((m + kHierLeaf - 1) / kHierLeaf);
@@ -1561,11 +1572,12 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         }
         if (batch <= 2) break;
     }
-    P.runs = (P.leaves + P.run - 1) / P.run;
+    P.runs = (real_leaves + P.run - 1) / P.run;
     const int64_t ntop = (P.leaves + kHierTopLeaves - 1) / kHierTopLeaves;
     // moments of every box and expansions of every leaf of a vector; about 1 GB at a time
     int64_t boxes[kHierLevels], total = 0;
-    for (int l = 0; l < kHierLevels; ++l) total += boxes[l] = (H.mpad / kHierLeaf) >> (2 * l);
+    for (int l = 0; l < kHierLevels; ++l)
+        total += boxes[l] = (P.leaves + (1 << (2 * l)) - 1) >> (2 * l);
     const bool far = real_leaves > 2;
     P.ntop = (int)ntop;
     const bool top = ntop >= kTopKernel;

@@ -143,6 +143,7 @@ struct HierData {
     int use = 0;          // dense executes take this path (else the FFT schedules)
     int use_ragged = 0;   // ragged executes take it
     int64_t mpad = 0;     // packed indices per channel, padded to whole 2048-boxes
+    int64_t mrev = 0;     // the same for reversed vectors (transpose)
     void* tab = nullptr;  // one allocation: s, the two Hankel tables, leaf and transfer weights
     void* s = nullptr;    // s[-32 .. mpad]
     void* hf = nullptr;   // Hankel table, forward

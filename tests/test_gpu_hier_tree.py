@@ -1,0 +1,73 @@
+"""The hierarchical product's tree (needs a GPU): sizes at the edges of its boxes in batches large
+enough that the direct product does not take them, forward and transposed, vector groups of the
+wide far-field kernel, chunks of vectors, and inputs that only the far field sees.
+
+Bound, as in the direct product's test: off the diagonal every entry of these kinds has one sign,
+so sum |A_jk| |alpha_k| is at most |A| |alpha| plus twice the diagonal's part; a result is within 64
+roundings of it and the far field's claim (float32 2.5e-8, float64 1e-14), in the norm.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+U = {"fp64": 2.0 ** -53, "fp32": 2.0 ** -24}
+FAR = {"fp64": 1e-14, "fp32": 2.5e-8}
+KINDS = {"leg2cheb": ("leg2cheb", oracle.LEG2CHEB, None),
+         "cheb2leg": ("cheb2leg", oracle.CHEB2LEG, None),
+         "ultra": ("ultra2ultra", oracle.ULTRA, (0.9, 0.2)),
+         "jacobi": ("jac2jac", oracle.JAC, (0.05, 0.3, 0.95, 0.3))}
+
+
+@pytest.fixture(scope="module")
+def tdh():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1604_07486_gb300 as m
+    from paper_1604_07486_gb300 import build
+    build.build()
+    return m
+
+
+def _check_vectors(name, x, y, picks, prec, tr, rows=None):
+    """Rows `rows` (all if None) of the vectors `picks` against the oracle."""
+    _, okind, params = KINDS[name]
+    n = x.shape[1]
+    r = np.arange(n) if rows is None else rows
+    ref = oracle.matvec(okind, params, x[picks], rows=r, transpose=tr)
+    size = np.abs(oracle.matvec(okind, params, np.abs(x[picks]), rows=r, transpose=tr))
+    t, h, d1, d2 = oracle.split(okind, params, n)
+    diag = np.abs(d1 * t[0] * h[::2] * d2)
+    if name == "cheb2leg":
+        diag[0] = 1.0
+    size = size + 2 * diag[r] * np.abs(x[picks][:, r])
+    err = np.linalg.norm(y[np.ix_(picks, r)] - ref, axis=1)
+    assert np.all(err <= (64 * U[prec] + FAR[prec]) * np.linalg.norm(size, axis=1)), \
+        (name, n, prec, tr, (err / np.linalg.norm(size, axis=1)).max())
+
+
+# packed lengths just above one, two and four boxes of 32, 128, 512 and 2048, and odd ones between
+# (two channels: n = 2 m)
+@pytest.mark.parametrize("n", [130, 150, 257, 300, 514, 516, 1030, 1537, 2049, 2060, 4100, 8195])
+@pytest.mark.parametrize("name", sorted(KINDS))
+def test_tree_at_box_edges(tdh, name, n):
+    import torch
+    kind, _, params = KINDS[name]
+    for prec in ("fp32", "fp64"):
+        # past the direct product's limit: lane operations, as it counts them, above 1e8
+        channels = 1 if kind == "jac2jac" else 2
+        m = (n + channels - 1) // channels
+        batch = max(12, int(1e8 / (channels * m / 4 * (5 * (m / 2 + 16) + 640))) + 1)
+        x = workloads.coefficients(n, batch, decay=0.5, seed=n)
+        if prec == "fp32":
+            x = x.astype(np.float32).astype(np.float64)
+        plan = tdh.Plan(kind, n, prec=prec, params=params or ())
+        xt = torch.tensor(x, dtype=plan.dtype, device="cuda")
+        picks = np.unique([0, 1, batch // 2, batch - 1])
+        for fn, tr in ((plan.execute, False), (plan.adjoint, True)):
+            y = fn(xt).double().cpu().numpy()
+            _check_vectors(name, x, y, picks, prec, tr)
