@@ -1460,12 +1460,14 @@ bool direct_serves(int NC, int64_t m, int64_t batch) {
     // few launches take about the same time for any short vectors (float32 21 us, Jacobi 16;
     // float64 185 and 125 us), or its one launch where there is no far field (two leaves: float32
     // 6 to 9 us, float64 60 to 100).  Measured, direct: float64 113 us at 45e6 (Leg->Cheb 5700 x 4),
-    // 60 us at 21e6 (100 x 1000), 114 us at 52e6 (64 x 4096, the tree 63); float32 13.5 us at 33e6
-    // (1024 x 64, the tree 17.6), 17.7 us at 68e6 (256 x 1024, the tree 14.9).
+    // 60 us at 21e6 (100 x 1000), 114 us at 52e6 (64 x 4096, the tree 63); float32 Leg->Cheb
+    // 15.4 us at 31e6 (1000 x 64, the tree 19.4), 19.3 us at 48e6 (4096 x 8, the tree 25.2 and the
+    // FFTs 23.9), 25.6 us at 49e6 (6000 x 4, 24.3), 23.6 us at 63e6 (1000 x 128, 19.9); Jacobi
+    // 17.4 us at 39e6 (1000 x 48, 18.9), 19.4 us at 49e6 (200 x 800, 18.2).
     const double cost = NC * (double)m * (double)((batch + V - 1) / V) *
                         ((V + 1) * (0.5 * (double)m + 16) + 160 * V);
     if (m <= 2 * kHierLeaf) return cost <= (sizeof(T) == 4 ? 14.5e6 : 22e6);
-    return cost <= (sizeof(T) == 4 ? 35e6 : NC == 2 ? 70e6 : 44e6);
+    return cost <= (sizeof(T) == 4 ? (NC == 2 ? 48e6 : 40e6) : NC == 2 ? 70e6 : 44e6);
 }
 
 template <typename T, int NC, int V, int WR>
