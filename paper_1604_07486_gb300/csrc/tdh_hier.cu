@@ -259,6 +259,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_hier_up(co
     constexpr int NL = VW / RPI > 0 ? VW / RPI : 1;    // load instructions per leaf
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (ragged: the lists were written by the previous kernel, and no kernel after this one may
+    // read them before they are there, so the next starts only from here on)
+    if constexpr (RAGGED) pdl_wait();
     pdl_trigger();
     const int ntop = (P.leaves + kHierTopLeaves - 1) / kHierTopLeaves;
     const int top = blockIdx.x % ntop;
@@ -1184,6 +1187,56 @@ __global__ void k_hier_scatter(const int64_t* __restrict__ offs, int64_t batch, 
     if (b >= 0) list[atomicAdd(&hist[b], 1)] = (int)v;
 }
 
+// The same in one launch of one CTA (hist[0 .. bins) unused): each launch of the three and the
+// clearing of their counts costs 2 to 3 us, more than a few thousand vectors do.  Leg->Cheb float32
+// 128 x 512: 24.7 -> 16.9 us, 200 x 512: 31.8 -> 22.1, 512 x 2048: 42.4 -> 33.6 (with one scratch
+// block for lists and tree, and the moments' launch overlapping this one); the FFT classes take
+// 21.7, 23.5 and 45.2.
+constexpr int kSmallSort = 4 * kSortThreads;  // vectors
+__global__ void __launch_bounds__(kSortThreads) k_hier_sort(const int64_t* __restrict__ offs,
+                                                            int batch, int64_t n_max, int unit,
+                                                            int bins, int* __restrict__ hist,
+                                                            int* __restrict__ list, const char* in,
+                                                            const char* out, int esz, int* status) {
+    __shared__ int at[kSortThreads], wsum[kSortThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_trigger();
+    if (ragged_alias(offs, batch, in, out, esz)) {
+        if (tid == 0) {
+            hist[bins] = 0;
+            if (status) atomicOr(status, TDH_STATUS_ALIAS);
+        }
+        return;
+    }
+    at[tid] = 0;
+    __syncthreads();
+    int bin[kSmallSort / kSortThreads], bad = 0;
+#pragma unroll
+    for (int k = 0; k < kSmallSort / kSortThreads; ++k) {
+        const int v = k * kSortThreads + tid;
+        bin[k] = v < batch ? ragged_bin(offs, v, n_max, unit, bins, &bad) : -1;
+        if (bin[k] >= 0) atomicAdd(&at[bin[k]], 1);
+    }
+    if (bad && status) atomicOr(status, TDH_STATUS_LENGTH);
+    __syncthreads();
+    const int x = at[tid];
+    int s = x;
+    for (int k = 1; k < 32; k <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, s, k);
+        if (lane >= k) s += o;
+    }
+    if (lane == 31) wsum[warp] = s;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < warp; ++w) before += wsum[w];
+    at[tid] = before + s - x;
+    if (tid == kSortThreads - 1) hist[bins] = before + s;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSmallSort / kSortThreads; ++k)
+        if (bin[k] >= 0) list[atomicAdd(&at[bin[k]], 1)] = k * kSortThreads + tid;
+}
+
 // ------------------------------------------------------------------------------ host side
 
 double lagrange(const int* x, int P, int i, double at) {
@@ -1356,14 +1409,15 @@ cudaError_t launch_cfg(void (*kern)(const HierParams<T>), unsigned grid, size_t 
 
 template <typename T, int NC, bool RAGGED>
 int launch_up(const HierParams<T>& P, unsigned grid, cudaStream_t s) {
-    auto kern = k_hier_up<T, NC, RAGGED>;  // launched without overlap: its input may be the
-                                           // previous step's output
+    // dense: launched without overlap, as its input may be the previous step's output (ragged: it
+    // waits for the lists, whose kernels are launched without)
+    auto kern = k_hier_up<T, NC, RAGGED>;
     static PerDevice once;
     cudaError_t e = per_device(once, [&](int*) {
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kMaxSmem);
     });
-    if (e == cudaSuccess) e = launch_cfg<T>(kern, grid, up_smem<T>(NC, P.unvt), s, false, P);
+    if (e == cudaSuccess) e = launch_cfg<T>(kern, grid, up_smem<T>(NC, P.unvt), s, RAGGED && P.first == 0, P);
     if (e != cudaSuccess) {
         set_error("hierarchical moments: %s", cudaGetErrorString(e));
         return TDH_ERR_CUDA;
@@ -1502,9 +1556,44 @@ int launch_direct(const HierParams<T>& P, int64_t m, cudaStream_t s) {
     return launch_direct_wr<T, NC, V, 4>(P, m, (unsigned)grid(2), s);
 }
 
+// Lists of a ragged batch, into scr: hist[bins + 1], then list[batch].
+constexpr int kRaggedUnit = 2 * kHierLeaf;  // coefficients of a leaf (two channels)
+
+template <typename T>
+int ragged_lists(const Step& st, const void* in, void* out, const int64_t* offs, int64_t batch,
+                 int bins, int* scr, cudaStream_t s) {
+    int* list = scr + bins + 1;
+    cudaError_t e = cudaSuccess;
+    const unsigned grid = (unsigned)((batch + kThreads - 1) / kThreads);
+    const char* ci = static_cast<const char*>(in);
+    const char* co = static_cast<const char*>(out);
+    if (batch <= kSmallSort && bins <= kSortThreads) {
+        k_hier_sort<<<1, kSortThreads, 0, s>>>(offs, (int)batch, st.n, kRaggedUnit, bins, scr, list,
+                                               ci, co, (int)sizeof(T), st.status);
+        note_launches(1);
+        e = cudaGetLastError();
+    } else {
+        e = cudaMemsetAsync(scr, 0, sizeof(int) * (size_t)(bins + 1), s);
+        if (e == cudaSuccess) {
+            k_hier_hist<<<grid, kThreads, 0, s>>>(offs, batch, st.n, kRaggedUnit, bins, scr, ci, co,
+                                                  (int)sizeof(T), st.status);
+            k_hier_scan<<<1, kSortThreads, 0, s>>>(scr, bins);
+            k_hier_scatter<<<grid, kThreads, 0, s>>>(offs, batch, st.n, kRaggedUnit, bins, scr, list,
+                                                     ci, co, (int)sizeof(T));
+            note_launches(3);
+            e = cudaGetLastError();
+        }
+    }
+    if (e != cudaSuccess) {
+        set_error("ragged lists: %s", cudaGetErrorString(e));
+        return TDH_ERR_CUDA;
+    }
+    return TDH_OK;
+}
+
 template <typename T, int NC, bool RAGGED>
 int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, int64_t batch,
-              int adjoint, const int* list, const int* count, cudaStream_t s) {
+              int adjoint, cudaStream_t s) {
     constexpr int NP = HierP<T>::P;
     const HierData& H = st.hier;
     const int64_t m = (st.n + NC - 1) / NC;
@@ -1590,8 +1679,16 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     chunk = std::min(chunk, (int64_t)INT32_MAX / 4 / std::max<int64_t>(P.runs, ntop));
     chunk = std::max<int64_t>(unit, chunk / unit * unit);
     chunk = std::min<int64_t>(chunk, (batch + unit - 1) / unit * unit);
-    T* mom = nullptr;
-    if (far) TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&mom), (size_t)(per_vec * chunk), s));
+    // one block: the lists of a ragged batch, then the moments and expansions
+    const int bins = RAGGED ? (int)((st.n + kRaggedUnit - 1) / kRaggedUnit) : 0;
+    const size_t head =
+        RAGGED ? (sizeof(int) * (size_t)(bins + 1 + batch) + 255) / 256 * 256 : 0;
+    char* scr = nullptr;
+    if (RAGGED || far)
+        TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&scr),
+                              head + (far ? (size_t)(per_vec * chunk) : 0), s));
+    const int* list = reinterpret_cast<const int*>(scr) + bins + 1;
+    T* mom = far ? reinterpret_cast<T*>(scr + head) : nullptr;
     P.bpad = chunk;
     for (int l = 0; l < kHierLevels; ++l) {
         P.mom[l] = mom;
@@ -1600,6 +1697,8 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     P.loc = mom;
     P.top = top ? mom + boxes[0] * NC * NP * chunk : nullptr;
     int rc = TDH_OK;
+    if constexpr (RAGGED)
+        rc = ragged_lists<T>(st, in, out, offs, batch, bins, reinterpret_cast<int*>(scr), s);
     for (int64_t b0 = 0; rc == TDH_OK && b0 < batch; b0 += chunk) {
         const int64_t nb = std::min(chunk, batch - b0);
         P.batch = nb;
@@ -1609,7 +1708,7 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
             P.offs = offs;
             P.list = list + b0;
             P.first = b0;
-            P.count = count;
+            P.count = list - 1;
         } else {
             P.in += b0 * st.n;
             P.out += b0 * st.n;
@@ -1629,38 +1728,6 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         }
         if (rc == TDH_OK) rc = launch_near<T, NC, RAGGED>(P, NV, nb, far, s);
     }
-    if (far) scratch_free(P.mom[0], s);
-    return rc;
-}
-
-template <typename T>
-int ragged_typed(const Step& st, const void* in, void* out, const int64_t* offs, int64_t batch,
-                 cudaStream_t s) {
-    const int unit = 2 * kHierLeaf;
-    const int bins = (int)((st.n + unit - 1) / unit);
-    int* scr = nullptr;  // hist[bins + 1], list[batch]
-    TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&scr), sizeof(int) * (size_t)(bins + 1 + batch), s));
-    int* list = scr + bins + 1;
-    int rc = TDH_OK;
-    cudaError_t e = cudaMemsetAsync(scr, 0, sizeof(int) * (size_t)(bins + 1), s);
-    const unsigned grid = (unsigned)((batch + kThreads - 1) / kThreads);
-    const char* ci = static_cast<const char*>(in);
-    const char* co = static_cast<const char*>(out);
-    if (e == cudaSuccess) {
-        k_hier_hist<<<grid, kThreads, 0, s>>>(offs, batch, st.n, unit, bins, scr, ci, co,
-                                              (int)sizeof(T), st.status);
-        k_hier_scan<<<1, kSortThreads, 0, s>>>(scr, bins);
-        k_hier_scatter<<<grid, kThreads, 0, s>>>(offs, batch, st.n, unit, bins, scr, list, ci, co,
-                                                 (int)sizeof(T));
-        note_launches(3);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) {
-        set_error("ragged lists: %s", cudaGetErrorString(e));
-        rc = TDH_ERR_CUDA;
-    }
-    if (rc == TDH_OK)
-        rc = run_typed<T, 2, true>(st, in, out, offs, batch, 0, list, scr + bins, s);
     scratch_free(scr, s);
     return rc;
 }
@@ -1686,20 +1753,16 @@ void hier_release(HierData& h) {
 int hier_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
                 cudaStream_t s) {
     if (prec != TDH_FP64)
-        return st.full ? run_typed<float, 1, false>(st, in, out, nullptr, batch, adjoint, nullptr,
-                                                    nullptr, s)
-                       : run_typed<float, 2, false>(st, in, out, nullptr, batch, adjoint, nullptr,
-                                                    nullptr, s);
-    return st.full ? run_typed<double, 1, false>(st, in, out, nullptr, batch, adjoint, nullptr,
-                                                 nullptr, s)
-                   : run_typed<double, 2, false>(st, in, out, nullptr, batch, adjoint, nullptr,
-                                                 nullptr, s);
+        return st.full ? run_typed<float, 1, false>(st, in, out, nullptr, batch, adjoint, s)
+                       : run_typed<float, 2, false>(st, in, out, nullptr, batch, adjoint, s);
+    return st.full ? run_typed<double, 1, false>(st, in, out, nullptr, batch, adjoint, s)
+                   : run_typed<double, 2, false>(st, in, out, nullptr, batch, adjoint, s);
 }
 
 int hier_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s) {
-    return prec != TDH_FP64 ? ragged_typed<float>(st, in, out, offs, batch, s)
-                            : ragged_typed<double>(st, in, out, offs, batch, s);
+    return prec != TDH_FP64 ? run_typed<float, 2, true>(st, in, out, offs, batch, 0, s)
+                            : run_typed<double, 2, true>(st, in, out, offs, batch, 0, s);
 }
 
 }  // namespace tdh

@@ -71,3 +71,47 @@ def test_autotune_that_fails_leaves_the_plan_usable(tdh, n, prec):
         assert plan.status() == set()
         plan.close()
     assert failed >= 20
+
+
+@pytest.mark.parametrize("n", [1, 64, 128, 129, 256, 257, 512, 513, 3000])
+@pytest.mark.parametrize("kind", ["leg2cheb", "cheb2leg"])
+def test_small_ragged_calls(tdh, kind, n):
+    """Float32 ragged calls on both sides of the one-launch sort's limit (4096 vectors) agree with
+    the oracle and take no more launches than they need."""
+    import torch
+    okind = oracle.LEG2CHEB if kind == "leg2cheb" else oracle.CHEB2LEG
+    plan = tdh.Plan(kind, n, prec="fp32", ragged=True)
+    for batch in (1, 9, 4096, 4097):
+        lengths = np.random.default_rng(batch).integers(0, n + 1, batch)
+        lengths[0] = n
+        x, offs = workloads.ragged_coefficients(lengths, decay=0.5, seed=n)
+        xt, ot = torch.tensor(x, dtype=torch.float32, device="cuda"), torch.tensor(offs, device="cuda")
+        c0 = tdh.launch_count()
+        y = plan.execute_ragged(xt, ot).double().cpu().numpy()
+        launches = tdh.launch_count() - c0
+        far = 3 if n > 128 else 1  # moments, far and near field, or the near field alone
+        assert launches == (1 if batch <= 4096 else 3) + far, (batch, launches)
+        for v in np.r_[0:min(batch, 40), batch - 1]:
+            a, b = int(offs[v]), int(offs[v + 1])
+            if b > a:
+                ref = oracle.matvec(okind, None, x[a:b])
+                assert np.abs(y[a:b] - ref).max() <= TOL["fp32"] * np.abs(x[a:b]).sum()
+    assert plan.status() == set()
+
+
+def test_small_ragged_calls_report_bad_input(tdh):
+    """The one-launch sort records what the three launches do: vectors out of range are left
+    unwritten (LENGTH), overlapping input and output convert nothing (ALIAS)."""
+    import torch
+    n = 64
+    plan = tdh.Plan("leg2cheb", n, prec="fp32", ragged=True)
+    offs = torch.tensor([0, 64, 200, 190, 254], device="cuda")  # too long; decreasing
+    x = torch.randn(300, device="cuda")
+    y = torch.full_like(x, -7.0)
+    plan.execute_ragged(x, offs, out=y)
+    assert plan.status() == {"LENGTH"}
+    assert (y[64:190] == -7).all() and (y[:64] != -7).all() and (y[190:254] != -7).all()
+    buf = torch.randn(400, device="cuda")
+    keep = buf.clone()
+    plan.execute_ragged(buf[:300], torch.tensor([0, 64, 128], device="cuda"), out=buf[32:332])
+    assert plan.status() == {"ALIAS"} and torch.equal(buf, keep)
