@@ -750,9 +750,8 @@ int tdh_plan_create(int kind, int64_t n_max, const tdh_params* params, double to
             rc = TDH_ERR_UNSUPPORTED;
         } else {
             rc = exec_prepare_ragged(plan->steps[0], params->prec);
-            // (split bfloat16: the stall hook's FFTs; short float64 plans: their few-vector batches)
-            if (rc == TDH_OK && (!plan->steps[0].hier.use_ragged || params->prec == TDH_BF16X3 ||
-                                 (params->prec == TDH_FP64 && plan->steps[0].n <= kRaggedFftLen)))
+            // (split bfloat16: the stall hook's FFTs)
+            if (rc == TDH_OK && (!plan->steps[0].hier.use_ragged || params->prec == TDH_BF16X3))
                 rc = exec_build(plan->steps[0], params->prec, s);
         }
         const size_t ncls = plan->steps.empty() ? 0 : plan->steps[0].rcls.size();

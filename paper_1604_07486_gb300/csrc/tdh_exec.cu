@@ -725,10 +725,7 @@ static int require_built(const ExecData& ex) {
 int exec_launch_ragged(const Step& st, int prec, const void* in, void* out, const int64_t* offs,
                        int64_t batch, cudaStream_t s, const std::vector<cudaStream_t>& side,
                        const std::vector<cudaEvent_t>& ev) {
-    // A few short float64 vectors: the tree's latency (125 to 190 us, whatever the lengths) is
-    // longer than the FFTs take (41 us at 1024 x 2, 128 us at 4000 x 4; 270 us at 8000 x 4).
-    const bool few = prec == TDH_FP64 && st.n <= kRaggedFftLen && st.n * batch <= 32768;
-    if (st.hier.use_ragged && !few && !tc_stalled(st))
+    if (st.hier.use_ragged && !tc_stalled(st))
         return hier_launch_ragged(st, prec, in, out, offs, batch, s);
     for (const ExecData& ex : st.rcls) TDH_TRY(require_built(ex));
     if (prec != TDH_FP64) return launch_ragged_typed<float>(st, in, out, offs, batch, s, side, ev);

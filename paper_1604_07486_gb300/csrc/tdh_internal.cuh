@@ -248,7 +248,6 @@ int exec_diagonals(Step& st, int prec, cudaStream_t s);
 // The tables of its FFT configurations (spectrum, twiddles, factors) that are not there yet:
 // at creation for steps that run their FFTs, else when a schedule is asked for.
 int exec_build(Step& st, int prec, cudaStream_t s);
-constexpr int64_t kRaggedFftLen = 4096;  // float64 ragged plans up to it keep their FFTs at hand
 void exec_release(ExecData& ex);
 // Configurations for every FFT length a ragged batch of vectors up to st.n can need.
 int exec_prepare_ragged(Step& st, int prec);

@@ -75,17 +75,18 @@ def test_autotune_that_fails_leaves_the_plan_usable(tdh, n, prec):
 
 @pytest.mark.parametrize("n", [1, 64, 128, 129, 256, 257, 512, 513, 3000])
 @pytest.mark.parametrize("kind", ["leg2cheb", "cheb2leg"])
-def test_small_ragged_calls(tdh, kind, n):
-    """Float32 ragged calls on both sides of the one-launch sort's limit (4096 vectors) agree with
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_small_ragged_calls(tdh, prec, kind, n):
+    """Ragged calls on both sides of the one-launch sort's limit (4096 vectors) agree with
     the oracle and take no more launches than they need."""
     import torch
     okind = oracle.LEG2CHEB if kind == "leg2cheb" else oracle.CHEB2LEG
-    plan = tdh.Plan(kind, n, prec="fp32", ragged=True)
+    plan = tdh.Plan(kind, n, prec=prec, ragged=True)
     for batch in (1, 9, 4096, 4097):
         lengths = np.random.default_rng(batch).integers(0, n + 1, batch)
         lengths[0] = n
         x, offs = workloads.ragged_coefficients(lengths, decay=0.5, seed=n)
-        xt, ot = torch.tensor(x, dtype=torch.float32, device="cuda"), torch.tensor(offs, device="cuda")
+        xt, ot = torch.tensor(x, dtype=plan.dtype, device="cuda"), torch.tensor(offs, device="cuda")
         c0 = tdh.launch_count()
         y = plan.execute_ragged(xt, ot).double().cpu().numpy()
         launches = tdh.launch_count() - c0
@@ -95,7 +96,7 @@ def test_small_ragged_calls(tdh, kind, n):
             a, b = int(offs[v]), int(offs[v + 1])
             if b > a:
                 ref = oracle.matvec(okind, None, x[a:b])
-                assert np.abs(y[a:b] - ref).max() <= TOL["fp32"] * np.abs(x[a:b]).sum()
+                assert np.abs(y[a:b] - ref).max() <= TOL[prec] * np.abs(x[a:b]).sum()
     assert plan.status() == set()
 
 
