@@ -8,7 +8,8 @@
  * D1 sum_r D_{u_r} T D_{u_r} D2 alpha with u_r = l_r / sqrt(a_r) (Eq. (5)),
  * each Toeplitz product by zero-padded FFTs of length about 2N (Sec. 1).
  * T o H itself is also smooth away from the diagonal, and executes use that instead where it
- * holds (every conversion but Laguerre changes of one or more): its far blocks by interpolation
+ * holds (every conversion but Laguerre changes of one or more, in float64 of any size, and in
+ * float32 up to 4096 coefficients): its far blocks by interpolation
  * in a tree of boxes, its near ones entry by entry, in O(N) operations and without a truncation
  * (the hierarchical product).  The FFT form runs any plan whose FFT schedule is asked for
  * (tdh_plan_set_schedule) or found the faster one (tdh_plan_autotune).

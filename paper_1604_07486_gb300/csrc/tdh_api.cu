@@ -179,10 +179,17 @@ constexpr size_t kKeepBytes = (size_t)64 << 20;
 // Steps whose T and H are smooth away from the diagonal, as the hierarchical product needs: every
 // T o H step of a parameter change below one (Cases 2 and 3), and Legendre / Chebyshev.  A
 // Laguerre change beyond that has a Toeplitz part that alternates or ends.
-bool hier_serves(const Step& st) {
+//
+// Laguerre's H is all ones, so its FFT form is one FFT pair instead of K of them.  In float64 the
+// FFTs stay: T falls off slowly, so what the interpolation leaves out is not far below the result
+// (relative error 1.5e-14 at n = 9001, a -> a - 1/2, FFTs 5e-16).  In float32 the tree takes over
+// where the FFT no longer fits one CTA (5000 x 64: 21.8 us, FFTs 33.7; 65536 x 64: 61 and 179;
+// below it 4096 x 64: 21.6 and 15.0, 500 x 256: 17.8 and 11.0).  Split bfloat16: the tree always
+// (64 x 16: 9.8 us, tensor-core FFTs 27; 1024 x 64: 17.6 and 31.5; 4096 x 4096: 180 and 394).
+bool hier_serves(const Step& st, int prec) {
     if (st.kind != TDH_LAG2LAG) return true;
-    const double d = st.p[0] - st.p[1];
-    return std::fabs(d) < 1.0;
+    if (!(std::fabs(st.p[0] - st.p[1]) < 1.0) || prec == TDH_FP64) return false;
+    return prec == TDH_BF16X3 || st.n > 4096;
 }
 
 int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStream_t s) {
@@ -193,7 +200,7 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
     // Whatever the precision and the length: split-bfloat16 plans' tensor-core FFTs take 28 us at
     // n = 512 x 16 and 3267 us at 65536 x 256, the float32 hierarchical product 9.4 and 161 us with
     // smaller errors.  Their FFT tables are built with the plan all the same (tdh_test_tc_stall).
-    const bool hier = hier_serves(st);
+    const bool hier = hier_serves(st, prec);
     const int64_t ns = hier ? hier_length(st) : n;
     TDH_TRY(dev_alloc_t(&st.t, ns));
     TDH_TRY(dev_alloc_t(&st.h, 2 * ns - 1));

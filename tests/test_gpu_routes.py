@@ -116,3 +116,26 @@ def test_small_ragged_calls_report_bad_input(tdh):
     keep = buf.clone()
     plan.execute_ragged(buf[:300], torch.tensor([0, 64, 128], device="cuda"), out=buf[32:332])
     assert plan.status() == {"ALIAS"} and torch.equal(buf, keep)
+
+
+def test_laguerre_route_and_accuracy(tdh):
+    """Laguerre changes below one: one FFT pair where that is the faster or the more exact form
+    (float32 up to 4096 coefficients, float64), the tree beyond.  Float64 FFT errors are at most
+    64 roundings of the result in the norm (an FFT pair of 2^15 points rounds about 2 log2 L u);
+    the interpolation's are 2e-14 and would not pass."""
+    import torch
+    for n, prec, launches in ((4096, "fp32", 1), (4097, "fp32", 3), (4096, "bf16x3", 3)):
+        plan = tdh.Plan("lag2lag", n, prec=prec, params=(0.3, -0.2))
+        x = torch.randn(64, n, dtype=plan.dtype, device="cuda")
+        c0 = tdh.launch_count()
+        plan.execute(x)
+        assert tdh.launch_count() - c0 == launches, (n, prec)
+    n = 9001
+    rows = np.unique(np.r_[0:64, np.random.default_rng(0).integers(0, n, 300), n - 64:n])
+    x = np.random.default_rng(3).standard_normal((2, n))
+    for params in ((0.3, -0.2), (100.5, 100.1), (0.5, 0.25)):
+        plan = tdh.Plan("lag2lag", n, prec="fp64", params=params)
+        for fn, tr in ((plan.execute, False), (plan.adjoint, True)):
+            y = fn(torch.tensor(x, device="cuda")).cpu().numpy()[:, rows]
+            ref = oracle.matvec(oracle.LAG, params, x, rows=rows, transpose=tr)
+            assert np.linalg.norm(y - ref) <= 64 * 2.0 ** -53 * np.linalg.norm(ref), (params, tr)
