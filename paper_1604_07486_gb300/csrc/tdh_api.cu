@@ -287,6 +287,8 @@ bool overlaps(const void* a, const void* b, size_t bytes) {
     return x < y + bytes && y < x + bytes;
 }
 
+constexpr size_t kChainBytes = (size_t)1 << 30;  // scratch of a chain's chunk of vectors
+
 int run(tdh_plan_t plan, const void* in, void* out, int64_t batch, void* stream, int adjoint) {
     clear_error();
     if (!plan) {
@@ -329,32 +331,55 @@ int run(tdh_plan_t plan, const void* in, void* out, int64_t batch, void* stream,
     auto wide_after = [&](size_t i) {
         return i + 1 < nsteps && step(i).sp_sums == 2 && step(i + 1).sp_sums == 2;
     };
-    bool need_tmp = false, need_wide = false;
-    int flips = 0;  // buffer changes still ahead: step i writes `out` when they are even
+    bool need_wide = false, mid = false;
+    int changes = 0;  // buffer changes: step i writes `out` when those still ahead are even
     for (size_t i = 0; i < nsteps; ++i) {
-        if (i > 0 && distinct(i)) ++flips;
+        if (i > 0 && distinct(i)) ++changes;
         need_wide = need_wide || wide_after(i);
+        mid = mid || step(i).sp_sums == 2;  // pairs of floats between the step's own factors
+        if (step(i).sp_M > 0) TDH_TRY(sparse_check(step(i), plan->params.prec, batch, i > 0));
     }
-    need_tmp = flips > 0;
-    char* scratch = nullptr;
-    const size_t tmp_bytes = need_tmp ? (bytes + 255) / 256 * 256 : 0;
-    if (need_tmp || need_wide)
-        TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&scratch),
-                              tmp_bytes + (need_wide ? 2 * bytes : 0), s));
-    const void* src = in;
-    int rc = TDH_OK;
-    for (size_t i = 0; rc == TDH_OK && i < nsteps; ++i) {
-        if (i > 0 && distinct(i)) --flips;
-        const Step& st = step(i);
-        const bool win = i > 0 && wide_after(i - 1), wout = wide_after(i);
-        void* dst = wout ? scratch + tmp_bytes : flips % 2 ? scratch : out;
-        rc = st.sp_M > 0 ? sparse_launch(st, plan->params.prec, src, dst, batch, adjoint, win,
-                                         wout, s)
-                         : exec_launch(st, plan->params.prec, src, dst, batch, adjoint, s);
-        src = dst;
+    // Scratch per vector: the alternate buffer, and the pairs of floats between steps and within
+    // one.  Vectors are independent, so a batch that would take more than kChainBytes of it goes
+    // through the whole chain in chunks (whole multiples of 16 bytes), smaller ones if even that
+    // cannot be had.
+    const size_t vec_bytes = esz * (size_t)plan->n_max;
+    const size_t per_vec = vec_bytes * ((changes > 0) + 2 * (need_wide + mid));
+    const int64_t group = (int64_t)(16 / esz);
+    int64_t chunk = batch;
+    if (per_vec > 0 && kChainBytes / per_vec < (size_t)batch)
+        chunk = std::max<int64_t>(group, (int64_t)(kChainBytes / per_vec) / group * group);
+    int64_t b0 = 0;
+    for (;;) {
+        const size_t chunk_bytes = vec_bytes * (size_t)chunk;
+        const size_t tmp_bytes = changes > 0 ? (chunk_bytes + 255) / 256 * 256 : 0;
+        char* scratch = nullptr;
+        int rc = TDH_OK;
+        if (changes > 0 || need_wide)
+            rc = scratch_alloc(reinterpret_cast<void**>(&scratch),
+                               tmp_bytes + (need_wide ? 2 * chunk_bytes : 0), s);
+        while (rc == TDH_OK && b0 < batch) {
+            const int64_t nb = std::min(chunk, batch - b0);
+            const void* src = static_cast<const char*>(in) + vec_bytes * (size_t)b0;
+            char* res = static_cast<char*>(out) + vec_bytes * (size_t)b0;
+            int ahead = changes;
+            for (size_t i = 0; rc == TDH_OK && i < nsteps; ++i) {
+                if (i > 0 && distinct(i)) --ahead;
+                const Step& st = step(i);
+                const bool win = i > 0 && wide_after(i - 1), wout = wide_after(i);
+                void* dst = wout ? scratch + tmp_bytes : ahead % 2 ? scratch : res;
+                rc = st.sp_M > 0 ? sparse_launch(st, plan->params.prec, src, dst, nb, adjoint, win,
+                                                 wout, s)
+                                 : exec_launch(st, plan->params.prec, src, dst, nb, adjoint, s);
+                src = dst;
+            }
+            if (rc == TDH_OK) b0 += nb;
+        }
+        if (scratch) scratch_free(scratch, s);
+        if (rc != TDH_ERR_NOMEM || chunk <= group || per_vec * (size_t)chunk <= kLeastScratch)
+            return rc;
+        chunk = std::max<int64_t>(group, std::min(chunk, batch) / 2 / group * group);
     }
-    if (scratch) scratch_free(scratch, s);
-    return rc;
 }
 
 // Host buffers: the batch goes through the device in chunks, two device slots each way, so

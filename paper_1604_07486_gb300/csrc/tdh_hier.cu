@@ -1685,8 +1685,15 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
         RAGGED ? (sizeof(int) * (size_t)(bins + 1 + batch) + 255) / 256 * 256 : 0;
     char* scr = nullptr;
     if (RAGGED || far)
-        TDH_TRY(scratch_alloc(reinterpret_cast<void**>(&scr),
-                              head + (far ? (size_t)(per_vec * chunk) : 0), s));
+        for (;;) {  // (fewer vectors at a time where memory is short)
+            const int rc = scratch_alloc(reinterpret_cast<void**>(&scr),
+                                         head + (far ? (size_t)(per_vec * chunk) : 0), s);
+            if (rc == TDH_OK) break;
+            if (rc != TDH_ERR_NOMEM || !far || chunk <= unit ||
+                (size_t)(per_vec * chunk) <= kLeastScratch)
+                return rc;
+            chunk = std::max<int64_t>(unit, chunk / 2 / unit * unit);
+        }
     const int* list = reinterpret_cast<const int*>(scr) + bins + 1;
     T* mom = far ? reinterpret_cast<T*>(scr + head) : nullptr;
     P.bpad = chunk;

@@ -102,6 +102,10 @@ int pchol_weights(const double* t, const double* d1, const double* d2, const dou
                   double* tmax, cudaStream_t s);
 int pchol_unweight(double* u, const double* w, int64_t K, int64_t n, cudaStream_t s);
 
+// A call that runs short of scratch goes on with fewer vectors at a time while the block it asked
+// for is larger than this.
+constexpr size_t kLeastScratch = (size_t)16 << 20;
+
 // ----------------------------------------------------------------------------- a3-a7
 // FFT geometry of one execute configuration: L = C * LC points, local radix R.
 struct Geometry {
@@ -234,7 +238,9 @@ namespace tdh {
 // the factors (or of their inverses) applied to in, or its transpose; in == out allowed.
 enum { SP_ULTRA = 0, SP_JACOBI = 1, SP_IDENTITY = 2 };
 int sparse_prepare(Step& st, int prec, cudaStream_t s);
-// wide_in / wide_out (steps with sp_sums == 2 only): in / out hold pairs of floats.
+// wide_in / wide_out (steps with sp_sums == 2 only): in / out hold pairs of floats.  sparse_check
+// says whether the step takes a batch (inplace: it may run in place), however it is cut up.
+int sparse_check(const Step& st, int prec, int64_t batch, bool inplace);
 int sparse_launch(const Step& st, int prec, const void* in, void* out, int64_t batch, int adjoint,
                   bool wide_in, bool wide_out, cudaStream_t s);
 // out[j] = Gamma(j + a) / Gamma(j + b), j < count, float64 device array.

@@ -868,10 +868,6 @@ int forward_typed(const Step& st, const void* in, void* out, int64_t batch, int 
         return TDH_OK;
     }
     const int64_t ntiles = (n + kTile - 1) / kTile;
-    if (batch * ntiles > INT32_MAX) {
-        set_error("sparse factors: batch * tiles above 2^31");
-        return TDH_ERR_UNSUPPORTED;
-    }
     const int H = OFF * st.sp_M;
     T* halo = nullptr;
     if (inplace) {
@@ -896,10 +892,6 @@ int inverse_typed(const Step& st, const void* in, void* out, int64_t batch, int 
                   cudaStream_t s) {
     const int64_t n = st.n;
     const int64_t ntiles = (n + Scan<T>::tile - 1) / Scan<T>::tile;
-    if (batch * ntiles > INT32_MAX || batch > INT32_MAX) {
-        set_error("back-substitution: batch * tiles above 2^31");
-        return TDH_ERR_UNSUPPORTED;
-    }
     using A = Aff<T, OFF>;
     constexpr size_t smem = 3 * sizeof(T) * (size_t)Scan<T>::smem;
     static PerDevice attr_once;
@@ -957,10 +949,6 @@ template <typename A, typename TI, typename TO, typename M, int OFF, bool REV, b
 int sums_typed(const Step& st, const void* in, void* out, int64_t batch, cudaStream_t s) {
     using S = ChainSum<A, OFF>;
     const int64_t n = st.n, ntiles = (n + SumTile<A>::tile - 1) / SumTile<A>::tile;
-    if (batch * ntiles > INT32_MAX) {
-        set_error("back-substitution: batch * tiles above 2^31");
-        return TDH_ERR_UNSUPPORTED;
-    }
     const unsigned grid = (unsigned)(batch * ntiles);
     // two sets of tile sums: a factor reads one while it writes the next factor's
     const size_t sum_bytes = (sizeof(S) * 2 * (size_t)grid + 255) / 256 * 256;
@@ -1162,6 +1150,27 @@ int sparse_prepare(Step& st, int prec, cudaStream_t s) {
         k_sparse_tables<double><<<blocks, kThreads, 0, s>>>(F, st.scale_out, st.scale_in,
                                                             static_cast<double*>(st.sp_tab));
     TDH_CUDA(cudaGetLastError());
+    return TDH_OK;
+}
+
+int sparse_check(const Step& st, int prec, int64_t batch, bool inplace) {
+    static_assert(SumTile<float>::tile == Scan<float>::tile &&
+                      SumTile<FF>::tile == Scan<float>::tile &&
+                      SumTile<double>::tile == Scan<double>::tile,
+                  "sums and affine scans take the same batches");
+    if (!st.sp_inverse) {
+        const bool whole = prec != TDH_FP64 && st.sp_M == 1 && st.n % 4 == 0 && !inplace;
+        if (!whole && batch * ((st.n + kTile - 1) / kTile) > INT32_MAX) {
+            set_error("sparse factors: batch * tiles above 2^31");
+            return TDH_ERR_UNSUPPORTED;
+        }
+        return TDH_OK;
+    }
+    const int64_t tile = prec != TDH_FP64 ? Scan<float>::tile : Scan<double>::tile;
+    if (batch * ((st.n + tile - 1) / tile) > INT32_MAX) {
+        set_error("back-substitution: batch * tiles above 2^31");
+        return TDH_ERR_UNSUPPORTED;
+    }
     return TDH_OK;
 }
 

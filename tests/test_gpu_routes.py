@@ -139,3 +139,44 @@ def test_laguerre_route_and_accuracy(tdh):
             y = fn(torch.tensor(x, device="cuda")).cpu().numpy()[:, rows]
             ref = oracle.matvec(oracle.LAG, params, x, rows=rows, transpose=tr)
             assert np.linalg.norm(y - ref) <= 64 * 2.0 ** -53 * np.linalg.norm(ref), (params, tr)
+
+
+def test_chain_scratch_is_bounded(tdh):
+    """Float32 chains take at most about 1 GB of scratch however large the batch (the pairs of floats
+    between two inverse factors of 512 x 2^20 would take 4 GB), and cut batches give what whole
+    ones do: every vector's sums are its own, bit for bit."""
+    import torch
+    n, batch = 1 << 20, 512
+    plan = tdh.Plan("ultra2ultra", n, prec="fp32", params=(2.25, 0.25))
+    x = torch.randn(batch, n, device="cuda")
+    y = torch.empty_like(x)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    for fn in (plan.execute, plan.adjoint):
+        fn(x, out=y)
+        torch.cuda.synchronize()
+        assert free0 - torch.cuda.mem_get_info()[0] <= 3 << 29
+        for v in (0, 127, 128, 300, batch - 1):
+            assert torch.equal(fn(x[v:v + 1]), y[v:v + 1]), v
+
+
+@pytest.mark.parametrize("kind,params", [("jac2jac", (0.1, -0.3, 0.6, 0.2)),
+                                         ("jac2jac", (2.5, 1.25, -0.3, -0.4)),
+                                         ("leg2cheb", ())])
+def test_executes_get_by_with_less_scratch(tdh, kind, params):
+    """A scratch allocation that fails is tried again with fewer vectors at a time: chains (before:
+    in place) and the tree both still convert the batch."""
+    import torch
+    n, batch = 5000, 3000
+    plan = tdh.Plan(kind, n, prec="fp32", params=params)
+    x = torch.randn(batch, n, device="cuda") / torch.arange(1, n + 1, device="cuda")
+    ref = plan.execute(x), plan.adjoint(x)
+    for k in (1, 2, 3):
+        for fn, r in zip((plan.execute, plan.adjoint), ref):
+            tdh.inject_alloc_failure(k)
+            y = fn(x)
+            tdh.inject_alloc_failure(0)
+            scale = r.abs().amax(1) + x.abs().sum(1)
+            assert float(((y - r).abs().amax(1) / scale).max()) <= 2 * TOL["fp32"], k
+    torch.cuda.synchronize()
+    assert tdh.alloc_stats()[2] == 0
