@@ -176,6 +176,7 @@ struct Step {
     int sp_alone = 0;      // the plan's only step, one factor
     int sp_sums = 0;       // inverses: 0 affine scans, 1 weighted prefix sums, 2 the same in pairs
                            // of floats (float32 chains)
+    float sp_gain[16] = {};  // sums: power of two that the transpose takes off W, per factor
     int sp_flip = 0;       // Jacobi: factors conjugated by diag((-1)^k) (reflected frame)
     double sp_par0 = 0;    // parameter of the first factor (l, or a of S_(a,b))
     double sp_dir = 1;     // parameter change from one factor to the next (+1 or -1)

@@ -525,12 +525,17 @@ __global__ void __launch_bounds__(kThreads) k_scan_solve(const T* in, T* out, in
 //   x_j = W_j sum_{i >= j, i = j mod off} U_i c_i,   U = rho / W,
 // (and its transpose x_i = U_i sum_{j <= i} W_j g_j): a plain sum per chain between two
 // products, where the affine scan above carries a multiplier.  W and U are closed forms:
-//   ultraspherical  W_j = l + j,                                    U_j = 1 / (p_j W_j);
+//   ultraspherical  W_j = (l + j) / l,                              U_j = 1 / (p_j W_j) = 1;
 //   Jacobi          W_j = (2j+s+1) Gamma(j+s+1) / Gamma(j+b+1),     U_j = 1 / (p_j W_j),  s = a+b
-// (W_0 = mu_0 W_1), scaled so that both stay near 1 in the middle of their range; signs of a
-// flipped factor and the diagonal scalings fold into them.  Taken where ln W spans at most
-// kSumRange, so that products with ordinary inputs neither overflow nor vanish in float32; the
-// affine scan stays for larger parameters.
+// (W_0 = mu_0 W_1), scaled so that the smallest W is 1; signs of a flipped factor and the diagonal
+// scalings fold into them.  A suffix sum is then x_j / W_j <= x_j, a term U_i c_i the difference of
+// two of them, so nothing overflows before the result does (times two).  In the transpose the
+// prefix sums are x_i / U_i, so there W comes down, and U goes up, by a power of two (sp_gain) that
+// makes the smallest U about 1.  U falls to about 1 / W:
+// terms below the type's least normal value lose digits that only matter to results as small,
+// so they are taken where ln W spans at most sum_range (float32: 24, full precision down to inputs
+// of 2^-91; parameters a below 0.7 at n = 2^20, 1.1 at 2^16), and the affine scan stays for larger
+// parameters.  (Ultraspherical: any range.)
 //
 // Precision.  A single factor sums in its own precision (log2 n roundings per sum instead of n).
 // Float32 chains of several factors or steps amplify what one inverse leaves behind (a factor
@@ -543,7 +548,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_solve(const T* in, T* out, in
 // factor needs.  16 x 2^20 float32, C^(1.25) -> C^(0.25): 46 us against 140 us for the three
 // kernels of the affine scan (a plain copy of the batch: 20 us); two factors in pairs of
 // floats, C^(2.25) -> C^(0.25): 216 against 277 us.
-constexpr double kSumRange = 40.0;
+constexpr double sum_range(int prec) { return prec == TDH_FP64 ? 40.0 : 24.0; }
 constexpr int kSumChunks = 4;  // pieces per thread
 
 // A pair of floats h + l, |l| <= ulp(h) / 2 (Dekker 1971; Knuth's two-sum).
@@ -581,6 +586,10 @@ __device__ __forceinline__ void from_double(FF& o, double v) {
     o.h = (float)v;
     o.l = isfinite(o.h) ? (float)(v - (double)o.h) : 0.0f;
 }
+// v times a power of two
+__device__ __forceinline__ float scaled(float v, float g) { return v * g; }
+__device__ __forceinline__ double scaled(double v, float g) { return v * (double)g; }
+__device__ __forceinline__ FF scaled(FF v, float g) { return FF{v.h * g, v.l * g}; }
 template <bool DOWN, typename A>
 __device__ __forceinline__ A shfl_by(A v, int d) {
     if constexpr (std::is_same<A, FF>::value)
@@ -667,11 +676,12 @@ __device__ __forceinline__ ChainSum<A, OFF> block_sum(ChainSum<A, OFF> x, ChainS
     return t;
 }
 
-// sum[v ntiles + t]: per chain (j mod OFF), the sum of weight_j in_j over tile t.
-template <typename A, typename TI, int OFF, bool ALIGNED>
+// sum[v ntiles + t]: per chain (j mod OFF), the sum of weight_j in_j over tile t (GAIN: the weights
+// times gain).
+template <typename A, typename TI, int OFF, bool GAIN, bool ALIGNED>
 __global__ void __launch_bounds__(kThreads) k_sum_tiles(const TI* __restrict__ in, int64_t n,
                                                         int64_t ntiles,
-                                                        const A* __restrict__ weight,
+                                                        const A* __restrict__ weight, float gain,
                                                         ChainSum<A, OFF>* __restrict__ sum) {
     constexpr int V = SumTile<A>::V;
     __shared__ ChainSum<A, OFF> red[kThreads / 32];
@@ -690,7 +700,10 @@ __global__ void __launch_bounds__(kThreads) k_sum_tiles(const TI* __restrict__ i
 #pragma unroll
     for (int k = 0; k < kSumChunks; ++k)
 #pragma unroll
-        for (int i = 0; i < V; ++i) s.v[i % OFF] = add(s.v[i % OFF], mul(wv[k][i], xv[k][i]));
+        for (int i = 0; i < V; ++i) {
+            const A w = GAIN ? scaled(wv[k][i], gain) : wv[k][i];
+            s.v[i % OFF] = add(s.v[i % OFF], mul(w, xv[k][i]));
+        }
     s = block_sum<A, OFF>(s, red);
     if (threadIdx.x == 0) sum[blockIdx.x] = s;
 }
@@ -699,13 +712,15 @@ __global__ void __launch_bounds__(kThreads) k_sum_tiles(const TI* __restrict__ i
 // given, the tile sums of next_j out_j.  The block's carry is the sum of the tiles after (before)
 // its own, added in a fixed order.  In place allowed: a block reads its tile before writing it.
 // `first`: the input is older than the previous kernel, so it may be read before waiting for it.
+// gain, next_gain: the transpose's powers of two on win and next (wout's is 1 / gain).
 template <typename A, typename TI, typename TO, int OFF, bool REV, bool ALIGNED>
 __global__ void __launch_bounds__(kThreads) k_sum_solve(const TI* in, TO* out, int64_t n,
                                                         int64_t ntiles, const A* __restrict__ win,
                                                         const A* __restrict__ wout,
                                                         const ChainSum<A, OFF>* sum,
                                                         const A* __restrict__ next,
-                                                        ChainSum<A, OFF>* next_sum, int first) {
+                                                        ChainSum<A, OFF>* next_sum, int first,
+                                                        float gain, float next_gain) {
     constexpr int V = SumTile<A>::V;
     constexpr int NW = kThreads / 32;
     __shared__ ChainSum<A, OFF> red[NW], part[kSumChunks * NW];
@@ -728,7 +743,8 @@ __global__ void __launch_bounds__(kThreads) k_sum_solve(const TI* in, TO* out, i
 #pragma unroll
         for (int k = 0; k < kSumChunks; ++k) {
 #pragma unroll
-            for (int i = 0; i < V; ++i) v[k][i] = mul(w[k][i], xv[k][i]);
+            for (int i = 0; i < V; ++i)
+                v[k][i] = mul(REV ? w[k][i] : scaled(w[k][i], gain), xv[k][i]);
             if constexpr (REV) {
 #pragma unroll
                 for (int i = V - 1 - OFF; i >= 0; --i) v[k][i] = add(v[k][i], v[k][i + OFF]);
@@ -796,13 +812,15 @@ __global__ void __launch_bounds__(kThreads) k_sum_solve(const TI* in, TO* out, i
         A o[V];
         load_piece<V, ALIGNED>(wout, j, n, o);
 #pragma unroll
-        for (int i = 0; i < V; ++i) o[i] = mul(o[i], add(v[k][i], before[k].v[i % OFF]));
+        for (int i = 0; i < V; ++i)
+            o[i] = mul(REV ? o[i] : scaled(o[i], 1.0f / gain), add(v[k][i], before[k].v[i % OFF]));
         if (next) {
             A nw[V];
             load_piece<V, ALIGNED>(next, j, n, nw);
 #pragma unroll
             for (int i = 0; i < V; ++i)
-                ns.v[i % OFF] = add(ns.v[i % OFF], mul(nw[i], o[i]));
+                ns.v[i % OFF] =
+                    add(ns.v[i % OFF], mul(REV ? nw[i] : scaled(nw[i], next_gain), o[i]));
         }
         TO t[V];
 #pragma unroll
@@ -835,7 +853,7 @@ __global__ void k_sum_tables(FactorSpec F, int f, const double* __restrict__ g, 
     double p, q, W;
     factor_pq(U, par, j, &p, &q);
     if (F.family == SP_ULTRA) {
-        W = (par + x) * scale;
+        W = (par + x) / par;  // U = 1
     } else if (j == 0) {
         W = -q / p * (s + 3.0) * g[1] * scale;  // mu_0 W_1
     } else {
@@ -845,8 +863,7 @@ __global__ void k_sum_tables(FactorSpec F, int f, const double* __restrict__ g, 
     const double so = f == F.M - 1 && sout ? sout[j] : 1.0;
     const double si = f == 0 && sin ? sin[j] : 1.0;
     from_double(t[j], so * W * sign);
-    from_double(t[F.ld + j],
-                sign * si * (F.family == SP_ULTRA ? 1.0 / (par * scale) : 1.0 / (p * W)));
+    from_double(t[F.ld + j], sign * si * (F.family == SP_ULTRA ? 1.0 : 1.0 / (p * W)));
 }
 
 unsigned blocks_for(int64_t count) { return (unsigned)((count + kThreads - 1) / kThreads); }
@@ -970,8 +987,10 @@ int sums_typed(const Step& st, const void* in, void* out, int64_t batch, cudaStr
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_sum_tiles<A, TI, OFF, ALIGNED>,
-                                       static_cast<const TI*>(in), n, ntiles, row(0, REV), sum);
+    auto gain = [&](int f) { return st.sp_gain[REV ? f : st.sp_M - 1 - f]; };
+    cudaError_t e =
+        cudaLaunchKernelEx(&cfg, k_sum_tiles<A, TI, OFF, !REV, ALIGNED>,
+                           static_cast<const TI*>(in), n, ntiles, row(0, REV), gain(0), sum);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     for (int f = 0; f < st.sp_M && e == cudaSuccess; ++f) {
@@ -979,21 +998,22 @@ int sums_typed(const Step& st, const void* in, void* out, int64_t batch, cudaStr
         const A* next = last ? nullptr : row(f + 1, REV);
         const S* from = sum + (f & 1) * (size_t)grid;
         S* to = sum + ((f + 1) & 1) * (size_t)grid;
+        const float g = gain(f), ng = last ? 1.0f : gain(f + 1);
         if (first && last)
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, TI, TO, OFF, REV, ALIGNED>,
                                    static_cast<const TI*>(in), static_cast<TO*>(out), n, ntiles,
-                                   row(f, REV), row(f, !REV), from, next, to, 1);
+                                   row(f, REV), row(f, !REV), from, next, to, 1, g, ng);
         else if (first)
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, TI, M, OFF, REV, ALIGNED>,
                                    static_cast<const TI*>(in), mid, n, ntiles, row(f, REV),
-                                   row(f, !REV), from, next, to, 1);
+                                   row(f, !REV), from, next, to, 1, g, ng);
         else if (last)
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, M, TO, OFF, REV, ALIGNED>,
                                    (const M*)mid, static_cast<TO*>(out), n, ntiles, row(f, REV),
-                                   row(f, !REV), from, next, to, 0);
+                                   row(f, !REV), from, next, to, 0, g, ng);
         else
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, M, M, OFF, REV, ALIGNED>, (const M*)mid,
-                                   mid, n, ntiles, row(f, REV), row(f, !REV), from, next, to, 0);
+                                   mid, n, ntiles, row(f, REV), row(f, !REV), from, next, to, 0, g, ng);
     }
     scratch_free(scr, s);
     if (e != cudaSuccess) {
@@ -1068,17 +1088,17 @@ void weight_range(const FactorSpec& F, int f, double* lo, double* hi) {
     *hi = F.n > 1 ? lnw(last) : *lo;
 }
 
-bool sums_serve(const FactorSpec& F) {
-    for (int f = 0; f < F.M; ++f) {
+bool sums_serve(const FactorSpec& F, int prec) {
+    for (int f = 0; f < F.M && F.family != SP_ULTRA; ++f) {
         double lo, hi;
         weight_range(F, f, &lo, &hi);
-        if (!(std::fabs(hi - lo) <= kSumRange)) return false;
+        if (!(std::fabs(hi - lo) <= sum_range(prec))) return false;
     }
     return true;
 }
 
 template <typename A>
-int sum_tables(const Step& st, const FactorSpec& F, cudaStream_t s) {
+int sum_tables(Step& st, const FactorSpec& F, cudaStream_t s) {
     double* g = nullptr;  // Gamma ratios of one factor (Jacobi; entry 1 is read even for n = 1)
     const int64_t count = std::max<int64_t>(F.n, 2);
     if (F.family == SP_JACOBI) TDH_TRY(dev_alloc_t(&g, (size_t)count));
@@ -1089,10 +1109,9 @@ int sum_tables(const Step& st, const FactorSpec& F, cudaStream_t s) {
         const double par = F.par0 + F.dir * (double)f;
         if (g) rc = gamma_ratio_launch(par + F.b + 1.0, F.b + 1.0, count, g, s);
         if (rc != TDH_OK) break;
-        // ultraspherical U is the constant 1 / (l scale): a power of two, so that rounding it
-        // leaves no error common to all terms
-        double scale = std::exp(-0.5 * (lo + hi));
-        if (F.family == SP_ULTRA) scale = std::exp2(std::round(std::log2(scale * par))) / par;
+        const double scale = std::exp(-std::min(lo, hi));
+        st.sp_gain[f] =
+            F.family == SP_ULTRA ? 1.0f : (float)std::exp2(-std::ceil(std::fabs(hi - lo) / M_LN2));
         k_sum_tables<A><<<blocks_for(F.ld), kThreads, 0, s>>>(
             F, f, g, scale, st.scale_out, st.scale_in, static_cast<A*>(st.sp_tab));
         if (cudaGetLastError() != cudaSuccess) {
@@ -1130,7 +1149,7 @@ int sparse_prepare(Step& st, int prec, cudaStream_t s) {
     F.n = st.n;
     F.ld = (st.n + 2 + 3) / 4 * 4;  // float4 rows stay 16-byte aligned
     st.sp_ld = F.ld;
-    if (!st.sp_inverse || !sums_serve(F))
+    if (!st.sp_inverse || !sums_serve(F, prec))
         st.sp_sums = 0;
     else if (st.sp_alone)
         st.sp_sums = 1;
