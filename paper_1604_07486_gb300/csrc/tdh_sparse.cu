@@ -708,9 +708,47 @@ __global__ void __launch_bounds__(kThreads) k_sum_tiles(const TI* __restrict__ i
     if (threadIdx.x == 0) sum[blockIdx.x] = s;
 }
 
+// sum[v ntiles + t] <- the sum of the tiles after (REV) or before t: where a vector has many tiles,
+// adding them up in every block would be quadratic in n (2^27 coefficients: as many bytes as the
+// vector's).  One block per vector, a thread takes a strip of tiles.  Float32 C^(1.25) -> C^(0.25):
+// 2^27 690 -> 600 us, 2^29 5.7 -> 2.3 ms, two factors 24 -> 8.4 ms (affine scan 5.5 and 11 ms); at
+// 4 x 2^24 it costs as much as it saves (269 and 261 us).
+constexpr int kCarryTiles = 4097;  // tiles of a vector from which this pays
+template <typename A, int OFF, bool REV>
+__global__ void __launch_bounds__(kThreads) k_sum_carry(ChainSum<A, OFF>* __restrict__ sum,
+                                                        int64_t ntiles) {
+    __shared__ ChainSum<A, OFF> tot[kThreads];
+    ChainSum<A, OFF>* s = sum + (int64_t)blockIdx.x * ntiles;
+    const int64_t per = (ntiles + kThreads - 1) / kThreads;
+    const int64_t t0 = min((int64_t)threadIdx.x * per, ntiles), t1 = min(t0 + per, ntiles);
+    ChainSum<A, OFF> mine{};
+    for (int64_t t = t0; t < t1; ++t)
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) mine.v[c] = add(mine.v[c], s[t].v[c]);
+    // inclusive scan of the strips, in the direction of the sums
+    const int at = REV ? kThreads - 1 - (int)threadIdx.x : (int)threadIdx.x;
+    tot[at] = mine;
+    __syncthreads();
+    for (int d = 1; d < kThreads; d <<= 1) {
+        const ChainSum<A, OFF> o = at >= d ? tot[at - d] : ChainSum<A, OFF>{};
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) tot[at].v[c] = add(tot[at].v[c], o.v[c]);
+        __syncthreads();
+    }
+    ChainSum<A, OFF> run = at > 0 ? tot[at - 1] : ChainSum<A, OFF>{};
+    for (int64_t i = 0; i < t1 - t0; ++i) {
+        const int64_t t = REV ? t1 - 1 - i : t0 + i;
+        const ChainSum<A, OFF> x = s[t];
+        s[t] = run;
+#pragma unroll
+        for (int c = 0; c < OFF; ++c) run.v[c] = add(run.v[c], x.v[c]);
+    }
+}
+
 // out_j = wout_j (sum over the chain of win_i in_i, i >= j (REV) or i <= j); then, where `next` is
 // given, the tile sums of next_j out_j.  The block's carry is the sum of the tiles after (before)
-// its own, added in a fixed order.  In place allowed: a block reads its tile before writing it.
+// its own, added in a fixed order (carried: sum holds it).  In place allowed: a block reads its tile before writing it.
 // `first`: the input is older than the previous kernel, so it may be read before waiting for it.
 // gain, next_gain: the transpose's powers of two on win and next (wout's is 1 / gain).
 template <typename A, typename TI, typename TO, int OFF, bool REV, bool ALIGNED>
@@ -720,7 +758,8 @@ __global__ void __launch_bounds__(kThreads) k_sum_solve(const TI* in, TO* out, i
                                                         const ChainSum<A, OFF>* sum,
                                                         const A* __restrict__ next,
                                                         ChainSum<A, OFF>* next_sum, int first,
-                                                        float gain, float next_gain) {
+                                                        float gain, float next_gain,
+                                                        int carried) {
     constexpr int V = SumTile<A>::V;
     constexpr int NW = kThreads / 32;
     __shared__ ChainSum<A, OFF> red[NW], part[kSumChunks * NW];
@@ -778,7 +817,9 @@ __global__ void __launch_bounds__(kThreads) k_sum_solve(const TI* in, TO* out, i
     if (first) asm volatile("griddepcontrol.wait;" ::: "memory");
     // the other tiles' sums
     ChainSum<A, OFF> carry{};
-    for (int64_t t = (REV ? tile + 1 : 0) + tid; t < (REV ? ntiles : tile); t += kThreads)
+    if (carried && tid == 0) carry = sum[blockIdx.x];
+    for (int64_t t = carried ? ntiles : (REV ? tile + 1 : 0) + tid; t < (REV ? ntiles : tile);
+         t += kThreads)
 #pragma unroll
         for (int c = 0; c < OFF; ++c) carry.v[c] = add(carry.v[c], sum[vec * ntiles + t].v[c]);
     carry = block_sum<A, OFF>(carry, red);  // its barrier also publishes `part`
@@ -987,6 +1028,7 @@ int sums_typed(const Step& st, const void* in, void* out, int64_t batch, cudaStr
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    const int carried = ntiles >= kCarryTiles;
     auto gain = [&](int f) { return st.sp_gain[REV ? f : st.sp_M - 1 - f]; };
     cudaError_t e =
         cudaLaunchKernelEx(&cfg, k_sum_tiles<A, TI, OFF, !REV, ALIGNED>,
@@ -999,28 +1041,37 @@ int sums_typed(const Step& st, const void* in, void* out, int64_t batch, cudaStr
         const S* from = sum + (f & 1) * (size_t)grid;
         S* to = sum + ((f + 1) & 1) * (size_t)grid;
         const float g = gain(f), ng = last ? 1.0f : gain(f + 1);
+        if (carried) {
+            cfg.gridDim = dim3((unsigned)batch);
+            cfg.numAttrs = 0;
+            e = cudaLaunchKernelEx(&cfg, k_sum_carry<A, OFF, REV>, sum + (f & 1) * (size_t)grid,
+                                   ntiles);
+            cfg.gridDim = dim3(grid);
+            cfg.numAttrs = 1;
+            if (e != cudaSuccess) break;
+        }
         if (first && last)
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, TI, TO, OFF, REV, ALIGNED>,
                                    static_cast<const TI*>(in), static_cast<TO*>(out), n, ntiles,
-                                   row(f, REV), row(f, !REV), from, next, to, 1, g, ng);
+                                   row(f, REV), row(f, !REV), from, next, to, 1, g, ng, carried);
         else if (first)
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, TI, M, OFF, REV, ALIGNED>,
                                    static_cast<const TI*>(in), mid, n, ntiles, row(f, REV),
-                                   row(f, !REV), from, next, to, 1, g, ng);
+                                   row(f, !REV), from, next, to, 1, g, ng, carried);
         else if (last)
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, M, TO, OFF, REV, ALIGNED>,
                                    (const M*)mid, static_cast<TO*>(out), n, ntiles, row(f, REV),
-                                   row(f, !REV), from, next, to, 0, g, ng);
+                                   row(f, !REV), from, next, to, 0, g, ng, carried);
         else
             e = cudaLaunchKernelEx(&cfg, k_sum_solve<A, M, M, OFF, REV, ALIGNED>, (const M*)mid,
-                                   mid, n, ntiles, row(f, REV), row(f, !REV), from, next, to, 0, g, ng);
+                                   mid, n, ntiles, row(f, REV), row(f, !REV), from, next, to, 0, g, ng, carried);
     }
     scratch_free(scr, s);
     if (e != cudaSuccess) {
         set_error("back-substitution: %s", cudaGetErrorString(e));
         return TDH_ERR_CUDA;
     }
-    note_launches(1 + st.sp_M);
+    note_launches(1 + (carried ? 2 : 1) * st.sp_M);
     return TDH_OK;
 }
 

@@ -61,3 +61,36 @@ def test_no_loss_at_small_inputs(tdh, kind, params):
         x = _input(n, plan.dtype)
         for fn in (plan.execute, plan.adjoint):
             assert torch.equal(fn(x * 2.0 ** -68), fn(x) * 2.0 ** -68), n
+
+
+@pytest.mark.parametrize("n,prec,params", [((1 << 24) + 4100, "fp32", (1.25, 0.25)),
+                                           ((1 << 24) + 1, "fp32", (2.25, 0.25)),
+                                           ((1 << 23) + 2049, "fp64", (1.25, 0.25))])
+def test_many_tiles(tdh, n, prec, params):
+    """From 4097 tiles on their sums are scanned once per vector.  C^(l+1) -> C^(l) is
+    x_j = (l + j)/l sum_{i >= j, i = j mod 2} c_i: componentwise error at most 34 roundings (as for
+    fewer tiles) and one for every addition of the scan, 17 + 8 + 17 more; chains of two
+    factors (float32: pairs of floats) at most twice one rounding plus the reference's own."""
+    import torch
+    u = 2.0 ** (-24 if prec == "fp32" else -53)
+    plan = tdh.Plan("ultra2ultra", n, prec=prec, params=params)
+    x = torch.randn(1, n, dtype=plan.dtype, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+
+    def steps(v, transpose):
+        lams = [params[0] - 1 - i for i in range(round(params[0] - params[1]))]
+        for lam in (lams[::-1] if transpose else lams):
+            w = (np.arange(n) + np.longdouble(lam)) / np.longdouble(lam)
+            v = v * w if transpose else v
+            out = np.empty_like(v)
+            for e in range(2):
+                p = v[:, e::2]
+                out[:, e::2] = np.cumsum(p, 1) if transpose else np.cumsum(p[:, ::-1], 1)[:, ::-1]
+            v = out if transpose else out * w
+        return v
+
+    xd = x.double().cpu().numpy().astype(np.longdouble)
+    c = 2 if params[0] - params[1] > 1 else 34 + 42
+    for fn, tr in ((plan.execute, False), (plan.adjoint, True)):
+        y = fn(x).double().cpu().numpy()
+        err = np.abs(y - steps(xd, tr))
+        assert np.all(err <= c * u * steps(np.abs(xd), tr)), float((err / (u * steps(np.abs(xd), tr))).max())
