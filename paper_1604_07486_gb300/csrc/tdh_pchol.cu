@@ -9,12 +9,14 @@
 // <= tol * max(diag H).  u_r = l_r / sqrt(a_r) in the paper's notation, so
 // H ~ sum_r l_r l_r^T / a_r = sum_r u_r u_r^T.
 //
-// One cooperative launch for all steps: every block owns a fixed slice of indices and after each
-// step publishes the argmax of its slice of the updated d; a grid-wide barrier later every block
-// reduces the few hundred entries to the next pivot and takes the same stop decision from the
-// same data.  Latency-bound: a step is two barriers' worth of dependent loads (one launch per
-// step, with the host reading a stop flag every eight, took about 19 us a step at n = 2^16; the
-// barrier's waits are bounded, and a wait that ran out is reported as an error).
+// One launch per step over a grid of blocks, each launch on its way while the one before it drains
+// (programmatic dependent launch); a block owns a fixed slice of indices and publishes the argmax
+// of its slice of the updated d, and every block of the next step reduces the few hundred entries
+// to the pivot and takes the same stop decision from the same data.  No block waits for another,
+// so any number of SMs that the process may use will do (all steps in one cooperative launch need
+// every block resident at once, for 585 against 608 us per plan at n = 2^16).  Latency-bound: a step
+// is one chain of dependent loads.  The host reads the stop state after the first kFirstSteps steps, then every
+// kNextSteps; steps launched past the end return at once.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -29,10 +31,9 @@ constexpr int kThreads = 256;
 constexpr int kKmaxShared = 1024;  // u_i[p] for i < r staged in shared memory
 
 struct State {
+    double thresh;  // tol * max(diag H)
     int64_t K;      // steps taken
-    int done;       // stopped before the last step it may take, or by its target
-    int timeout;    // a barrier's wait ran out
-    unsigned count; // the barrier
+    int done;
 };
 
 // What a block publishes of its slice after a step: the largest residual diagonal entry (its
@@ -40,7 +41,7 @@ struct State {
 // factors of the truncation bound as bit patterns.  All comparisons are integer ones: a float64
 // comparison takes the SM's two float64 lanes sixteen cycles a warp, and the reductions need
 // hundreds of them.
-struct Part {
+struct __align__(16) Part {
     int64_t key;
     int64_t i;
     int64_t b1, b2;  // max (D1_j / w_j)^2 d_j, max (D2_j / w_j)^2 d_j (not below 0)
@@ -98,53 +99,29 @@ __device__ __forceinline__ Part part_of(const TargetSpec& T, int64_t j, double d
     return p;
 }
 
-// Grid-wide barrier of a cooperative launch: block 0 ... gridDim.x - 1 count up to gen *
-// gridDim.x.  Returns false when the wait ran out (a second; the other blocks then run out too).
-constexpr long long kBarrierNs = 1000000000ll;
-__device__ __forceinline__ long long global_ns() {
-    long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
+__device__ __forceinline__ void pdl_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-__device__ bool grid_barrier(unsigned* count, unsigned gen) {
-    __shared__ int ok;
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The maximum of the block's values to part[blockIdx.x].
+__device__ __forceinline__ void publish(Part own, Part* s_part, Part* part) {
+    own = warp_max(own);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = own;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(count, 1u);
-        const unsigned goal = gen * gridDim.x;
-        const long long t0 = global_ns();
-        int good = 1;
-        while (*(volatile unsigned*)count < goal) {
-            if (global_ns() - t0 > kBarrierNs) {
-                good = 0;
-                break;
-            }
-        }
-        __threadfence();
-        ok = good;
+        for (int i = 1; i < kThreads / 32; ++i) own = pmax(own, s_part[i]);
+        part[blockIdx.x] = own;
     }
-    __syncthreads();
-    return ok != 0;
 }
 
-// All steps.  The column's dot products read the earlier factors kBatch at a time (independent
-// loads in flight), and subtract in order.  part: [2][gridDim.x], alternating between steps.
-constexpr int kBatch = 8;
-
-__global__ void __launch_bounds__(kThreads, 2) pchol_all(
-    const double* __restrict__ h, int64_t n, int64_t j0, const double* __restrict__ w, double tol,
-    TargetSpec T, int kmax, double* u, int64_t* __restrict__ piv, double* __restrict__ d,
-    Part* part, State* st) {
-    __shared__ double s_up[kKmaxShared];
+// d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf); publishes the blocks' maxima.
+__global__ void __launch_bounds__(kThreads) pchol_init(const double* __restrict__ h, int64_t n,
+                                                       int64_t j0, const double* __restrict__ w,
+                                                       TargetSpec T, double* __restrict__ d,
+                                                       Part* __restrict__ part) {
     __shared__ Part s_part[kThreads / 32];
-    __shared__ double s_inv, s_wp;
-    __shared__ int64_t s_p;
-    const int nparts = gridDim.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    unsigned gen = 0;
-    // d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf)
+    pdl_trigger();
     Part own = part_none();
     for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * kThreads) {
@@ -152,100 +129,120 @@ __global__ void __launch_bounds__(kThreads, 2) pchol_all(
         d[j] = v;
         own = pmax(own, part_of(T, j, v, j >= j0));
     }
-    double thresh = 0.0;  // warp 0, lane 0
-    for (int r = 0;; ++r) {
-        own = warp_max(own);
-        if (lane == 0) s_part[warp] = own;
-        __syncthreads();
-        Part* pub = part + (r & 1) * nparts;
-        if (threadIdx.x == 0) {
-            for (int i = 1; i < kThreads / 32; ++i) own = pmax(own, s_part[i]);
-            pub[blockIdx.x] = own;
-        }
-        if (!grid_barrier(&st->count, ++gen)) {
-            if (threadIdx.x == 0) st->timeout = 1;
-            return;
-        }
-        // warp 0 of every block reduces the same partials (identical pivot and decision
-        // everywhere), gathers the pivot row of the factors and forms its scale
-        if (warp == 0) {
-            Part best = part_none();
-            for (int i = lane; i < nparts; i += 32) {
-                const volatile Part* q = pub + i;
-                Part o;
-                o.key = q->key;
-                o.i = q->i;
-                o.b1 = q->b1;
-                o.b2 = q->b2;
-                best = pmax(best, o);
-            }
-            best = warp_max(best);
-            const int64_t p = best.i;
-            int stop = 0;  // 1: done, 2: the last step taken
-            if (lane == 0) {
-                const double v = order_value(best.key);
-                if (r == 0) thresh = tol * v;
-                const bool met = T.a1 && *T.tmax * sqrt(__longlong_as_double(best.b1)) *
-                                                 sqrt(__longlong_as_double(best.b2)) <= T.target;
-                if (met || !(v > thresh) || p < j0 || p >= n)
-                    stop = 1;
-                else if (r == kmax)
-                    stop = 2;
-            }
-            stop = __shfl_sync(0xffffffffu, stop, 0);
-            if (!stop) {
-                // (factors of this launch are read past L1, which other SMs' writes do not reach)
-                for (int i = lane; i < r; i += 32) s_up[i] = __ldcg(u + (int64_t)i * n + p);
-                __syncwarp();
-                if (lane == 0) {
-                    const double wp = w ? w[p] : 1.0;
-                    double a = h[2 * p] * wp * wp;
-                    for (int i = 0; i < r; ++i) a -= s_up[i] * s_up[i];
-                    if (!(a > thresh)) stop = 1;
-                    s_wp = wp;
-                    s_inv = 1.0 / sqrt(a);
-                }
-            }
-            if (lane == 0) {
-                s_p = stop ? -1 : p;
-                if (stop && blockIdx.x == 0) {
-                    st->K = r;
-                    st->done = stop == 1;
-                }
-            }
-        }
-        __syncthreads();
-        const int64_t p = s_p;
-        if (p < 0) return;
-        const double inv = s_inv, wp = s_wp;
-        own = part_none();
-        double* ur = u + (int64_t)r * n;
-        for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
-             j += (int64_t)gridDim.x * kThreads) {
-            double val = 0.0;
-            double dj = -INFINITY;
-            if (j >= j0) {
-                double c = h[j + p] * (w ? w[j] * wp : 1.0);
-                const double dold = d[j];
-                const double* uj = u + j;  // this thread's own writes
-                int i = 0;
-                for (; i + kBatch <= r; i += kBatch) {
-                    double v[kBatch];
+    publish(own, s_part, part);
+}
+
+// Step r.  Warp 0 decides, gathers the pivot row of the factors and forms its scale; the column's
+// dot products read the earlier factors kBatch at a time (independent loads in flight), and subtract
+// in order.  What earlier steps wrote is read past L1.
+constexpr int kBatch = 8;
+
+__global__ void __launch_bounds__(kThreads) pchol_step(
+    const double* __restrict__ h, int64_t n, int64_t j0, const double* __restrict__ w, double tol,
+    TargetSpec T, int r, double* u, int64_t* __restrict__ piv, double* d, const Part* part_in,
+    Part* part_out, State* st) {
+    __shared__ double s_up[kKmaxShared];
+    __shared__ Part s_part[kThreads / 32];
+    __shared__ double s_inv, s_wp;
+    __shared__ int64_t s_p;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    pdl_trigger();
+    const double tmax = T.a1 ? *T.tmax : 0.0;
+    const int64_t jf = (int64_t)blockIdx.x * kThreads + threadIdx.x;  // this thread's first index
+    const double wf = w && jf < n ? w[jf] : 1.0;
+    pdl_wait();
+    // what does not depend on the pivot is on its way before the decision
+    double df = 0.0, uf[kBatch];
+    if (jf < n) {
+        df = __ldcg(d + jf);
 #pragma unroll
-                    for (int b = 0; b < kBatch; ++b) v[b] = __ldcg(uj + (int64_t)(i + b) * n);
-#pragma unroll
-                    for (int b = 0; b < kBatch; ++b) c -= v[b] * s_up[i + b];
-                }
-                for (; i < r; ++i) c -= __ldcg(uj + (int64_t)i * n) * s_up[i];
-                val = c * inv;
-                dj = dold - val * val;
-                d[j] = dj;
-            }
-            ur[j] = val;
-            own = pmax(own, part_of(T, j, dj, j >= j0));
-        }
-        if (lead) piv[r] = p;
+        for (int b = 0; b < kBatch; ++b) uf[b] = b < r ? __ldcg(u + jf + (int64_t)b * n) : 0.0;
     }
+    // every block reduces the same partials: identical pivot and decision everywhere
+    Part best = part_none();
+    for (int i = threadIdx.x; i < gridDim.x; i += kThreads) {
+        const longlong2* q = reinterpret_cast<const longlong2*>(part_in + i);
+        const longlong2 a = __ldcg(q), b = __ldcg(q + 1);
+        best = pmax(best, Part{a.x, a.y, b.x, b.y});
+    }
+    best = warp_max(best);
+    if (lane == 0) s_part[warp] = best;
+    __syncthreads();
+    if (warp == 0) {
+        best = warp_max(lane < kThreads / 32 ? s_part[lane] : part_none());
+        const int64_t p = best.i;
+        // One thread reads the state: block 0 may set `done` while other blocks of this step still
+        // look at it, so the threads of a block must not each decide from their own reading.  (A
+        // block that sees this step's `done` stops as its own data would have it.)
+        int stop = 0, done = 0;
+        double thresh = 0.0;
+        if (lane == 0) {
+            const double v = order_value(best.key);
+            done = *(volatile int*)&st->done;
+            thresh = r == 0 ? tol * v : *(volatile double*)&st->thresh;
+            const bool met = T.a1 && tmax * sqrt(__longlong_as_double(best.b1)) *
+                                           sqrt(__longlong_as_double(best.b2)) <= T.target;
+            stop = done || met || !(v > thresh) || p < j0 || p >= n;
+        }
+        stop = __shfl_sync(0xffffffffu, stop, 0);
+        if (!stop) {
+            for (int i = lane; i < r; i += 32) s_up[i] = __ldcg(u + (int64_t)i * n + p);
+            __syncwarp();
+            if (lane == 0) {
+                const double wp = w ? w[p] : 1.0;
+                double a = h[2 * p] * wp * wp;
+                for (int i = 0; i < r; ++i) a -= s_up[i] * s_up[i];
+                if (!(a > thresh)) stop = 1;
+                s_wp = wp;
+                s_inv = 1.0 / sqrt(a);
+            }
+        }
+        if (lane == 0) s_p = stop ? -1 : p;
+        if (lead && !done) {  // (only this thread ever sets `done`)
+            st->K = stop ? r : r + 1;
+            if (stop) st->done = 1;
+            if (r == 0) st->thresh = thresh;
+        }
+    }
+    __syncthreads();
+    const int64_t p = s_p;
+    if (p < 0) return;
+    const double wp = s_wp;
+    const double inv = s_inv;
+    Part own = part_none();
+    double* ur = u + (int64_t)r * n;
+    for (int64_t j = jf; j < n; j += (int64_t)gridDim.x * kThreads) {
+        double val = 0.0;
+        double dj = -INFINITY;
+        if (j >= j0) {
+            const bool first = j == jf;
+            double c = h[j + p] * (w ? (first ? wf : w[j]) * wp : 1.0);
+            const double dold = first ? df : __ldcg(d + j);
+            const double* uj = u + j;
+            int i = 0;
+            if (first && r >= kBatch) {
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) c -= uf[b] * s_up[b];
+                i = kBatch;
+            }
+            for (; i + kBatch <= r; i += kBatch) {
+                double x[kBatch];
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) x[b] = __ldcg(uj + (int64_t)(i + b) * n);
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) c -= x[b] * s_up[i + b];
+            }
+            for (; i < r; ++i) c -= __ldcg(uj + (int64_t)i * n) * s_up[i];
+            val = c * inv;
+            dj = dold - val * val;
+            d[j] = dj;
+        }
+        ur[j] = val;
+        own = pmax(own, part_of(T, j, dj, j >= j0));
+    }
+    publish(own, s_part, part_out);
+    if (lead) piv[r] = p;
 }
 
 }  // namespace
@@ -253,31 +250,48 @@ __global__ void __launch_bounds__(kThreads, 2) pchol_all(
 namespace {
 
 // The steps of a factorisation on stream s: state, residual diagonal and partials given.
+constexpr int64_t kFirstSteps = 20, kNextSteps = 12;
+
 cudaError_t pchol_steps(const double* h, const double* w, int64_t n, int64_t j0, double tol,
                         int64_t kmax, const TargetSpec& T, double* u, int64_t* pivots, double* d,
                         Part* part, int nblk, State* st, State* host, cudaStream_t s) {
     *host = State{};
-    int kk = (int)kmax;
     cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
     if (e == cudaSuccess) {
-        TargetSpec TT = T;
-        void* args[] = {&h, &n, &j0, &w, &tol, &TT, &kk, &u, &pivots, &d, &part, &st};
-        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pchol_all), dim3(nblk),
-                                        dim3(kThreads), args, 0, s);
+        pchol_init<<<nblk, kThreads, 0, s>>>(h, n, j0, w, T, d, part);
+        e = cudaGetLastError();
     }
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && host->timeout) e = cudaErrorLaunchTimeout;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblk);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int64_t poll = kFirstSteps;
+    for (int64_t r = 0; e == cudaSuccess && r < kmax; ++r) {
+        const Part* in = part + (r & 1) * nblk;
+        e = cudaLaunchKernelEx(&cfg, pchol_step, h, n, j0, w, tol, T, (int)r, u, pivots, d, in,
+                               part + ((r + 1) & 1) * nblk, st);
+        if (e == cudaSuccess && (r + 1 == poll || r + 1 == kmax)) {
+            poll += kNextSteps;
+            e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (host->done) break;
+        }
+    }
     return e;
 }
 
 }  // namespace
 
-// Blocks of the launch: all resident at once (two of at most 128 registers a thread per SM).
+// Blocks of a step: six per SM at most (more partials to reduce, for no more loads in flight than
+// the memory system takes).
 int pchol_blocks(int64_t n) {
     return (int)std::max<int64_t>(
-        1, std::min<int64_t>((n + kThreads - 1) / kThreads, 2 * (int64_t)sm_count()));
+        1, std::min<int64_t>((n + kThreads - 1) / kThreads, 6 * (int64_t)sm_count()));
 }
 
 int pchol_run(const double* h, const double* w, int64_t n, int64_t j0, double tol, int64_t kmax,
@@ -403,7 +417,7 @@ extern "C" int tdh_pchol(const double* h, int64_t n, int64_t j0, double tol, int
 // array and it keeps the contents of the last call: the state words that must start at zero
 // are cleared by every call, the rest is fully rewritten.  Two calls whose work overlaps on
 // the GPU (different streams, or different host threads) race on the array; serialise them.
-// Each call synchronises `stream` (it reads the stop state back every few steps).
+// Each call synchronises `stream` (it reads the stop state back).
 namespace tdh {
 namespace {
 
