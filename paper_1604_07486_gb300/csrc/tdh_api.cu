@@ -232,7 +232,9 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
         }
         // room for kFirstRank terms first (no plan of the common kinds needs more); a run that
         // fills it starts again with all of kcap
+        int64_t rows = 0;
         for (int64_t cap = std::min(kcap, kFirstRank); rc == TDH_OK; cap = kcap) {
+            rows = cap;
             dev_free(ubig);
             ubig = nullptr;
             rc = dev_alloc_t(&ubig, (size_t)(cap * n));
@@ -247,7 +249,7 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
             dev_free(w);
         }
         if (rc == TDH_OK && K > 0) {
-            if (sizeof(double) * (size_t)(kFirstRank * n) <= kKeepBytes) {
+            if (sizeof(double) * (size_t)(rows * n) <= kKeepBytes) {
                 std::swap(st.u64, ubig);  // small: kept with its spare rows
             } else {
                 rc = dev_alloc_t(&st.u64, (size_t)K * n);

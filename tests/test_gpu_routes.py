@@ -180,3 +180,17 @@ def test_executes_get_by_with_less_scratch(tdh, kind, params):
             assert float(((y - r).abs().amax(1) / scale).max()) <= 2 * TOL["fp32"], k
     torch.cuda.synchronize()
     assert tdh.alloc_stats()[2] == 0
+
+
+def test_plans_keep_only_their_rank(tdh):
+    """A plan whose factorisation fills its first 64 terms starts again with room for kmax; it keeps
+    the terms it took, and at most 64 MB of spare rows."""
+    import torch
+    n = 20000
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    plan = tdh.Plan("jac2jac", n, prec="fp64", params=(10.2, 3.0, 10.9, 3.0), kmax=1000)
+    torch.cuda.synchronize()
+    held = free0 - torch.cuda.mem_get_info()[0]
+    assert plan.K > 64
+    assert held <= 8 * n * plan.K + (64 << 20) + (32 << 20), (held, plan.K)
