@@ -1246,6 +1246,26 @@ double lagrange(const int* x, int P, int i, double at) {
     return v;
 }
 
+// Factors that make s_0 and h's first entry on the diagonal (index 2 j0) powers of two: entry
+// (j, j) = D1_j s_0 h_2j D2_j then carries no rounding of s_0, and the first one none of h.  (The
+// leading coefficients dominate decaying inputs, and a rounding common to all of them shows in
+// full.)  The mantissas taken out go to D1, which is rounded once for all of it.
+// Float64 keeps the symbols as they are: they are float64 already.
+template <typename T>
+__device__ __forceinline__ double mantissa(double v) {
+    if (sizeof(T) == 8 || v == 0.0 || !isfinite(v)) return 1.0;
+    int e;
+    return fabs(frexp(v, &e)) * 2.0;
+}
+
+// D1 for the tables below
+template <typename T>
+__global__ void k_hier_diagonal(const double* __restrict__ t, const double* __restrict__ h, int j0,
+                                const double* __restrict__ d1, int64_t n, T* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (i < n) out[i] = (T)(d1[i] * (mantissa<T>(t[0]) * mantissa<T>(h[2 * j0])));
+}
+
 // table copies in execute precision: s_m = t[stride m] (32 zeros before, zero past mpad),
 // hf_l = h[stride l], hr_i = hf[2 mrev - 1 - i] (zero past 2 mrev); entry 0 of h dropped where
 // (0, 0) is direct
@@ -1254,10 +1274,11 @@ __global__ void k_hier_tables(const double* __restrict__ t, const double* __rest
                               int64_t mpad, int64_t mrev, int stride, int j0, T* __restrict__ s,
                               T* __restrict__ hf, T* __restrict__ hr) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const double mt = mantissa<T>(t[0]), mh = mantissa<T>(h[2 * j0]);
     if (i < kHierSZero) s[i - kHierSZero] = T(0);
-    if (i < mpad) s[i] = (T)t[stride * i];
+    if (i < mpad) s[i] = (T)(t[stride * i] / mt);
     if (i < 2 * mpad + kHierHPad) {
-        const T v = (i >= 2 * mpad || (j0 == 1 && i == 0)) ? T(0) : (T)h[stride * i];
+        const T v = (i >= 2 * mpad || (j0 == 1 && i == 0)) ? T(0) : (T)(h[stride * i] / mh);
         hf[i] = v;
         if (i < 2 * mrev)
             hr[2 * mrev - 1 - i] = v;
@@ -1316,7 +1337,8 @@ int prepare_typed(Step& st, cudaStream_t s) {
     const bool top = ntop >= kTopKernel;
     const int64_t nps = top ? ntop * P * P : 0, nph = top ? (2 * ntop - 1) * NC * P * P : 0;
     const size_t at = (ns + 2 * nh + nw + 3) / 4 * 4;  // 16-byte aligned
-    int rc = dev_alloc(&H.tab, sizeof(T) * (at + (size_t)(nps + 2 * nph)));
+    const size_t nd = sizeof(T) == 4 ? (size_t)(st.n + 3) / 4 * 4 : 0;  // D1 of the scaled tables
+    int rc = dev_alloc(&H.tab, sizeof(T) * (at + (size_t)(nps + 2 * nph) + nd));
     std::vector<T> w(nw);
     if (rc == TDH_OK) {
         T* tab = static_cast<T*>(H.tab);
@@ -1328,6 +1350,13 @@ int prepare_typed(Step& st, cudaStream_t s) {
         k_hier_tables<T><<<(unsigned)((cnt + kThreads - 1) / kThreads), kThreads, 0, s>>>(
             st.t, st.h, H.mpad, H.mrev, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
             static_cast<T*>(H.hr));
+        H.d1 = st.d1x;
+        if (nd) {
+            T* d1 = tab + at + nps + 2 * nph;
+            k_hier_diagonal<T><<<(unsigned)((st.n + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+                st.t, st.h, (int)st.j0, st.d1, st.n, d1);
+            H.d1 = d1;
+        }
         if (top) {
             H.st = tab + at;
             H.ht[0] = tab + at + nps;
@@ -1607,8 +1636,8 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     P.ht = static_cast<const T*>(H.ht[adjoint ? 1 : 0]);
     P.lw = static_cast<const T*>(H.w);
     P.tr = P.lw + NP * kHierLeaf;
-    P.din = static_cast<const T*>(adjoint ? st.d1x : st.d2x);
-    P.dout = static_cast<const T*>(adjoint ? st.d2x : st.d1x);
+    P.din = static_cast<const T*>(adjoint ? H.d1 : st.d2x);
+    P.dout = static_cast<const T*>(adjoint ? st.d2x : H.d1);
     P.a00 = st.j0 == 1 ? static_cast<const T*>(st.row0) : nullptr;
     P.rev = adjoint;
     P.aligned = st.n * (int64_t)sizeof(T) % 16 == 0;

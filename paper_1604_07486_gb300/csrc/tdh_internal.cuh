@@ -152,6 +152,7 @@ struct HierData {
     void* s = nullptr;    // s[-32 .. mpad]
     void* hf = nullptr;   // Hankel table, forward
     void* hr = nullptr;   // Hankel table, reversed (transpose)
+    void* d1 = nullptr;   // D1 that goes with them
     void* w = nullptr;    // Lagrange weights: leaf [P][32], then transfers [3][4][P][P]
     void* st = nullptr;   // long vectors: s at the 2048-boxes' points, [distance][P][P]
     void* ht[2] = {};     // and h, forward and reversed, [sum of indices][NC][P][P]

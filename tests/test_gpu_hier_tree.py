@@ -71,3 +71,18 @@ def test_tree_at_box_edges(tdh, name, n):
         for fn, tr in ((plan.execute, False), (plan.adjoint, True)):
             y = fn(xt).double().cpu().numpy()
             _check_vectors(name, x, y, picks, prec, tr)
+
+
+@pytest.mark.parametrize("batch", [1, 3000])
+def test_leading_entry_is_exact(tdh, batch):
+    """C_0 = 1 for every parameter, A_00 = 1: the float32 tables hold s_0 and h_0 as powers of two and
+    what was taken out of them in D1, whose first entry is then one too, so the constant is
+    converted exactly (direct product and tree, forward and transposed)."""
+    import torch
+    n = 150
+    for params in ((0.05, 1.04), (0.488, 1.297), (0.9, 0.2), (0.3, 0.8), (100.2, 100.7), (0.7, 0.25)):
+        plan = tdh.Plan("ultra2ultra", n, prec="fp32", params=params)
+        x = torch.zeros(batch, n, device="cuda")
+        x[:, 0] = 1.0
+        for fn in (plan.execute, plan.adjoint):
+            assert (fn(x)[:, 0] == 1.0).all(), (params, float(fn(x)[0, 0]) - 1)
