@@ -86,3 +86,58 @@ def test_leading_entry_is_exact(tdh, batch):
         x[:, 0] = 1.0
         for fn in (plan.execute, plan.adjoint):
             assert (fn(x)[:, 0] == 1.0).all(), (params, float(fn(x)[0, 0]) - 1)
+
+
+@pytest.mark.parametrize("kind", ["leg2cheb", "cheb2leg", "jacobi"])
+def test_wide_far_field_and_top_exchange(tdh, kind):
+    """Float32 against float64 of the same input, in the norm of the result: inputs that live only in
+    the last box of 2048 of long vectors (forward; the first for the transpose), rows two boxes and
+    more away, so that every value comes through the exchange of the 2048-boxes -- by itself
+    (>= 32 boxes) and within the far kernel -- and through each of its smaller levels; batches of one
+    vector group and of the 16-vector far CTAs.  Bound: 64 roundings of |A| |alpha| and the
+    interpolation's 2.5e-8; the entries here have one sign, so |A| |alpha| is A |alpha|."""
+    import torch
+    name, _, params = KINDS[kind]
+    channels = 1 if kind == "jacobi" else 2
+    for n, batch in ((channels * 2048 * 40 + 77, 3), (channels * 2048 * 5 + 1, 40),
+                     (channels * 2048 * 2 + 9, 200)):
+        lo = tdh.Plan(name, n, prec="fp32", params=params or ())
+        hi = tdh.Plan(name, n, prec="fp64", params=params or ())
+        g = torch.Generator("cuda").manual_seed(n)
+        far = torch.randn(batch, n, device="cuda", generator=g)
+        for size in (2048, 512, 128, 32):
+            w = channels * size
+            if 3 * w >= n:  # no rows that far away
+                continue
+            for tr in (False, True):
+                x = torch.zeros_like(far)
+                keep = slice(n - w, n) if not tr else slice(0, w)
+                x[:, keep] = far[:, keep]
+                fn, ref = (lo.adjoint, hi.adjoint) if tr else (lo.execute, hi.execute)
+                rows = slice(0, n - 3 * w) if not tr else slice(3 * w, n)
+                y, r = fn(x).double()[:, rows], ref(x.double())[:, rows]
+                a = ref(x.double().abs())[:, rows]
+                err = (y - r).norm(dim=1) / a.norm(dim=1)
+                assert float(err.max()) <= 64 * U["fp32"] + FAR["fp32"], (n, size, tr, float(err.max()))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_chunks_of_vectors(tdh, prec):
+    """More vectors than one pass of the tree takes (about 1 GB of moments): those on both sides of
+    the cut, dense and ragged, against the oracle, and the same vector everywhere the same."""
+    import torch
+    n, batch = 300, 330000 if prec == "fp64" else 1300000
+    x = workloads.coefficients(n, 50, decay=0.5, seed=1)
+    if prec == "fp32":
+        x = x.astype(np.float32).astype(np.float64)
+    plan = tdh.Plan("cheb2leg", n, prec=prec, ragged=True)
+    base = torch.tensor(x, dtype=plan.dtype, device="cuda")
+    big = base.repeat((batch + 49) // 50, 1)[:batch]
+    offs = torch.arange(batch + 1, device="cuda") * n
+    for tr, y in ((False, plan.execute(big)), (True, plan.adjoint(big)),
+                  (False, plan.execute_ragged(big.flatten(), offs).reshape(batch, n))):
+        first = y[:50].double().cpu().numpy()
+        _check_vectors("cheb2leg", x, first, np.arange(50), prec, tr)
+        assert all(torch.equal(y[k:k + 50], y[:50]) for k in range(0, batch - 50, 50 * 800))
+        assert torch.equal(y[batch - 50:], y[:50])
+    assert plan.status() == set()
