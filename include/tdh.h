@@ -350,7 +350,9 @@ int tdh_test_fail_alloc(int64_t k);
  * second; the kernels then skip their remaining waits, finish, free their tensor memory and
  * record TDH_STATUS_TIMEOUT (tdh_plan_status).  Their outputs are not valid.  The setting is
  * process-wide and read when an execute is enqueued (a captured CUDA graph keeps the value it
- * was captured with).  Returns TDH_OK.
+ * was captured with).  Factorisations of plans created meanwhile, and tdh_pchol's, find the waits
+ * between their blocks run out after about a tenth of a second, as they would where the blocks are
+ * not all resident at once, and run launch by launch, with the same results.  Returns TDH_OK.
  */
 int tdh_test_tc_stall(int on);
 

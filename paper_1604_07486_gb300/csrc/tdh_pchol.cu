@@ -9,14 +9,14 @@
 // <= tol * max(diag H).  u_r = l_r / sqrt(a_r) in the paper's notation, so
 // H ~ sum_r l_r l_r^T / a_r = sum_r u_r u_r^T.
 //
-// One launch per step over a grid of blocks, each launch on its way while the one before it drains
-// (programmatic dependent launch); a block owns a fixed slice of indices and publishes the argmax
-// of its slice of the updated d, and every block of the next step reduces the few hundred entries
-// to the pivot and takes the same stop decision from the same data.  No block waits for another,
-// so any number of SMs that the process may use will do (all steps in one cooperative launch need
-// every block resident at once, for 585 against 608 us per plan at n = 2^16).  Latency-bound: a step
-// is one chain of dependent loads.  The host reads the stop state after the first kFirstSteps steps, then every
-// kNextSteps; steps launched past the end return at once.
+// One launch for all steps: a block owns a fixed slice of indices, publishes the argmax of its slice
+// of the updated d, and after a grid-wide barrier every block reduces the few hundred entries to the
+// pivot and takes the same stop decision from the same data.  The blocks fit the device all at once,
+// but beside other work, or where the process may not use every SM, they need not be resident
+// together, so nothing relies on it: the barrier's waits are bounded, a wait that runs out ends the
+// launch, and the factorisation then runs as one launch per step, whose blocks wait for nobody.
+// Latency-bound, a step is one chain of dependent loads: plan creation at n = 2^16 takes 650 us in
+// one launch, 720 us in one per step.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -34,6 +34,8 @@ struct State {
     double thresh;  // tol * max(diag H)
     int64_t K;      // steps taken
     int done;
+    int timeout;    // a barrier's wait ran out
+    unsigned count; // the barrier
 };
 
 // What a block publishes of its slice after a step: the largest residual diagonal entry (its
@@ -115,13 +117,41 @@ __device__ __forceinline__ void publish(Part own, Part* s_part, Part* part) {
     }
 }
 
-// d_j = H_jj = h[2j] for j >= j0 (excluded indices get -inf); publishes the blocks' maxima.
-__global__ void __launch_bounds__(kThreads) pchol_init(const double* __restrict__ h, int64_t n,
-                                                       int64_t j0, const double* __restrict__ w,
-                                                       TargetSpec T, double* __restrict__ d,
-                                                       Part* __restrict__ part) {
-    __shared__ Part s_part[kThreads / 32];
-    pdl_trigger();
+// Grid-wide barrier, for the gen-th time: blocks count up to gen gridDim.x (+ stall, for a test of
+// the limit).  Returns false when the wait, or another block's, ran out.
+constexpr long long kBarrierNs = 100000000ll;
+__device__ __forceinline__ long long global_ns() {
+    long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ bool grid_barrier(State* st, unsigned gen, unsigned stall) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&st->count, 1u);
+        const unsigned goal = gen * gridDim.x + stall;
+        const long long t0 = global_ns();
+        int good = 1;
+        while (*(volatile unsigned*)&st->count < goal) {
+            if (*(volatile int*)&st->timeout || global_ns() - t0 > kBarrierNs) {
+                good = 0;
+                break;
+            }
+        }
+        __threadfence();
+        ok = good;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+// d_j = H_jj = h[2j] of the block's slice for j >= j0 (excluded indices get -inf); their maximum
+// goes to part[blockIdx.x].
+__device__ __forceinline__ void init_slice(const double* h, int64_t n, int64_t j0, const double* w,
+                                           const TargetSpec& T, double* d, Part* part,
+                                           Part* s_part) {
     Part own = part_none();
     for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * kThreads) {
@@ -132,131 +162,168 @@ __global__ void __launch_bounds__(kThreads) pchol_init(const double* __restrict_
     publish(own, s_part, part);
 }
 
-// Step r.  Warp 0 decides, gathers the pivot row of the factors and forms its scale; the column's
-// dot products read the earlier factors kBatch at a time (independent loads in flight), and subtract
-// in order.  What earlier steps wrote is read past L1.
+__global__ void __launch_bounds__(kThreads) pchol_init(const double* __restrict__ h, int64_t n,
+                                                       int64_t j0, const double* __restrict__ w,
+                                                       TargetSpec T, double* d, Part* part) {
+    __shared__ Part s_part[kThreads / 32];
+    pdl_trigger();
+    init_slice(h, n, j0, w, T, d, part, s_part);
+}
+
+// ALL: every step (r0 = 0); else step r0, overlapping the end of the kernel before it.  Warp 0
+// decides, gathers the pivot row of the factors and forms its scale; the column's dot products
+// read the earlier factors kBatch at a time (independent loads in flight), and subtract in order.
+// What other blocks wrote is read past L1.  part: [2][gridDim.x], alternating between steps.
 constexpr int kBatch = 8;
 
-__global__ void __launch_bounds__(kThreads) pchol_step(
+template <bool ALL>
+__global__ void __launch_bounds__(kThreads, 2) pchol_step(
     const double* __restrict__ h, int64_t n, int64_t j0, const double* __restrict__ w, double tol,
-    TargetSpec T, int r, double* u, int64_t* __restrict__ piv, double* d, const Part* part_in,
-    Part* part_out, State* st) {
+    TargetSpec T, int r0, int kmax, double* u, int64_t* __restrict__ piv, double* d, Part* part,
+    State* st, unsigned stall) {
     __shared__ double s_up[kKmaxShared];
     __shared__ Part s_part[kThreads / 32];
     __shared__ double s_inv, s_wp;
     __shared__ int64_t s_p;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    pdl_trigger();
     const double tmax = T.a1 ? *T.tmax : 0.0;
     const int64_t jf = (int64_t)blockIdx.x * kThreads + threadIdx.x;  // this thread's first index
     const double wf = w && jf < n ? w[jf] : 1.0;
-    pdl_wait();
-    // what does not depend on the pivot is on its way before the decision
-    double df = 0.0, uf[kBatch];
-    if (jf < n) {
-        df = __ldcg(d + jf);
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) uf[b] = b < r ? __ldcg(u + jf + (int64_t)b * n) : 0.0;
+    if constexpr (ALL) {
+        init_slice(h, n, j0, w, T, d, part, s_part);
+    } else {
+        pdl_trigger();
+        pdl_wait();
     }
-    // every block reduces the same partials: identical pivot and decision everywhere
-    Part best = part_none();
-    for (int i = threadIdx.x; i < gridDim.x; i += kThreads) {
-        const longlong2* q = reinterpret_cast<const longlong2*>(part_in + i);
-        const longlong2 a = __ldcg(q), b = __ldcg(q + 1);
-        best = pmax(best, Part{a.x, a.y, b.x, b.y});
-    }
-    best = warp_max(best);
-    if (lane == 0) s_part[warp] = best;
-    __syncthreads();
-    if (warp == 0) {
-        best = warp_max(lane < kThreads / 32 ? s_part[lane] : part_none());
-        const int64_t p = best.i;
-        // One thread reads the state: block 0 may set `done` while other blocks of this step still
-        // look at it, so the threads of a block must not each decide from their own reading.  (A
-        // block that sees this step's `done` stops as its own data would have it.)
-        int stop = 0, done = 0;
-        double thresh = 0.0;
-        if (lane == 0) {
-            const double v = order_value(best.key);
-            done = *(volatile int*)&st->done;
-            thresh = r == 0 ? tol * v : *(volatile double*)&st->thresh;
-            const bool met = T.a1 && tmax * sqrt(__longlong_as_double(best.b1)) *
-                                           sqrt(__longlong_as_double(best.b2)) <= T.target;
-            stop = done || met || !(v > thresh) || p < j0 || p >= n;
+    for (int r = r0; ALL ? r < kmax : r == r0; ++r) {
+        if (ALL && !grid_barrier(st, (unsigned)r + 1u, stall)) {
+            if (threadIdx.x == 0) st->timeout = 1;
+            return;
         }
-        stop = __shfl_sync(0xffffffffu, stop, 0);
-        if (!stop) {
-            for (int i = lane; i < r; i += 32) s_up[i] = __ldcg(u + (int64_t)i * n + p);
-            __syncwarp();
+        // what does not depend on the pivot is on its way before the decision
+        double df = 0.0, uf[kBatch];
+        if (jf < n) {
+            df = __ldcg(d + jf);
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) uf[b] = b < r ? __ldcg(u + jf + (int64_t)b * n) : 0.0;
+        }
+        // every block reduces the same partials: identical pivot and decision everywhere
+        const Part* in = part + (r & 1) * (int)gridDim.x;
+        Part best = part_none();
+        for (int i = threadIdx.x; i < gridDim.x; i += kThreads) {
+            const longlong2* q = reinterpret_cast<const longlong2*>(in + i);
+            const longlong2 a = __ldcg(q), b = __ldcg(q + 1);
+            best = pmax(best, Part{a.x, a.y, b.x, b.y});
+        }
+        best = warp_max(best);
+        if (lane == 0) s_part[warp] = best;
+        __syncthreads();
+        if (warp == 0) {
+            best = warp_max(lane < kThreads / 32 ? s_part[lane] : part_none());
+            const int64_t p = best.i;
+            // One thread reads the state: block 0 may set `done` while other blocks of this step
+            // still look at it, so the threads of a block must not each decide from their own
+            // reading.  (A block that sees this step's `done` stops as its own data would have it.)
+            int stop = 0, done = 0;
+            double thresh = 0.0;
             if (lane == 0) {
-                const double wp = w ? w[p] : 1.0;
-                double a = h[2 * p] * wp * wp;
-                for (int i = 0; i < r; ++i) a -= s_up[i] * s_up[i];
-                if (!(a > thresh)) stop = 1;
-                s_wp = wp;
-                s_inv = 1.0 / sqrt(a);
+                const double v = order_value(best.key);
+                if (!ALL) done = *(volatile int*)&st->done;
+                thresh = r == 0 ? tol * v : *(volatile double*)&st->thresh;
+                const bool met = T.a1 && tmax * sqrt(__longlong_as_double(best.b1)) *
+                                                 sqrt(__longlong_as_double(best.b2)) <= T.target;
+                stop = done || met || !(v > thresh) || p < j0 || p >= n;
+            }
+            stop = __shfl_sync(0xffffffffu, stop, 0);
+            if (!stop) {
+                const double wp = w ? w[p] : 1.0, hp = h[2 * p];
+                for (int i = lane; i < r; i += 32) s_up[i] = __ldcg(u + (int64_t)i * n + p);
+                __syncwarp();
+                if (lane == 0) {
+                    double a = hp * wp * wp;
+                    for (int i = 0; i < r; ++i) a -= s_up[i] * s_up[i];
+                    if (!(a > thresh)) stop = 1;
+                    s_wp = wp;
+                    s_inv = 1.0 / sqrt(a);
+                }
+            }
+            if (lane == 0) s_p = stop ? -1 : p;
+            if (lead && !done) {  // (only this thread ever sets `done`)
+                st->K = stop ? r : r + 1;
+                if (stop) st->done = 1;
+                if (r == 0) st->thresh = thresh;
             }
         }
-        if (lane == 0) s_p = stop ? -1 : p;
-        if (lead && !done) {  // (only this thread ever sets `done`)
-            st->K = stop ? r : r + 1;
-            if (stop) st->done = 1;
-            if (r == 0) st->thresh = thresh;
+        __syncthreads();
+        const int64_t p = s_p;
+        if (p < 0) return;
+        const double wp = s_wp;
+        const double inv = s_inv;
+        Part own = part_none();
+        double* ur = u + (int64_t)r * n;
+        for (int64_t j = jf; j < n; j += (int64_t)gridDim.x * kThreads) {
+            double val = 0.0;
+            double dj = -INFINITY;
+            if (j >= j0) {
+                const bool first = j == jf;
+                double c = h[j + p] * (w ? (first ? wf : w[j]) * wp : 1.0);
+                const double dold = first ? df : __ldcg(d + j);
+                const double* uj = u + j;
+                int i = 0;
+                if (first && r >= kBatch) {
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b) c -= uf[b] * s_up[b];
+                    i = kBatch;
+                }
+                for (; i + kBatch <= r; i += kBatch) {
+                    double x[kBatch];
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b) x[b] = __ldcg(uj + (int64_t)(i + b) * n);
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b) c -= x[b] * s_up[i + b];
+                }
+                for (; i < r; ++i) c -= __ldcg(uj + (int64_t)i * n) * s_up[i];
+                val = c * inv;
+                dj = dold - val * val;
+                d[j] = dj;
+            }
+            ur[j] = val;
+            own = pmax(own, part_of(T, j, dj, j >= j0));
         }
+        publish(own, s_part, part + ((r + 1) & 1) * (int)gridDim.x);
+        if (lead) piv[r] = p;
     }
-    __syncthreads();
-    const int64_t p = s_p;
-    if (p < 0) return;
-    const double wp = s_wp;
-    const double inv = s_inv;
-    Part own = part_none();
-    double* ur = u + (int64_t)r * n;
-    for (int64_t j = jf; j < n; j += (int64_t)gridDim.x * kThreads) {
-        double val = 0.0;
-        double dj = -INFINITY;
-        if (j >= j0) {
-            const bool first = j == jf;
-            double c = h[j + p] * (w ? (first ? wf : w[j]) * wp : 1.0);
-            const double dold = first ? df : __ldcg(d + j);
-            const double* uj = u + j;
-            int i = 0;
-            if (first && r >= kBatch) {
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) c -= uf[b] * s_up[b];
-                i = kBatch;
-            }
-            for (; i + kBatch <= r; i += kBatch) {
-                double x[kBatch];
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) x[b] = __ldcg(uj + (int64_t)(i + b) * n);
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) c -= x[b] * s_up[i + b];
-            }
-            for (; i < r; ++i) c -= __ldcg(uj + (int64_t)i * n) * s_up[i];
-            val = c * inv;
-            dj = dold - val * val;
-            d[j] = dj;
-        }
-        ur[j] = val;
-        own = pmax(own, part_of(T, j, dj, j >= j0));
-    }
-    publish(own, s_part, part_out);
-    if (lead) piv[r] = p;
 }
 
 }  // namespace
 
 namespace {
 
-// The steps of a factorisation on stream s: state, residual diagonal and partials given.
+// The steps of a factorisation on stream s: state, residual diagonal and partials given (2 nblk of
+// them).  Launch by launch, the host reads the stop state after kFirstSteps, then every kNextSteps
+// steps; those launched past the end return at once.
 constexpr int64_t kFirstSteps = 20, kNextSteps = 12;
+
+cudaError_t read_state(State* host, const State* st, cudaStream_t s) {
+    cudaError_t e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
 
 cudaError_t pchol_steps(const double* h, const double* w, int64_t n, int64_t j0, double tol,
                         int64_t kmax, const TargetSpec& T, double* u, int64_t* pivots, double* d,
                         Part* part, int nblk, State* st, State* host, cudaStream_t s) {
     *host = State{};
     cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
+    if (e == cudaSuccess) {
+        pchol_step<true><<<nblk, kThreads, 0, s>>>(h, n, j0, w, tol, T, 0, (int)kmax, u, pivots, d,
+                                                   part, st, tc_stall_enabled() ? 1u : 0u);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = read_state(host, st, s);
+    if (e != cudaSuccess || !host->timeout) return e;
+    // not all of its blocks were resident: from the start again, a launch per step
+    e = cudaMemsetAsync(st, 0, sizeof(State), s);
     if (e == cudaSuccess) {
         pchol_init<<<nblk, kThreads, 0, s>>>(h, n, j0, w, T, d, part);
         e = cudaGetLastError();
@@ -272,13 +339,11 @@ cudaError_t pchol_steps(const double* h, const double* w, int64_t n, int64_t j0,
     cfg.numAttrs = 1;
     int64_t poll = kFirstSteps;
     for (int64_t r = 0; e == cudaSuccess && r < kmax; ++r) {
-        const Part* in = part + (r & 1) * nblk;
-        e = cudaLaunchKernelEx(&cfg, pchol_step, h, n, j0, w, tol, T, (int)r, u, pivots, d, in,
-                               part + ((r + 1) & 1) * nblk, st);
+        e = cudaLaunchKernelEx(&cfg, pchol_step<false>, h, n, j0, w, tol, T, (int)r, (int)kmax, u,
+                               pivots, d, part, st, 0u);
         if (e == cudaSuccess && (r + 1 == poll || r + 1 == kmax)) {
             poll += kNextSteps;
-            e = cudaMemcpyAsync(host, st, sizeof(State), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            e = read_state(host, st, s);
             if (host->done) break;
         }
     }
@@ -287,11 +352,11 @@ cudaError_t pchol_steps(const double* h, const double* w, int64_t n, int64_t j0,
 
 }  // namespace
 
-// Blocks of a step: six per SM at most (more partials to reduce, for no more loads in flight than
-// the memory system takes).
+// Blocks of the launch: all resident at once on an idle device (two of at most 128 registers a
+// thread per SM).
 int pchol_blocks(int64_t n) {
     return (int)std::max<int64_t>(
-        1, std::min<int64_t>((n + kThreads - 1) / kThreads, 6 * (int64_t)sm_count()));
+        1, std::min<int64_t>((n + kThreads - 1) / kThreads, 2 * (int64_t)sm_count()));
 }
 
 int pchol_run(const double* h, const double* w, int64_t n, int64_t j0, double tol, int64_t kmax,

@@ -194,3 +194,30 @@ def test_plans_keep_only_their_rank(tdh):
     held = free0 - torch.cuda.mem_get_info()[0]
     assert plan.K > 64
     assert held <= 8 * n * plan.K + (64 << 20) + (32 << 20), (held, plan.K)
+
+
+@pytest.mark.parametrize("kind,params", [("leg2cheb", ()), ("cheb2leg", ()),
+                                         ("jac2jac", (0.1, -0.3, 0.6, 0.2))])
+def test_factorisation_without_all_blocks_resident(tdh, kind, params):
+    """The factorisation's one launch gives up when its blocks cannot meet (here: a bounded wait that
+    the test hook makes run out) and goes launch by launch: same pivots, factors and ranks."""
+    import torch
+    n = 5000
+    sym = tdh.symbols("leg2cheb", n)[1]
+    u0, p0 = tdh.pchol(sym, n, 0, 1e-13)
+    want = [tdh.Plan(kind, n, prec=prec, params=params).K for prec in ("fp32", "fp64")]
+    few = tdh.Plan(kind, n, prec="fp64", params=params, kmax=3).K
+    tdh.inject_tc_stall(True)
+    try:
+        u1, p1 = tdh.pchol(sym, n, 0, 1e-13)
+        plans = [tdh.Plan(kind, n, prec=prec, params=params) for prec in ("fp32", "fp64")]
+        assert tdh.Plan(kind, n, prec="fp64", params=params, kmax=3).K == few == 3
+    finally:
+        tdh.inject_tc_stall(False)
+    assert torch.equal(p0, p1) and torch.equal(u0, u1)
+    assert [p.K for p in plans] == want
+    x = torch.tensor(workloads.coefficients(n, 2, decay=1.0, seed=2), device="cuda")
+    plans[1].set_schedule(0)  # (the FFT form multiplies with the factors)
+    ref = tdh.Plan(kind, n, prec="fp64", params=params)
+    ref.set_schedule(0)
+    assert torch.equal(plans[1].execute(x), ref.execute(x))
