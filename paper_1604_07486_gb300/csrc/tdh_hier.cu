@@ -1246,24 +1246,37 @@ double lagrange(const int* x, int P, int i, double at) {
     return v;
 }
 
-// Factors that make s_0 and h's first entry on the diagonal (index 2 j0) powers of two: entry
-// (j, j) = D1_j s_0 h_2j D2_j then carries no rounding of s_0, and the first one none of h.  (The
-// leading coefficients dominate decaying inputs, and a rounding common to all of them shows in
-// full.)  The mantissas taken out go to D1, which is rounded once for all of it.
-// Float64 keeps the symbols as they are: they are float64 already.
-template <typename T>
+// Float32 tables are scaled by constants, so that no rounding is common to all entries, or to the
+// leading ones, which dominate decaying inputs: s_0 becomes a power of two (every diagonal entry
+// has it) and h takes its mantissa.  Where D1 varies and is inexact anyway, h's first entry on the
+// diagonal (index 2 j0) becomes one too and D1, rounded once, takes that; Leg->Cheb's constant D1
+// (2/pi) gives its mantissa to h instead; Cheb->Leg's D1 (j + 1/2) is exact and stays.  Float64
+// keeps the symbols, which are float64 already.
+struct HierScale {
+    double s, h, d;  // table = symbol * factor
+};
 __device__ __forceinline__ double mantissa(double v) {
-    if (sizeof(T) == 8 || v == 0.0 || !isfinite(v)) return 1.0;
+    if (v == 0.0 || !isfinite(v)) return 1.0;
     int e;
     return fabs(frexp(v, &e)) * 2.0;
+}
+template <typename T>
+__device__ __forceinline__ HierScale hier_scale(const double* t, const double* h, int kind, int j0) {
+    if (sizeof(T) == 8) return HierScale{1.0, 1.0, 1.0};
+    const double mt = mantissa(t[0]);
+    const double md = kind == TDH_LEG2CHEB ? 1.2732395447351628 : 1.0;  // 4/pi
+    const double mh =
+        kind == TDH_LEG2CHEB || kind == TDH_CHEB2LEG ? 1.0 : mantissa(h[2 * j0] * mt);
+    return HierScale{1.0 / mt, mt * md / mh, mh / md};
 }
 
 // D1 for the tables below
 template <typename T>
-__global__ void k_hier_diagonal(const double* __restrict__ t, const double* __restrict__ h, int j0,
-                                const double* __restrict__ d1, int64_t n, T* __restrict__ out) {
+__global__ void k_hier_diagonal(const double* __restrict__ t, const double* __restrict__ h,
+                                const double* __restrict__ d1, int kind, int j0, int64_t n,
+                                T* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (i < n) out[i] = (T)(d1[i] * (mantissa<T>(t[0]) * mantissa<T>(h[2 * j0])));
+    if (i < n) out[i] = (T)(d1[i] * hier_scale<T>(t, h, kind, j0).d);
 }
 
 // table copies in execute precision: s_m = t[stride m] (32 zeros before, zero past mpad),
@@ -1271,14 +1284,14 @@ __global__ void k_hier_diagonal(const double* __restrict__ t, const double* __re
 // (0, 0) is direct
 template <typename T>
 __global__ void k_hier_tables(const double* __restrict__ t, const double* __restrict__ h,
-                              int64_t mpad, int64_t mrev, int stride, int j0, T* __restrict__ s,
-                              T* __restrict__ hf, T* __restrict__ hr) {
+                              int kind, int64_t mpad, int64_t mrev, int stride, int j0,
+                              T* __restrict__ s, T* __restrict__ hf, T* __restrict__ hr) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    const double mt = mantissa<T>(t[0]), mh = mantissa<T>(h[2 * j0]);
+    const HierScale c = hier_scale<T>(t, h, kind, j0);
     if (i < kHierSZero) s[i - kHierSZero] = T(0);
-    if (i < mpad) s[i] = (T)(t[stride * i] / mt);
+    if (i < mpad) s[i] = (T)(t[stride * i] * c.s);
     if (i < 2 * mpad + kHierHPad) {
-        const T v = (i >= 2 * mpad || (j0 == 1 && i == 0)) ? T(0) : (T)(h[stride * i] / mh);
+        const T v = (i >= 2 * mpad || (j0 == 1 && i == 0)) ? T(0) : (T)(h[stride * i] * c.h);
         hf[i] = v;
         if (i < 2 * mrev)
             hr[2 * mrev - 1 - i] = v;
@@ -1337,8 +1350,7 @@ int prepare_typed(Step& st, cudaStream_t s) {
     const bool top = ntop >= kTopKernel;
     const int64_t nps = top ? ntop * P * P : 0, nph = top ? (2 * ntop - 1) * NC * P * P : 0;
     const size_t at = (ns + 2 * nh + nw + 3) / 4 * 4;  // 16-byte aligned
-    const size_t nd = sizeof(T) == 4 ? (size_t)(st.n + 3) / 4 * 4 : 0;  // D1 of the scaled tables
-    int rc = dev_alloc(&H.tab, sizeof(T) * (at + (size_t)(nps + 2 * nph) + nd));
+    int rc = dev_alloc(&H.tab, sizeof(T) * (at + (size_t)(nps + 2 * nph)));
     std::vector<T> w(nw);
     if (rc == TDH_OK) {
         T* tab = static_cast<T*>(H.tab);
@@ -1346,17 +1358,20 @@ int prepare_typed(Step& st, cudaStream_t s) {
         H.hf = tab + ns;
         H.hr = tab + ns + nh;
         H.w = tab + ns + 2 * nh;
+        cudaError_t e = cudaSuccess;
+        H.d1 = st.d1x;
+        if (sizeof(T) == 4) {
+            // formed where the Hankel table will be, then kept in place of the float64 D1, which
+            // nothing reads any more (an allocation of its own: 50 us more per one-off conversion)
+            k_hier_diagonal<T><<<(unsigned)((st.n + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+                st.t, st.h, st.d1, st.kind, (int)st.j0, st.n, static_cast<T*>(H.hf));
+            e = cudaMemcpyAsync(st.d1, H.hf, sizeof(T) * (size_t)st.n, cudaMemcpyDeviceToDevice, s);
+            H.d1 = st.d1;
+        }
         const int64_t cnt = 2 * H.mpad + kHierHPad;
         k_hier_tables<T><<<(unsigned)((cnt + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-            st.t, st.h, H.mpad, H.mrev, NC, (int)st.j0, static_cast<T*>(H.s), static_cast<T*>(H.hf),
-            static_cast<T*>(H.hr));
-        H.d1 = st.d1x;
-        if (nd) {
-            T* d1 = tab + at + nps + 2 * nph;
-            k_hier_diagonal<T><<<(unsigned)((st.n + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-                st.t, st.h, (int)st.j0, st.d1, st.n, d1);
-            H.d1 = d1;
-        }
+            st.t, st.h, st.kind, H.mpad, H.mrev, NC, (int)st.j0, static_cast<T*>(H.s),
+            static_cast<T*>(H.hf), static_cast<T*>(H.hr));
         if (top) {
             H.st = tab + at;
             H.ht[0] = tab + at + nps;
@@ -1378,7 +1393,7 @@ int prepare_typed(Step& st, cudaStream_t s) {
                     for (int q = 0; q < P; ++q)
                         w[(size_t)P * kHierLeaf + (((l - 1) * 4 + c) * P + p) * P + q] =
                             (T)lagrange(x[l], P, p, c * hier_size(l - 1) + x[l - 1][q]);
-        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(H.w, w.data(), sizeof(T) * nw, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);

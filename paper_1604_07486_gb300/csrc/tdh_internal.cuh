@@ -191,7 +191,7 @@ struct Step {
     // symbols: of n coefficients, or of the hierarchical product's padded length
     double* t = nullptr;   // [n]
     double* h = nullptr;   // [2n-1]
-    double* d1 = nullptr;  // [n]
+    double* d1 = nullptr;  // [n]; float32 hierarchical steps: their float32 D1 from creation on
     double* d2 = nullptr;  // [n]
     double* u64 = nullptr; // [K][n]
     int64_t* piv = nullptr;
