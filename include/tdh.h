@@ -53,7 +53,8 @@ extern "C" {
 #define TDH_FP64  0 /* float64 in/out, float64 FFT                                             */
 #define TDH_FP32  1 /* float32 in/out, float32 FFT (plan factors rounded once from float64)    */
 /* float32 in/out; steps the hierarchical product serves run it in float32, as TDH_FP32 plans do
- * (faster than the FFTs below at every length); in the FFT form, within one thread-block cluster (FFTs of up to 2^17 points) the radix-16
+ * (faster than the FFTs below at every length); in the FFT form, within one thread-block cluster
+ * (FFTs of up to 2^17 points) the radix-16
  * (radix-8 for short FFTs) middle passes of every FFT run on the tensor cores as DFT matrix
  * products in split bfloat16: each operand x = hi + lo (bfloat16 parts) and the three products
  * hi*hi + lo*hi + hi*lo accumulate in float32 (tcgen05, tensor memory); every other pass and
@@ -103,7 +104,9 @@ typedef struct {
  *   a3  the spectrum of the Toeplitz symbol for each FFT length in use.
  * For TDH_CHEB2LEG the factorisation covers indices 1..n_max-1 and row 0 is applied directly
  * (Sec. 5.1).  tol > 0 is relative to the largest diagonal entry of H; Sec. 2.1 sets it
- * near the unit roundoff of the arithmetic used.
+ * near the unit roundoff of the arithmetic used.  tol and kmax bound the rank of the FFT form
+ * only: steps that run the hierarchical product (the default where it serves) are not truncated,
+ * whatever they say; tdh_plan_query reports the rank all the same.
  * With TDH_FLAG_TARGET, tol is instead the accuracy asked of each T o H step's truncation:
  * the factorisation pivots on the congruent W H W, w_j = sqrt(|D1_j D2_j|) (1 where zero;
  * the same A = D1 W^-1 (T o W H W) W^-1 D2, so the greedy pivot chases the residual that the
@@ -170,7 +173,8 @@ int tdh_plan_execute(tdh_plan_t plan, const void* in, void* out, int64_t batch, 
  * grouped by FFT length; each length class is converted by one persistent launch that takes
  * vectors from a work counter, and the classes run concurrently on plan-owned streams forked
  * from `stream`.  Both are capturable in a CUDA graph.  Calls from several host threads are
- * serialised while they enqueue (the fork and join events are the plan's).  Asynchronous; scratch is stream-ordered (see Scratch above).
+ * serialised while they enqueue (the fork and join events are the plan's).  Asynchronous;
+ * scratch is stream-ordered (see Scratch above).
  */
 int tdh_plan_execute_ragged(tdh_plan_t plan, const void* in, void* out, const int64_t* offsets,
                             int64_t batch, void* stream);
@@ -346,8 +350,8 @@ int tdh_test_fail_alloc(int64_t k);
 /*
  * tdh_test_tc_stall -- failure injection for tests (the paper has no counterpart): while on
  * (on != 0), executes enqueued from then on with TDH_BF16X3 plans run the FFT form (where it has
- * tensor-core passes) and issue none of their tensor-core products, so the first bounded wait of every CTA runs out after about one
- * second; the kernels then skip their remaining waits, finish, free their tensor memory and
+ * tensor-core passes) and issue none of their tensor-core products, so the first bounded wait of
+ * every CTA runs out after about one second; the kernels then skip their remaining waits, finish, free their tensor memory and
  * record TDH_STATUS_TIMEOUT (tdh_plan_status).  Their outputs are not valid.  The setting is
  * process-wide and read when an execute is enqueued (a captured CUDA graph keeps the value it
  * was captured with).  Factorisations of plans created meanwhile, and tdh_pchol's, find the waits

@@ -1,6 +1,7 @@
 """GB300 Toeplitz-dot-Hankel polynomial basis conversion (Townsend, Webb & Olver,
-arXiv:1604.07486): beta = A alpha with A = D1 (T o H) D2, H compressed by pivoted Cholesky,
-each Toeplitz product by FFT -- all in the CUDA library libtdh.so (include/tdh.h).
+arXiv:1604.07486): beta = A alpha with A = D1 (T o H) D2, T o H multiplied by interpolation in a
+tree of boxes or, on an FFT schedule, with H compressed by pivoted Cholesky and each Toeplitz
+product by FFT -- all in the CUDA library libtdh.so (include/tdh.h).
 
 This module only marshals arguments to that C ABI.  PyTorch supplies device memory and
 streams; every step of the conversion runs in the library's kernels.  There is no CPU
@@ -116,10 +117,12 @@ def _kind(kind):
 
 
 class Plan:
-    """A conversion plan (tdh_plan_create): symbols, pivoted Cholesky and FFT tables for
-    vectors of n coefficients, built on the current CUDA device in float64.  tol is relative
-    to max diag(H); with target=True it is the accuracy asked of the truncation instead
-    (fewest rank terms whose residual bound gives max|beta_K - beta| <= tol ||alpha||_1).
+    """A conversion plan (tdh_plan_create): symbols, pivoted Cholesky and product tables for
+    vectors of n coefficients, built on the current CUDA device in float64.  tol and kmax bound
+    the rank of the FFT form (set_schedule, autotune; the hierarchical product that runs otherwise
+    is not truncated).  tol is relative to max diag(H); with target=True it is the accuracy asked
+    of the truncation instead (fewest rank terms whose residual bound gives
+    max|beta_K - beta| <= tol ||alpha||_1).
     Without tol the plan is accuracy-targeted at half the precision's tolerance: 2.5e-6
     (float32), 5e-6 (split bfloat16, "bf16x3") or 5e-13 (float64)."""
 
@@ -339,5 +342,6 @@ def measure_dsmem_rate(stream=None):
 
 def inject_tc_stall(on):
     """While on, split-bfloat16 executes issue no tensor-core products, so their bounded waits
-    run out and TIMEOUT is recorded (tdh_test_tc_stall; outputs invalid)."""
+    run out and TIMEOUT is recorded (tdh_test_tc_stall; outputs invalid); factorisations of plans
+    created meanwhile run launch by launch, with the same results."""
     _check(lib().tdh_test_tc_stall(1 if on else 0))

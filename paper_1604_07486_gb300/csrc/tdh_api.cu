@@ -198,7 +198,7 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
         return sparse_prepare(st, prec, s);
     TDH_TRY(exec_choose(st, prec));
     // Whatever the precision and the length: split-bfloat16 plans' tensor-core FFTs take 28 us at
-    // n = 512 x 16 and 3267 us at 65536 x 256, the float32 hierarchical product 9.4 and 161 us with
+    // n = 512 x 16 and 3267 us at 65536 x 256, the float32 hierarchical product 9.4 and 160 us with
     // smaller errors.  Their FFT tables are built with the plan all the same (tdh_test_tc_stall).
     const bool hier = hier_serves(st, prec);
     const int64_t ns = hier ? hier_length(st) : n;

@@ -18,7 +18,8 @@
 // Parity kinds (T_jk = 0 for odd k - j) run as two channels of packed indices, k = 2a + e,
 // with s_m = t_{2m} and h_l = h_{2l}, the odd channel's Hankel table being the even one's
 // shifted by one (h_{2(a+b)+2e}).  The transpose is the same product on reversed indices
-// (k' = N - 1 - k, N the padded length), with the reversed Hankel table.
+// (k' = N - 1 - k, N whole boxes of the largest size that exchanges anything), with the reversed
+// Hankel table.
 #pragma once
 
 #include "tdh_internal.cuh"
