@@ -189,7 +189,6 @@ __global__ void __launch_bounds__(kThreads, 2) pchol_step(
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     const double tmax = T.a1 ? *T.tmax : 0.0;
     const int64_t jf = (int64_t)blockIdx.x * kThreads + threadIdx.x;  // this thread's first index
-    const double wf = w && jf < n ? w[jf] : 1.0;
     if constexpr (ALL) {
         init_slice(h, n, j0, w, T, d, part, s_part);
     } else {
@@ -200,13 +199,6 @@ __global__ void __launch_bounds__(kThreads, 2) pchol_step(
         if (ALL && !grid_barrier(st, (unsigned)r + 1u, stall)) {
             if (threadIdx.x == 0) st->timeout = 1;
             return;
-        }
-        // what does not depend on the pivot is on its way before the decision
-        double df = 0.0, uf[kBatch];
-        if (jf < n) {
-            df = __ldcg(d + jf);
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) uf[b] = b < r ? __ldcg(u + jf + (int64_t)b * n) : 0.0;
         }
         // every block reduces the same partials: identical pivot and decision everywhere
         const Part* in = part + (r & 1) * (int)gridDim.x;
@@ -266,16 +258,10 @@ __global__ void __launch_bounds__(kThreads, 2) pchol_step(
             double val = 0.0;
             double dj = -INFINITY;
             if (j >= j0) {
-                const bool first = j == jf;
-                double c = h[j + p] * (w ? (first ? wf : w[j]) * wp : 1.0);
-                const double dold = first ? df : __ldcg(d + j);
+                double c = h[j + p] * (w ? w[j] * wp : 1.0);
+                const double dold = __ldcg(d + j);
                 const double* uj = u + j;
                 int i = 0;
-                if (first && r >= kBatch) {
-#pragma unroll
-                    for (int b = 0; b < kBatch; ++b) c -= uf[b] * s_up[b];
-                    i = kBatch;
-                }
                 for (; i + kBatch <= r; i += kBatch) {
                     double x[kBatch];
 #pragma unroll
