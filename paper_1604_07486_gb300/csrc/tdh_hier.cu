@@ -1680,9 +1680,10 @@ int run_typed(const Step& st, const void* in, void* out, const int64_t* offs, in
     constexpr int FMAX = sizeof(T) == 4 ? 16 : 8;
     P.seg_leaves = real_leaves > 4 ? 16 : 4;
     P.nseg = (P.leaves + P.seg_leaves - 1) / P.seg_leaves;
-    // Two vectors per far CTA while such CTAs do not fill the chip: a CTA's time grows with its
-    // vectors, its tables' share only matters once the SMs are full (Leg->Cheb 16000 x 8 float64:
-    // 343 us with 8, 188 us with 2, the near field's vectors chosen alike).
+    // Two vectors per far CTA while such CTAs do not fill the chip, as a CTA's time grows with its
+    // vectors (Leg->Cheb 16000 x 8 float64: 343 us with 8, 188 us with 2, the near field's vectors
+    // chosen alike), else FMAX: nothing between, so just past the switch grids are small (65536 x 5
+    // float32: 64 CTAs) and slots empty.
     P.nvt = batch > 2 && (batch + 1) / 2 * P.nseg > sm_count() ? FMAX : 2;
     P.unvt = 32 / NP;
     // Near field: vectors of a warp (twice as many on half as many warps do the same work per SM
