@@ -213,7 +213,7 @@ int build_step(Step& st, double tol, int target, int64_t kmax, int prec, cudaStr
                 ? 1 : 0;
     st.K = 0;
     if (st.j0 < n) {
-        int64_t kcap = std::min<int64_t>(kmax, n - st.j0);
+        const int64_t kcap = std::min<int64_t>({kmax, n - st.j0, kPcholSteps});
         double* ubig = nullptr;
         TDH_TRY(dev_alloc_t(&st.piv, (size_t)kcap));
         int64_t K = 0;

@@ -92,6 +92,7 @@ struct PcholTarget {
     const double* tmax;  // max |t|
     double tol;
 };
+constexpr int kPcholSteps = 1024;  // steps a run takes at most, whatever kmax
 int pchol_run(const double* h, const double* w, int64_t n, int64_t j0, double tol, int64_t kmax,
               const PcholTarget* target, double* u, int64_t* pivots, int64_t* K, cudaStream_t s);
 // Weights w_j = sqrt(|D1_j D2_j|) of the accuracy-targeted factorisation (1 where zero) with its

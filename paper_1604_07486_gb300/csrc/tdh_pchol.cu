@@ -28,7 +28,7 @@ namespace tdh {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kKmaxShared = 1024;  // u_i[p] for i < r staged in shared memory
+constexpr int kKmaxShared = kPcholSteps;  // u_i[p] for i < r staged in shared memory
 
 struct State {
     double thresh;  // tol * max(diag H)

@@ -221,3 +221,11 @@ def test_factorisation_without_all_blocks_resident(tdh, kind, params):
     ref = tdh.Plan(kind, n, prec="fp64", params=params)
     ref.set_schedule(0)
     assert torch.equal(plans[1].execute(x), ref.execute(x))
+
+
+def test_large_kmax_asks_for_no_more_rows_than_steps(tdh):
+    """The factorisation takes at most 1024 steps, so a larger kmax asks for 1024 rows (here it would
+    be 320 GB)."""
+    n = 200000
+    plan = tdh.Plan("jac2jac", n, prec="fp64", params=(10.2, 3.0, 10.9, 3.0), kmax=10 ** 9)
+    assert 64 < plan.K <= 1024
